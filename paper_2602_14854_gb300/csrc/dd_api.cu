@@ -281,7 +281,7 @@ dd_status noalloc_flux_impl(dd_dlra_t h, int scratch_doubles, double* out) {
     return fail(DD_ERR_ARG, "nsub * r_cap = " + std::to_string((long)h->nsub * h->RC) +
                                 " exceeds the allocation-free scratch of " +
                                 std::to_string(scratch_doubles) + " doubles");
-  dd::scalar_flux(h->P, h->d_X[0], h->d_V[0], h->d_S[0], h->d_r[0], h->d_noalloc, out, h->nx,
+  dd::scalar_flux(h->P, h->d_X[0], h->d_V[0], h->d_S[0], h->d_r[0], h->d_noalloc, out,
                   h->stream);
   DD_CUDA(cudaGetLastError());
   return DD_OK;
@@ -646,7 +646,7 @@ static dd_status create_impl(int ninst, const dd_grid* grids, const dd_tiling* t
   ok &= dalloc(&h->d_sm, (long)nsub * dd::NSMALL * RC * RC) == cudaSuccess;
   ok &= dalloc(&h->d_sig, (long)nsub * DD_MAXC) == cudaSuccess;
   ok &= dalloc(&h->d_rho, (long)h->ncells_out) == cudaSuccess;
-  ok &= dalloc(&h->d_fluxw, (long)nsub * RC) == cudaSuccess;
+  ok &= dalloc(&h->d_fluxw, std::max<long>(dd::FLUX_SCRATCH, (long)nsub * RC)) == cudaSuccess;
   ok &= dalloc(&h->d_m, nsub) == cudaSuccess;
   ok &= dalloc(&h->d_rt, nsub) == cudaSuccess;
   ok &= dalloc(&h->d_rx, 2 * nsub) == cudaSuccess;
@@ -844,7 +844,7 @@ dd_status dd_dlra_scalar_flux(dd_dlra_t h, double* out, int out_on_device) {
   g_err.clear();
   if (!h || !out) return fail(DD_ERR_ARG, "bad argument");
   double* dst = out_on_device ? out : h->d_rho;
-  dd::scalar_flux(h->P, h->d_X[0], h->d_V[0], h->d_S[0], h->d_r[0], h->d_fluxw, dst, h->nx, h->stream);
+  dd::scalar_flux(h->P, h->d_X[0], h->d_V[0], h->d_S[0], h->d_r[0], h->d_fluxw, dst, h->stream);
   DD_CUDA(cudaGetLastError());
   if (!out_on_device) {
     DD_CUDA(cudaMemcpyAsync(out, h->d_rho, sizeof(double) * (size_t)h->ncells_out,
@@ -857,7 +857,7 @@ dd_status dd_dlra_scalar_flux(dd_dlra_t h, double* out, int out_on_device) {
 dd_status dd_dlra_scalar_flux_instance(dd_dlra_t h, int inst, double* out, int out_on_device) {
   g_err.clear();
   if (!h || !out || inst < 0 || inst >= h->ninst) return fail(DD_ERR_ARG, "bad argument");
-  dd::scalar_flux(h->P, h->d_X[0], h->d_V[0], h->d_S[0], h->d_r[0], h->d_fluxw, h->d_rho, h->nx,
+  dd::scalar_flux(h->P, h->d_X[0], h->d_V[0], h->d_S[0], h->d_r[0], h->d_fluxw, h->d_rho,
                   h->stream);
   DD_CUDA(cudaGetLastError());
   const size_t cnt = (size_t)h->inst_nx[inst] * (size_t)h->inst_ny[inst];

@@ -204,8 +204,11 @@ bool oz_gram(const Problem& P, unsigned* status, cudaStream_t st, int spatial, c
 void advection_phase(const Problem& P, const PhaseBufs& B, int axis, cudaStream_t st);
 void collision_phase(const Problem& P, const PhaseBufs& B, cudaStream_t st);
 void mass_fix_phase(const Problem& P, const PhaseBufs& B, cudaStream_t st);
+// work: at least max(FLUX_SCRATCH, nsub r_cap) doubles (FLUX_SCRATCH suffices while
+// nsub r_cap does not exceed it)
+constexpr int FLUX_SCRATCH = 16384;
 void scalar_flux(const Problem& P, const double* X, const double* V, const double* S, const int* r,
-                 double* work, double* rho, int nx, cudaStream_t st);
+                 double* work, double* rho, cudaStream_t st);
 cudaError_t phase_init();   // kernel attributes for every capacity up to DD_MAXC
 size_t part_elems(const Problem& P);
 // Launch choices timed on the solver's own workspace (called once, when a solver is

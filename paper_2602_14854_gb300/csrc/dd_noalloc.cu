@@ -15,11 +15,10 @@
 #include "dd_internal.cuh"
 #include "dd_launch.h"
 
-// Scratch of the allocation-free readout: one vector of r_cap doubles per
-// subdomain.  Every GPU that loads the library holds this array until the
-// process exits.
-#define DD_FLUX_SCRATCH_DOUBLES 16384
-static __device__ __align__(256) double g_flux_scratch[DD_FLUX_SCRATCH_DOUBLES];
+// Scratch of the allocation-free readout: at least one vector of r_cap doubles per
+// subdomain, up to 16 partial ones while they fit.  Every GPU that loads the library
+// holds this array until the process exits.
+static __device__ __align__(256) double g_flux_scratch[dd::FLUX_SCRATCH];
 
 namespace dd {
 
@@ -42,5 +41,5 @@ cudaError_t noalloc_scratch_address(double** addr) {
 
 extern "C" dd_status dd_dlra_scalar_flux_noalloc(dd_dlra_t h, double* out) {
   if (!h || !out) return dd::set_error(DD_ERR_ARG, "null argument");
-  return dd::noalloc_flux_impl(h, DD_FLUX_SCRATCH_DOUBLES, out);
+  return dd::noalloc_flux_impl(h, dd::FLUX_SCRATCH, out);
 }

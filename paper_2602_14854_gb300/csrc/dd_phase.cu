@@ -18,6 +18,7 @@
 //   L-step  per direction q:  dL_q/dt = -(c Omega_q/h) [(I - T) L_q - G_lo Vh_q]  (Omega_q > 0)
 //                              dL_q/dt = -(c Omega_q/h) [(T^T - I) L_q + G_hi Vh_q] (Omega_q < 0)
 //           (per-direction upwinding of f = U L^T with ghost f^b = K^b V^T, Eq. (advx_evolL)).
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <vector>
@@ -1643,38 +1644,82 @@ __global__ void k_coll_final(Problem P, PhaseBufs B) {
 // ---------------------------------------------------------------------------
 // scalar flux  rho_c = X_c (S a) / sqrt(hx hy),  a = Vt^T sqrt(w)
 // ---------------------------------------------------------------------------
-__global__ void k_flux_prep(Problem P, const double* V, const double* S, const int* r, double* work) {
-  const int k = blockIdx.x, RC = P.g.RC, n = P.g.n;
-  const int rk = r[k];
-  __shared__ double red[40];
-  __shared__ double av[DD_MAXC];
-  for (int t = 0; t < rk; ++t) {
-    double s = 0.0;
-    for (int q = threadIdx.x; q < n; q += blockDim.x) s += V[((long)k * n + q) * RC + t] * P.sw[q];
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) av[t] = s;
+// Chunk c of subdomain k's direction rows: a_c[t] = sum_q V[q][t] sqrt(w_q) into
+// work[(k * gridDim.x + c) * RC + t].  The FP64 pipe bounds it (a warp instruction holds the
+// pipe whatever lanes are active), so the threads are laid out densely over (row, column):
+// thread t owns column t % r of the rows t / r, t / r + T / r, ...  One CTA per subdomain
+// walking its columns one by one spent 60 us on the 64 x 2048 x 20 directions of a 512 x 512
+// problem; split over the SMs like this it takes 5.
+__global__ void __launch_bounds__(DD_THREADS) k_flux_prep(Problem P, const double* V, const int* r,
+                                                          double* work) {
+  __shared__ double sh[DD_THREADS];
+  const int k = blockIdx.y, RC = P.g.RC, n = P.g.n, rk = r[k], tid = threadIdx.x;
+  const int ch = (n + gridDim.x - 1) / gridDim.x;
+  const int q0 = blockIdx.x * ch, q1 = min(n, q0 + ch);
+  double* out = work + ((long)k * gridDim.x + blockIdx.x) * RC;
+  if (rk <= 0) return;
+  const int ng = DD_THREADS / rk, gr = tid / rk, t = tid - gr * rk;
+  double s = 0.0;
+  if (gr < ng) {
+    const double* Vk = V + (long)k * n * RC + t;
+#pragma unroll 8
+    for (int q = q0 + gr; q < q1; q += ng) s += Vk[(long)q * RC] * P.sw[q];
   }
+  sh[tid] = s;
   __syncthreads();
-  for (int i = threadIdx.x; i < RC; i += blockDim.x) {
-    double s = 0.0;
-    if (i < rk)
-      for (int j = 0; j < rk; ++j) s += S[(long)k * RC * RC + i * RC + j] * av[j];
-    work[(long)k * RC + i] = s;
+  if (tid < rk) {
+    double x = 0.0;
+    for (int g = 0; g < ng; ++g) x += sh[g * rk + tid];
+    out[tid] = x;
   }
 }
 
-__global__ void k_flux(Problem P, const double* X, const int* r, const double* work, double* rho,
-                       int nx) {
-  const int k = blockIdx.y, RC = P.g.RC;
+// rho of 256 cells of subdomain k, a thread per cell: every CTA first forms
+// sa = S a / sqrt(hx hy) from the nch chunks of a (r^2 products, hidden behind the other
+// CTAs' loads); the scale is in sa, so no cell divides (an FP64 division costs as much of the
+// FP64 pipe as the whole dot product).  Rows on 16-byte boundaries (RC even) are read as
+// pairs.  512 x 512 cells at r = 20: 102 us before (fixed 16 CTAs per subdomain, a division
+// per cell, the columns of a one after another), 26 us now with k_flux_prep.
+__global__ void __launch_bounds__(DD_THREADS) k_flux(Problem P, const double* X, const double* S,
+                                                     const int* r, const double* work, int nch,
+                                                     double* rho) {
+  __shared__ double av[DD_MAXC], sa[DD_MAXC];
+  const int k = blockIdx.y, RC = P.g.RC, tid = threadIdx.x;
   const int N = P.g.N[k], rk = r[k], nxk = P.g.nxk[k];
-  const double* sa = work + (long)k * RC;
-  for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < N; cell += gridDim.x * blockDim.x) {
-    const double* Xr = X + ((long)P.g.rowoff[k] + cell) * RC;
-    double s = 0.0;
-    for (int t = 0; t < rk; ++t) s += Xr[t] * sa[t];
-    int il = cell % nxk, jl = cell / nxk;
-    rho[(long)P.g.fbase[k] + (long)(P.g.cy0[k] + jl) * P.g.fnx[k] + P.g.cx0[k] + il] = s / P.g.shk[k];
+  const int cell = blockIdx.x * DD_THREADS + tid;
+  if (blockIdx.x * DD_THREADS >= N) return;
+  if (tid < rk) {
+    double x = 0.0;
+    for (int c = 0; c < nch; ++c) x += work[((long)k * nch + c) * RC + tid];
+    av[tid] = x;
   }
+  __syncthreads();
+  if (tid < rk) {
+    const double* Sk = S + ((long)k * RC + tid) * RC;
+    double x = 0.0;
+    for (int j = 0; j < rk; ++j) x += Sk[j] * av[j];
+    sa[tid] = x / P.g.shk[k];
+  }
+  __syncthreads();
+  if (cell >= N) return;
+  const double* Xr = X + ((long)P.g.rowoff[k] + cell) * RC;
+  double s = 0.0;
+  if (RC & 1) {
+#pragma unroll 4
+    for (int t = 0; t < rk; ++t) s += Xr[t] * sa[t];
+  } else {
+    const double2* X2 = reinterpret_cast<const double2*>(Xr);
+    const int h = rk >> 1;
+#pragma unroll 5
+    for (int t = 0; t < h; ++t) {
+      const double2 x = X2[t];
+      s = fma(x.x, sa[2 * t], s);
+      s = fma(x.y, sa[2 * t + 1], s);
+    }
+    if (rk & 1) s += Xr[rk - 1] * sa[rk - 1];
+  }
+  const int il = cell % nxk, jl = cell / nxk;
+  rho[(long)P.g.fbase[k] + (long)(P.g.cy0[k] + jl) * P.g.fnx[k] + P.g.cx0[k] + il] = s;
 }
 
 // TC working set plus an FP64 copy of S2 and one FP64 vh per warp
@@ -2438,13 +2483,24 @@ void mass_fix_phase(const Problem& P, const PhaseBufs& B, cudaStream_t st) {
   tall(P, B, st, 0, B.V1, RC, B.rt, 0, nullptr, SM_VB, B.ro, 0, B.Vo, RC);
 }
 
+// chunks of k_flux_prep per subdomain: two CTAs per SM over all subdomains, at least 32 rows
+// each, within the smaller of the two scratch arrays (the allocation-free readout's), so that
+// both readouts sum in the same order
+static int flux_chunks(const Problem& P, long scratch) {
+  const long per = (long)P.g.nsub * P.g.RC;
+  const int want = std::min(std::min(16, (2 * P.nsm + P.g.nsub - 1) / P.g.nsub), (P.g.n + 31) / 32);
+  return (int)std::max(1L, std::min((long)want, scratch / per));
+}
+
 void scalar_flux(const Problem& P, const double* X, const double* V, const double* S, const int* r,
-                 double* work, double* rho, int nx, cudaStream_t st) {
+                 double* work, double* rho, cudaStream_t st) {
+  const int nch = flux_chunks(P, FLUX_SCRATCH);
   pbeg(st, KS_FLUX);
-  k_flux_prep<<<P.g.nsub, DD_THREADS, 0, st>>>(P, V, S, r, work);
+  k_flux_prep<<<dim3(nch, P.g.nsub), DD_THREADS, 0, st>>>(P, V, r, work);
   pend(st);
   pbeg(st, KS_FLUX);
-  k_flux<<<dim3(16, P.g.nsub), DD_THREADS, 0, st>>>(P, X, r, work, rho, nx);
+  k_flux<<<dim3((P.maxN + DD_THREADS - 1) / DD_THREADS, P.g.nsub), DD_THREADS, 0, st>>>(P, X, S, r,
+      work, nch, rho);
   pend(st);
 }
 
