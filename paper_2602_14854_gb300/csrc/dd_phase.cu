@@ -62,41 +62,53 @@ __global__ void k_aug_cols(Geo g, const int* r, int axis, int* m, const int* inf
   m[k] = r[k] + (lo >= 0 ? r[lo] : 0) + (hi >= 0 ? r[hi] : 0) + il + ih;
 }
 
-__global__ void k_build_L0(Geo g, const double* V, const double* S, const int* r, int axis,
-                           double* L0, const int* infl_on, const double* infl_hw,
-                           const double* infl_sc) {
+// A CTA forms 64 rows of V_k S_k^T once and writes them into every L0 that holds them: its own
+// (columns 0 ..), its upper neighbour's (the lower neighbour's block there) and its lower
+// neighbour's.  The product is FP64-bound; forming each block where it is read cost three times
+// as much (382 us at 64 x 2048 x 20, now 97).
+#define L0_ROWS 64
+size_t build_L0_smem(int RC) { return sizeof(double) * ((size_t)RC * RC + L0_ROWS * (RC | 1)); }
+__global__ void __launch_bounds__(DD_THREADS) k_build_L0(Geo g, const double* V, const double* S,
+                                                         const int* r, int axis, double* L0,
+                                                         const int* infl_on, const double* infl_hw,
+                                                         const double* infl_sc) {
   extern __shared__ double sh[];
-  const int k = blockIdx.y, RC = g.RC;
+  const int k = blockIdx.y, RC = g.RC, MC = g.MC, n = g.n, tid = threadIdx.x;
+  const int q0 = blockIdx.x * L0_ROWS, nq = min(L0_ROWS, n - q0), rk = r[k], pv = RC | 1;
   const int lo = g.nb[k * 4 + 2 * axis], hi = g.nb[k * 4 + 2 * axis + 1];
-  const int src[3] = {k, lo, hi};
-  int rr[3];
-  for (int b = 0; b < 3; ++b) rr[b] = src[b] >= 0 ? r[src[b]] : 0;
-  const int sl = 2 * axis, shi = 2 * axis + 1;
-  const int il = (lo < 0 && infl_on && infl_on[k * 4 + sl]) ? 1 : 0;
-  const int ih = (hi < 0 && infl_on && infl_on[k * 4 + shi]) ? 1 : 0;
-  // stage the three S blocks
-  for (int b = 0; b < 3; ++b)
-    for (int e = threadIdx.x; e < RC * RC; e += blockDim.x)
-      sh[b * RC * RC + e] = src[b] >= 0 ? S[(long)src[b] * RC * RC + e] : 0.0;
+  double* St = sh;                                  // S^T: entry (l, t) at l rk + t
+  double* Vs = sh + RC * RC;
+  for (int e = tid; e < rk * rk; e += DD_THREADS) {
+    const int t = e / rk, l = e - t * rk;
+    St[l * rk + t] = S[((long)k * RC + t) * RC + l];
+  }
+  for (int e = tid; e < nq * rk; e += DD_THREADS) {
+    const int q = e / rk, l = e - q * rk;
+    Vs[q * pv + l] = V[((long)k * n + q0 + q) * RC + l];
+  }
+  // the block's first column in the neighbours' L0
+  const int chi = hi >= 0 ? r[hi] : 0;
+  const int l2 = lo >= 0 ? g.nb[lo * 4 + 2 * axis] : -1;
+  const int clo = lo >= 0 ? r[lo] + (l2 >= 0 ? r[l2] : 0) : 0;
   __syncthreads();
-  const int mn = rr[0] + rr[1] + rr[2], m = mn + il + ih;
-  const int q0 = blockIdx.x * 32;
-  for (int e = threadIdx.x; e < 32 * m; e += blockDim.x) {
-    int q = q0 + e / m, col = e % m;
-    if (q >= g.n) continue;
-    if (col >= mn) {                               // inflow column: sqrt(w) m_in h |g|_x
-      const int side = (col == mn && il) ? sl : shi;
-      L0[((long)k * g.n + q) * g.MC + col] =
-          infl_hw[((long)k * 4 + side) * g.n + q] * infl_sc[k * 4 + side];
-      continue;
-    }
-    int b = 0, t = col;
-    while (t >= rr[b]) { t -= rr[b]; ++b; }
-    const double* Vq = V + ((long)src[b] * g.n + q) * RC;
-    const double* Sb = sh + b * RC * RC + t * RC;     // row t of S_b
+  for (int e = tid; e < nq * rk; e += DD_THREADS) {
+    const int q = e / rk, t = e - q * rk;
     double s = 0.0;
-    for (int l = 0; l < rr[b]; ++l) s += Vq[l] * Sb[l];
-    L0[((long)k * g.n + q) * g.MC + col] = s;
+    for (int l = 0; l < rk; ++l) s += Vs[q * pv + l] * St[l * rk + t];
+    L0[((long)k * n + q0 + q) * MC + t] = s;
+    if (hi >= 0) L0[((long)hi * n + q0 + q) * MC + chi + t] = s;
+    if (lo >= 0) L0[((long)lo * n + q0 + q) * MC + clo + t] = s;
+  }
+  // inflow columns: sqrt(w) m_in h |g|_x
+  if (!infl_on) return;
+  int col = rk + (lo >= 0 ? r[lo] : 0) + (hi >= 0 ? r[hi] : 0);
+  for (int side = 0; side < 2; ++side) {
+    const int sd = 2 * axis + side;
+    if ((side ? hi : lo) >= 0 || !infl_on[k * 4 + sd]) continue;
+    for (int q = tid; q < nq; q += DD_THREADS)
+      L0[((long)k * n + q0 + q) * MC + col] =
+          infl_hw[((long)k * 4 + sd) * n + q0 + q] * infl_sc[k * 4 + sd];
+    ++col;
   }
 }
 
@@ -1823,7 +1835,7 @@ cudaError_t phase_init() {
                            (int)(coll_lstep_smem(RC)));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_build_L0, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(sizeof(double) * 3 * RC * RC));
+                           (int)build_L0_smem(RC));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_tall, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)tall_smem(RC, RC));
@@ -2143,8 +2155,8 @@ void advection_phase(const Problem& P, const PhaseBufs& B, int axis, cudaStream_
   k_aug_cols<<<(nsub + 127) / 128, 128, 0, st>>>(g, B.r, axis, B.m, P.infl_on);
   pend(st);
   pbeg(st, KS_BUILD_L0);
-  k_build_L0<<<dim3((g.n + 31) / 32, nsub), DD_THREADS, sizeof(double) * 3 * RC * RC, st>>>(
-      g, B.V, B.S, B.r, axis, B.L0, P.infl_on, P.infl_hw, P.infl_sc);
+  k_build_L0<<<dim3((g.n + L0_ROWS - 1) / L0_ROWS, nsub), DD_THREADS, build_L0_smem(RC), st>>>(g, B.V,
+      B.S, B.r, axis, B.L0, P.infl_on, P.infl_hw, P.infl_sc);
   pend(st);
   {
     OrthArgs a = orth_args(P, B, 0, ORTH_AUG);
