@@ -58,9 +58,10 @@ struct OrthArgs {
 
 cudaError_t orth_init();
 // the per-subdomain steps of the orthonormalisation (dd_orth.cu)
-void launch_geig(const OrthArgs& a, const double* part, const int* cexp, int nchunk, double* sm,
-                 int sM, int* keep, cudaStream_t st);
-void launch_chol_inv(const OrthArgs& a, const double* part, int nchunk, double* sm, int sRi,
+// (nchunk: chunk stride of the partial Grams; crows > 0: a subdomain has one per crows rows)
+void launch_geig(const OrthArgs& a, const double* part, const int* cexp, int nchunk, int crows,
+                 double* sm, int sM, int* keep, cudaStream_t st);
+void launch_chol_inv(const OrthArgs& a, const double* part, int nchunk, int crows, double* sm, int sRi,
                      const int* keep, cudaStream_t st);
 void launch_complete(const OrthArgs& a, const int* keep, cudaStream_t st);
 // Spatial completion of a QR basis by Gram-Schmidt in coefficient space (dd_orth.cu):

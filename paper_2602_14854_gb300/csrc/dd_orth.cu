@@ -42,35 +42,31 @@
 //          sqrt(w)), then the unit vectors.
 #include "dd_internal.cuh"
 #include "dd_launch.h"
+#include "dd_small.cuh"
 
 #include <climits>
 #include <math_constants.h>
 
 namespace dd {
 
-// Rank decision (one thread).  sig[] descending; returns p, sets *keep and *r_out.
+// Rank decision (one warp).  sig[] descending; returns p, sets *keep and *r_out (every lane).
 __device__ int decide(const OrthArgs& a, int k, const double* sig, int nref, int* keep,
                       int* r_out) {
+  const int lane = threadIdx.x & 31;
+  const double s1 = nref > 0 ? sig[0] : 0.0, thr = a.tau * s1;
   int p = 0;
-  double s1 = nref > 0 ? sig[0] : 0.0;
-  if (s1 > 0.0)
-    for (int t = 0; t < nref; ++t)
-      if (sig[t] > a.tau * s1) ++p;
+  for (int t0 = 0; t0 < nref; t0 += 32)
+    p += __popc(__ballot_sync(0xffffffffu, s1 > 0.0 && t0 + lane < nref && sig[t0 + lane] > thr));
   if (a.sig_out)
-    for (int t = 0; t < DD_MAXC; ++t) a.sig_out[(long)k * DD_MAXC + t] = t < nref ? sig[t] : 0.0;
-  if (a.p_out) a.p_out[k] = p;
+    for (int t = lane; t < DD_MAXC; t += 32) a.sig_out[(long)k * DD_MAXC + t] = t < nref ? sig[t] : 0.0;
+  if (a.p_out && lane == 0) a.p_out[k] = p;
   if (a.mode == ORTH_QR) {
     *r_out = a.rout[k];
     *keep = min(p, *r_out);
   } else {  // ORTH_AUG
     int r_tail = p;
     if (a.rank_mode == 1) {
-      r_tail = nref;
-      for (int r = 0; r <= nref; ++r) {
-        double ss = 0.0;
-        for (int t = r; t < nref; ++t) ss += sig[t] * sig[t];
-        if (sqrt(ss) <= a.tol) { r_tail = r; break; }
-      }
+      r_tail = tail_rank(nref, a.tol, [&](int t) { return sig[t]; });
     }
     int r_sig = min(r_tail, p);
     int cap = min(min(a.g.raug[k], a.g.n), a.g.N[k]);
@@ -88,349 +84,270 @@ __device__ int decide(const OrthArgs& a, int k, const double* sig, int nref, int
 // map whole warps onto rows, and comparisons use the integer order of the bit
 // patterns (positive doubles order as their bits).
 
-// Pivoted Cholesky of the m x m (m <= 64) positive semidefinite A (column-major,
-// leading dimension ld; overwritten by its Schur complements): A = X X^T up to a
-// remainder whose diagonal is <= thr_rel times the largest diagonal entry of A.  X is
-// m x k, written to the first k columns of X with the rows in the original order
-// (column t is row t of the triangular factor in pivot order).  The pivot is the
-// largest remaining positive finite diagonal entry (lowest index on ties); *piv gets
-// the pivoted indices as a bit mask.  Block-wide; returns k.
-__device__ int pchol_cols(double* A, double* X, int m, int ld, double thr_rel,
-                          unsigned long long* piv) {
-  __shared__ double pc[2];
-  __shared__ int pi[1];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  unsigned long long done = 0ull;
-  long long thr_bits = 0;                          // lane 0 of warp 0 only
-  int k = 0;
-  for (; k < m; ++k) {
-    if (warp == 0) {
-      long long best = 0;
-      int bi = m;
-      for (int i = lane; i < m; i += 32) {
-        const long long b = __double_as_longlong(A[i * ld + i]);
-        const bool ok = !((done >> i) & 1ull) && b > 0 && b < 0x7ff0000000000000ll;
-        if (ok && b > best) { best = b; bi = i; }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-      }
-      if (lane == 0) {
-        if (k == 0) thr_bits = __double_as_longlong(thr_rel * __longlong_as_double(best));
-        const bool go = bi < m && best > thr_bits;
-        if (go) {
-          const double dv = __longlong_as_double(best), id = rsqrt(dv);
-          pc[0] = dv * id;
-          pc[1] = id;
-        }
-        pi[0] = go ? bi : -1;
-      }
-    }
-    __syncthreads();
-    const int bi = pi[0];
-    if (bi < 0) break;
-    const double d = pc[0], id = pc[1];
-    // column k of X (warp 0) and the Schur update (every warp) both read the pivot
-    // column of A, which no thread writes in this step (bi is done)
-    if (warp == 0)
-      for (int i = lane; i < m; i += 32)
-        X[k * ld + i] = ((done >> i) & 1ull) ? 0.0 : (i == bi ? d : A[bi * ld + i] * id);
-    done |= 1ull << bi;
-    for (int j = warp; j < m; j += nw) {
-      if ((done >> j) & 1ull) continue;
-      const double f = (A[bi * ld + j] * id) * id;   // one FMA per entry of the update
-      for (int i = lane; i < m; i += 32)
-        if (!((done >> i) & 1ull)) A[j * ld + i] = fma(-A[bi * ld + i], f, A[j * ld + i]);
-    }
-    __syncthreads();
-  }
-  *piv = done;
-  return k;
+// partial Grams of subdomain k: nchunk of them, or one per crows rows
+__device__ __forceinline__ int orth_chunks(const OrthArgs& a, int k, int nchunk, int crows) {
+  const int rows = a.spatial ? a.g.N[k] : a.g.n;
+  return crows > 0 ? min(nchunk, (rows + crows - 1) / crows) : nchunk;
 }
 
-// Completes the orthonormal columns 0..cur-1 of the m x m column-major V (leading
-// dimension ld) to m columns with unit vectors, first those of the indices outside
-// mask (in index order), then the others, each accepted when its squared norm after
-// Gram-Schmidt exceeds 0.01 (at every stage some unit vector keeps at least 1/m).
-// The candidates outside mask are taken as a block: the span of the first cur columns
-// is removed from all of them at once (twice), then each is Gram-Schmidt'd against the
-// block columns accepted before it; the rest, when needed, one by one against
-// everything (twice).  coef: m doubles, W: 2 ld^2 doubles of shared scratch.
-__device__ void complete_unit(double* V, int m, int cur, int ld, unsigned long long mask,
-                              double* coef, double* W, unsigned* status) {
-  __shared__ double cred[40];
-  __shared__ int cidx[64];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  if (cur >= m) return;
-  // indices outside mask, ascending
-  const unsigned long long out = ~mask & (m >= 64 ? ~0ull : ((1ull << m) - 1ull));
-  const int q = __popcll(out);
-  for (int t = tid; t < m; t += blockDim.x)
-    if ((out >> t) & 1ull) cidx[__popcll(out & ((1ull << t) - 1ull))] = t;
-  __syncthreads();
-  const int c0 = cur;
-  double* C = W + (long)ld * ld;
-  for (int e = tid; e < m * q; e += blockDim.x) {          // W = E - V V^T E
-    const int r = e % m, t = e / m, i = cidx[t];
-    double s = r == i ? 1.0 : 0.0;
-    for (int l = 0; l < c0; ++l) s -= V[l * ld + i] * V[l * ld + r];
-    W[t * ld + r] = s;
-  }
-  __syncthreads();
-  for (int e = tid; e < c0 * q; e += blockDim.x) {         // C = V^T W
-    const int l = e % c0, t = e / c0;
-    double s = 0.0;
-    for (int r = 0; r < m; ++r) s += V[l * ld + r] * W[t * ld + r];
-    C[t * ld + l] = s;
-  }
-  __syncthreads();
-  for (int e = tid; e < m * q; e += blockDim.x) {          // W -= V C
-    const int r = e % m, t = e / m;
-    double s = W[t * ld + r];
-    for (int l = 0; l < c0; ++l) s -= C[t * ld + l] * V[l * ld + r];
-    W[t * ld + r] = s;
-  }
-  __syncthreads();
-  for (int t = 0; t < q && cur < m; ++t) {
-    const int na = cur - c0;
-    for (int l = warp; l < na; l += nw) {
-      double s = 0.0;
-      for (int r = lane; r < m; r += 32) s += V[(c0 + l) * ld + r] * W[t * ld + r];
-      s = warp_sum(s);
-      if (lane == 0) coef[l] = s;
-    }
-    __syncthreads();
-    double* x = V + (long)cur * ld;
-    double n2 = 0.0;
-    for (int r = tid; r < m; r += blockDim.x) {
-      double s = W[t * ld + r];
-      for (int l = 0; l < na; ++l) s -= coef[l] * V[(c0 + l) * ld + r];
-      x[r] = s;
-      n2 += s * s;
-    }
-    n2 = block_sum(n2, cred);
-    if (n2 > 0.01) {
-      for (int r = tid; r < m; r += blockDim.x) x[r] *= rsqrt(n2);
-      ++cur;
-    }
-    __syncthreads();
-  }
-  for (int cand = 0; cand < 2 * m && cur < m; ++cand) {    // not expected: one by one
-    const int i = cand < m ? cand : cand - m;
-    const bool inmask = (mask >> i) & 1ull;
-    if ((cand < m) == inmask) continue;
-    double* x = V + (long)cur * ld;
-    for (int r = tid; r < m; r += blockDim.x) {
-      double s = r == i ? 1.0 : 0.0;
-      for (int l = 0; l < cur; ++l) s -= V[l * ld + i] * V[l * ld + r];
-      x[r] = s;
-    }
-    __syncthreads();
-    for (int l = warp; l < cur; l += nw) {
-      double s = 0.0;
-      for (int r = lane; r < m; r += 32) s += V[l * ld + r] * x[r];
-      s = warp_sum(s);
-      if (lane == 0) coef[l] = s;
-    }
-    __syncthreads();
-    double n2 = 0.0;
-    for (int r = tid; r < m; r += blockDim.x) {
-      double s = x[r];
-      for (int l = 0; l < cur; ++l) s -= coef[l] * V[l * ld + r];
-      x[r] = s;
-      n2 += s * s;
-    }
-    n2 = block_sum(n2, cred);
-    if (n2 > 0.01) {
-      for (int r = tid; r < m; r += blockDim.x) x[r] *= rsqrt(n2);
-      ++cur;
-    }
-    __syncthreads();
-  }
-  if (cur < m && threadIdx.x == 0) atomicOr(status, (unsigned)ST_COMPLETION);
+// the vectors lam, sig, nrm and perm, padded to 16 bytes (the FP32 region follows)
+__host__ __device__ __forceinline__ size_t geig_vec_bytes(int RC) {
+  const size_t b = 3 * small_region(RC) + (sizeof(double) * 2 + sizeof(float2) + sizeof(int)) * RC;
+  return ((b + 15) & ~(size_t)15) - 3 * small_region(RC);
 }
-
 size_t geig_smem_bytes(int RC) {
-  return sizeof(double) * (3 * RC * RC + 2 * RC) + 8 * ((jacobi_mixed_scratch_bytes(RC) + 7) / 8) +
-         sizeof(int) * (RC + 16);
+  return 3 * small_region(RC) + geig_vec_bytes(RC) + small_f32_region(RC);
 }
 
-// Eigendecomposition of G1 (m x m): one-sided Jacobi (FP32 sweeps, double-float
-// finish; the columns of G1 V are orthogonal with norms lambda_j, G1 being positive
-// semidefinite), then one FP64 refinement step of the eigenvectors (Ogita and
-// Aishima, 2018): with R = I - V^T V, S = V^T G1 V, lambda_i = s_ii / (1 - r_ii),
-// V <- V (I + E), e_ij = (s_ij + lambda_j r_ij) / (lambda_j - lambda_i) for
-// separated pairs, r_ij / 2 within clusters and on the diagonal.  The double-float
-// solution is accurate to ~1e-14 |G1|; the step brings it to the FP64 level, which the
-// parity with an FP64 SVD needs for eigenvectors whose eigenvalues sit near the rank
-// threshold (tau^2 lambda_1).  Writes M = V_keep diag(sigma_keep)^-1 (row-major,
-// slot sM), keep (per subdomain) and, for the augmentation, r_t.
-__global__ void __launch_bounds__(DD_THREADS, 1) k_geig(OrthArgs a, const double* part,
-                                                     const int* cexp, int nchunk, double* sm,
-                                                     int sM, int* keep_out) {
+// Singular values and leading right singular vectors of A from its Gram G1 (m x m, the sum of
+// the chunk partials): G1 = X X^T by pivoted Cholesky (columns graded), one-sided Jacobi on X:
+// the columns of X J = W are orthogonal, sigma_j = |w_j| and w_j / |w_j| are the eigenvectors of
+// G1.  Jacobi on the graded factor takes a fraction of the sweeps that Jacobi on G1 would, and
+// loses nothing against the Gram: an error F in the orthogonality of J turns into a relative
+// error F sigma_i sigma_j in the coupling of w_i and w_j, where G1 itself carries
+// eps sigma_1^2, so the directions near the rank threshold need no refinement against G1 (one
+// FP64 refinement step of all m vectors was 11-18% of the kernel and changed no result).
+// (jacobi_core, dd_small.cuh.)  The factor
+// goes down to the rounding level of G1 (1e-16 of the largest diagonal entry, or 1/100 of the
+// squared rank threshold when that is smaller): what it leaves out, against eigenvalues of
+// tau^2 sigma_1^2 = 1e-10 sigma_1^2, turns the directions near the threshold (at 1e-13 by 1e-2,
+// which cost the density three digits).  Writes M = V_keep diag(sigma_keep)^-1 (row-major, slot
+// sM), keep (per subdomain) and, for the augmentation, r_t.
+// One CTA per subdomain: bound by the latency of the Jacobi rounds (dd_small.cuh).
+// 64 subdomains of 64 x 64 cells, r_t = 40 (60 columns in the augmentation): 310 us (QR) and
+// 797 us (augmentation) before, 66 and 118 now.
+__global__ void __launch_bounds__(512, 1) k_geig(OrthArgs a, const double* part, const int* cexp,
+                                              int nchunk, int crows, double* sm, int sM,
+                                              int* keep_out) {
   extern __shared__ double shg[];
-  const int k = blockIdx.x, RC = a.g.RC;
+  const int k = blockIdx.x, RC = a.g.RC, ld = small_ld(RC), tid = threadIdx.x;
+  const int lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int m = a.acols[k];
-  const double* G = part + (long)k * nchunk * RC * RC;      // nchunk partial Grams
+  const double* G = part + (long)k * nchunk * RC * RC;      // nck partial Grams
+  const int nck = orth_chunks(a, k, nchunk, crows);
   double* M = sm + ((long)k * NSMALL + sM) * RC * RC;
-  double* Bc = shg;                 // column-major working copy
-  double* Jc = Bc + RC * RC;        // accumulated rotations
-  double* Gs = Jc + RC * RC;        // G1 (scaled), kept for the refinement
-  double* lam = Gs + RC * RC;       // eigenvalues
-  double* sig = lam + RC;           // singular values of A, descending
-  double* X = sig + RC;             // scratch of the SVD
-  int* perm = reinterpret_cast<int*>(X + (jacobi_mixed_scratch_bytes(RC) + 7) / 8);
-  int* iv = perm + RC;
-  const int tid = threadIdx.x;
+  double* A = shg;                                  // G1, then X in double-float
+  double* X = A + (size_t)ld * RC;                  // pivot columns, then W
+  const int ldf = small_ldf(RC);
+  double* R3 = X + (size_t)ld * RC;                 // scratch of the Jacobi
+  double* lam = X + 2 * (size_t)ld * RC;            // sigma^2, by column
+  double* sig = lam + RC;                           // pivots, then singular values of A, descending
+  float2* nrm = reinterpret_cast<float2*>(sig + RC);
+  float* B32 = reinterpret_cast<float*>(reinterpret_cast<char*>(shg) + 3 * small_region(RC) + geig_vec_bytes(RC));
+  float* J32 = B32 + (size_t)ldf * (ldf - 4);
+  int* perm = reinterpret_cast<int*>(nrm + RC);
   // the chunk partials are Grams of 2^-e_c A: G1 of 2^-emax A is their sum with
   // weights 4^(e_c - emax)
   __shared__ double fac[64];
+  __shared__ int s_keep;
   int emax = INT_MIN;
-  for (int c = 0; c < nchunk; ++c) emax = max(emax, cexp[(long)k * nchunk + c]);
-  for (int c = tid; c < nchunk; c += blockDim.x) {
+  bool scaled = false;
+  for (int c = 0; c < nck; ++c) {
+    const int ec = cexp[(long)k * nchunk + c];
+    emax = max(emax, ec);
+    scaled |= ec != 0;
+  }
+  for (int c = tid; c < nck; c += blockDim.x) {
     const int ec = cexp[(long)k * nchunk + c];
     fac[c] = ec == INT_MIN ? 0.0 : ldexp(1.0, 2 * max(ec - emax, -600));
   }
   __syncthreads();
   bool fin = true;
-  for (int e = tid; e < RC * RC; e += blockDim.x) {
-    const int col = e / RC, row = e % RC;
+  for (int e = tid; e < m * (m + 1) / 2; e += blockDim.x) {
+    int i, j;
+    tri_index(e, &i, &j);                           // i <= j: entry (j, i) of the lower triangle
     double x = 0.0;
-    if (col < m && row < m && emax != INT_MIN)
-      for (int c = 0; c < nchunk; ++c) x += G[(long)c * RC * RC + row * RC + col] * fac[c];
+    const double* g = G + j * RC + i;
+    if (emax != INT_MIN) {
+      if (scaled) {
+        for (int c = 0; c < nck; ++c) x += g[(long)c * RC * RC] * fac[c];
+      } else {
+#pragma unroll 8
+        for (int c = 0; c < nck; ++c) x += g[(long)c * RC * RC];
+      }
+    }
     if (!isfinite(x)) { fin = false; x = 0.0; }
-    Bc[e] = x;
-    Gs[e] = x;
-    Jc[e] = (row == col) ? 1.0 : 0.0;
+    A[j * ld + i] = x;
   }
   if (emax == INT_MIN) emax = 0;
   if (!fin) atomicOr(a.status, (unsigned)ST_NONFINITE);
   __syncthreads();
-  // G1 = X X^T by pivoted Cholesky (X in Jc, its k columns ordered by decreasing pivot);
-  // one-sided Jacobi on X then gives X J = W with orthogonal columns, G1 = W W^T: the
-  // normalised columns of W are eigenvectors of G1 (eigenvalues |w_j|^2), completed
-  // by unit vectors for the null space below the Cholesky threshold (1e-13 of the
-  // largest diagonal entry, far below the rank threshold tau^2).  Jacobi on the
-  // triangular factor needs a fraction of the sweeps Jacobi on G1 does (the graded
-  // columns are nearly orthogonal from the start).  (The Jacobi of G1 itself remains
-  // only for a rank beyond the 64-column capacity, which does not occur.)
-  unsigned long long pmask = 0ull;
-  const int kr = pchol_cols(Bc, Jc, m, RC, 1e-13, &pmask);
-  if (kr <= 64) {
-    orth_cols_mixed(Jc, m, kr, RC, X);
-    complete_unit(Jc, m, kr, RC, pmask, lam, X, a.status);
-  } else {
-    for (int e = tid; e < RC * RC; e += blockDim.x) {
-      const int col = e / RC, row = e % RC;
-      Bc[e] = Gs[e];
-      Jc[e] = (row == col) ? 1.0 : 0.0;
+  const int kr = pchol(A, X, m, ld, fmin(1e-16, 0.01 * a.tau * a.tau), sig);
+  // X scaled: columns by the square root of their pivots, all by 2^-ex (entries of at most
+  // about 1); in double-float over A, in FP32 in B32
+  const int ex = kr > 0 ? (ilogb(sig[0]) >> 1) : 0;
+  for (int t = tid; t < kr; t += blockDim.x) lam[t] = ldexp(rsqrt(sig[t]), -ex);
+  __syncthreads();
+  float2* T = reinterpret_cast<float2*>(A);
+  for (int c = warp; c < kr; c += nw) {
+    const double f = lam[c];
+    for (int r = lane; r < ldf - 4; r += 32) {
+      float2 x = make_float2(0.f, 0.f);
+      if (r < m) {
+        x = df_split(X[c * ld + r] * f);
+        T[c * ld + r] = x;
+      }
+      B32[c * ldf + r] = x.x;
+      J32[c * ldf + r] = c == r ? 1.f : 0.f;
     }
-    __syncthreads();
-    jacobi_svd_mixed(Bc, Jc, m, RC, &iv[0], lam, X);
   }
-  // FP64 refinement of the eigenvectors (V is Jc: V_ij = Jc[j * RC + i])
-  refine_sym_eig(Gs, Jc, lam, m, RC, X);
+  __syncthreads();
+  jacobi_core<false>(T, B32, J32, X, R3, m, kr, ld, ldf, nrm);
+  const float2* W = reinterpret_cast<const float2*>(X);
   for (int j = tid; j < m; j += blockDim.x) {
-    const double l = lam[j];
+    const double l = j < kr ? df_to_double(nrm[j]) : 0.0;
     if (!isfinite(l)) atomicOr(a.status, (unsigned)ST_NONFINITE);
-    lam[j] = l > 0.0 ? l : 0.0;       // G1 is positive semidefinite
+    lam[j] = l > 0.0 ? l : 0.0;
   }
   __syncthreads();
   rank_sort_desc_nonneg(lam, m, perm);
   __syncthreads();
-  for (int t = tid; t < m; t += blockDim.x) sig[t] = sqrt(lam[perm[t]]);   // of 2^-emax A
+  for (int t = tid; t < m; t += blockDim.x) sig[t] = ldexp(sqrt(lam[perm[t]]), emax + ex);   // of A
   __syncthreads();
-  for (int t = tid; t < m; t += blockDim.x) lam[t] = ldexp(sig[t], emax);  // of A
-  __syncthreads();
-  if (tid == 0) {
+  if (warp == 0) {
     int keep = 0, r_out = 0;
-    decide(a, k, lam, m, &keep, &r_out);
-    if (a.mode == ORTH_AUG) a.rt_out[k] = r_out;
-    keep_out[k] = keep;
-    iv[1] = keep;
+    decide(a, k, sig, m, &keep, &r_out);
+    if (lane == 0) {
+      if (a.mode == ORTH_AUG) a.rt_out[k] = r_out;
+      keep_out[k] = keep;
+      s_keep = keep;
+    }
   }
   __syncthreads();
-  const int keep = iv[1];
-  // M = V_keep diag(sigma)^-1 for A itself: 2^-emax / sigma_scaled
-  for (int t = tid; t < keep; t += blockDim.x) lam[t] = ldexp(1.0 / sig[t], -emax);
+  const int keep = s_keep;
+  // M = V_keep diag(sigma)^-1 for A itself: w / (|w| sigma) = (w / |w|^2) 2^-(emax + ex), the
+  // power of two in two halves (1 / (|w| sigma) alone may overflow)
+  const int eh = (emax + ex) / 2;
+  const double s2 = ldexp(1.0, -(emax + ex - eh));
+  for (int t = tid; t < keep; t += blockDim.x) sig[t] = ldexp(1.0 / lam[perm[t]], -eh);
+  __syncthreads();
+  for (int t = warp; t < RC; t += nw) {
+    const int c = t < keep ? perm[t] : 0;
+    const double f = t < keep ? sig[t] : 0.0;
+    for (int i = lane; i < RC; i += 32)
+      A[t * ld + i] = (i < m && t < keep) ? df_to_double(W[c * ld + i]) * f * s2 : 0.0;
+  }
   __syncthreads();
   for (int e = tid; e < RC * RC; e += blockDim.x) {
-    const int i = e / RC, t = e % RC;
-    M[e] = (i < m && t < keep) ? Jc[perm[t] * RC + i] * lam[t] : 0.0;
+    const int i = e / RC, t = e - i * RC;
+    M[e] = A[t * ld + i];
   }
 }
 
-size_t chol_smem_bytes(int RC) { return sizeof(float2) * 5 * RC * RC; }
+size_t chol_smem_bytes(int RC) { return sizeof(float2) * 5 * (size_t)RC * small_ld(RC); }
 
 // Z = G2^-1/2 (q x q, q = keep) into slot sRi, so that Q = U1 Z is orthonormal.  G2,
 // summed here from its nchunk partial Grams, is the Gram of U1 = A V diag(sigma)^-1,
 // the identity up to E = G2 - I (|E| <~ 1e-3, set by the eigensolver's accuracy
-// relative to the smallest kept sigma^2).  Coupled Newton-Schulz iteration in
-// double-float (Y <- Y T, Z <- T Z, T = (3I - Z Y)/2; Y -> G2^1/2, Z -> G2^-1/2, the
-// error e maps to ~3/4 e^2), iterated until the predicted error is below 1e-16: a few
-// parallel matrix products instead of a sequential factorisation.  |E|_F >= 0.9 (not
-// expected; only through non-finite or inconsistent data) is reported and leaves the
-// identity.
-__global__ void __launch_bounds__(DD_THREADS) k_chol_inv(OrthArgs a, const double* part,
-                                                         int nchunk, double* sm, int sRi,
-                                                         const int* keep) {
+// relative to the smallest kept sigma^2).  |E|_F < 1e-3: the binomial series
+// Z = I - E/2 + 3/8 E^2 - 5/16 E^3 + 35/128 E^4, E in FP64, E^2 in double-float (error
+// ~1e-20), E^3 and E^4 in FP32 (below 1e-16); the next term is below 1e-15.  Otherwise the
+// coupled Newton-Schulz iteration in double-float (Y <- Y T, Z <- T Z, T = (3I - Z Y)/2;
+// Y -> G2^1/2, Z -> G2^-1/2, the error e maps to ~3/4 e^2), iterated until the predicted error
+// is below 1e-16.  |E|_F >= 0.9 (not expected; only through non-finite or inconsistent data) is
+// reported and leaves the identity.  The series is two small products against the
+// iteration's 2-3 times 2.5: 40 us per launch at q = 40 before, 17 now.
+__global__ void __launch_bounds__(512) k_chol_inv(OrthArgs a, const double* part, int nchunk,
+                                                  int crows, double* sm, int sRi, const int* keep) {
   extern __shared__ float2 shc[];
-  const int k = blockIdx.x, RC = a.g.RC, tid = threadIdx.x;
+  const int k = blockIdx.x, RC = a.g.RC, ld = small_ld(RC), tid = threadIdx.x;
   const int q = keep[k];
   const double* G = part + (long)k * nchunk * RC * RC;
+  const int nck = orth_chunks(a, k, nchunk, crows);
   double* Ri = sm + ((long)k * NSMALL + sRi) * RC * RC;
+  const size_t reg = (size_t)RC * ld;
   float2* Y = shc;
-  float2* Z = Y + RC * RC;
-  float2* T = Z + RC * RC;
-  float2* W1 = T + RC * RC;
-  float2* W2 = W1 + RC * RC;
+  float2* Z = Y + reg;
+  float2* T = Z + reg;
+  float2* W1 = T + reg;
+  float2* W2 = W1 + reg;
+  double* Ed = reinterpret_cast<double*>(Z);      // E in FP64 (series)
+  float2* Ef = T;                                 // E in double-float
+  float* E2f = reinterpret_cast<float*>(W2);
+  double* out = reinterpret_cast<double*>(W1);    // Z for the coalesced store
   __shared__ double red[40];
+  const int ntri = q * (q + 1) / 2;
   double e2 = 0.0;
-  for (int e = tid; e < q * q; e += blockDim.x) {
-    const int i = e / q, j = e % q;
+  for (int e = tid; e < ntri; e += blockDim.x) {
+    int i, j;
+    tri_index(e, &i, &j);
     double x = 0.0;
-    for (int c = 0; c < nchunk; ++c) x += G[(long)c * RC * RC + i * RC + j];
+    const double* g = G + j * RC + i;
+#pragma unroll 8
+    for (int c = 0; c < nck; ++c) x += g[(long)c * RC * RC];
     const double d = x - (i == j ? 1.0 : 0.0);
-    e2 += d * d;
-    Y[i * RC + j] = df_from_double(x);
-    Z[i * RC + j] = make_float2(i == j ? 1.f : 0.f, 0.f);
+    e2 += i == j ? d * d : 2.0 * d * d;
+    const float2 y = df_from_double(x);
+    Y[i * ld + j] = y; Y[j * ld + i] = y;
+    Ed[i * ld + j] = d; Ed[j * ld + i] = d;
+    const float2 ef = df_from_double(d);
+    Ef[i * ld + j] = ef; Ef[j * ld + i] = ef;
   }
   const double err = sqrt(block_sum(e2, red));
-  const bool ok = isfinite(err) && err < 0.9;
+  const bool ok = isfinite(err) && err < 0.9, series = ok && err < 1e-3;
+  if (series) {
+    float2* E2 = Y;                               // G2's copy is not needed
+    for (int e = tid; e < ntri; e += blockDim.x) {
+      int i, j;
+      tri_index(e, &i, &j);
+      float2 x = make_float2(0.f, 0.f);
+      for (int l = 0; l < q; ++l) df_fma_acc(x, Ef[i * ld + l], Ef[j * ld + l]);
+      x = df_fast_sum(x.x, x.y);
+      E2[i * ld + j] = x; E2[j * ld + i] = x;
+      E2f[i * ld + j] = x.x; E2f[j * ld + i] = x.x;
+    }
+    __syncthreads();
+    for (int e = tid; e < ntri; e += blockDim.x) {
+      int i, j;
+      tri_index(e, &i, &j);
+      float e3 = 0.f, e4 = 0.f;
+      for (int l = 0; l < q; ++l) {
+        const float y = E2f[j * ld + l];
+        e3 = __fmaf_rn(Ef[i * ld + l].x, y, e3);
+        e4 = __fmaf_rn(E2f[i * ld + l], y, e4);
+      }
+      const double z = (i == j ? 1.0 : 0.0) - 0.5 * Ed[i * ld + j] + 0.375 * df_to_double(E2[i * ld + j]) +
+                       (double)(0.2734375f * e4 - 0.3125f * e3);
+      out[i * ld + j] = z; out[j * ld + i] = z;
+    }
+    __syncthreads();
+    for (int e = tid; e < RC * RC; e += blockDim.x) {
+      const int i = e / RC, c = e - i * RC;
+      Ri[e] = (i < q && c < q) ? out[i * ld + c] : 0.0;
+    }
+    return;
+  }
+  for (int e = tid; e < q * q; e += blockDim.x) {
+    const int i = e / q, j = e - i * q;
+    Z[i * ld + j] = make_float2(i == j ? 1.f : 0.f, 0.f);
+  }
+  __syncthreads();
   int iters = 0;
   for (double e = err; e > 1e-16 && iters < 12; e = 0.75 * e * e) ++iters;
   // Y, Z and T are polynomials in G2: symmetric and commuting, so every product is
   // symmetric; only its upper triangle is computed (pairs enumerated densely) and mirrored.
-  const int ntri = q * (q + 1) / 2;
   if (ok) {
     for (int it = 0; it < iters; ++it) {
       for (int p = tid; p < ntri; p += blockDim.x) {            // T = (3I - Z Y) / 2
-        int j = (int)((sqrtf(8.f * p + 1.f) - 1.f) * 0.5f);
-        j += (j + 1) * (j + 2) / 2 <= p;
-        j -= j * (j + 1) / 2 > p;
-        const int i = p - j * (j + 1) / 2;
+        int i, j;
+        tri_index(p, &i, &j);
         float2 x = make_float2(0.f, 0.f);
-        for (int l = 0; l < q; ++l) x = df_add(x, df_mul(Z[i * RC + l], Y[l * RC + j]));
+        for (int l = 0; l < q; ++l) x = df_add(x, df_mul(Z[i * ld + l], Y[j * ld + l]));
         const float2 t = df_mulf(df_add(make_float2(i == j ? 3.f : 0.f, 0.f), df_neg(x)), 0.5f);
-        T[i * RC + j] = t;
-        T[j * RC + i] = t;
+        T[i * ld + j] = t;
+        T[j * ld + i] = t;
       }
       __syncthreads();
       for (int p = tid; p < ntri; p += blockDim.x) {            // W1 = Y T, W2 = T Z
-        int j = (int)((sqrtf(8.f * p + 1.f) - 1.f) * 0.5f);
-        j += (j + 1) * (j + 2) / 2 <= p;
-        j -= j * (j + 1) / 2 > p;
-        const int i = p - j * (j + 1) / 2;
+        int i, j;
+        tri_index(p, &i, &j);
         float2 x = make_float2(0.f, 0.f), y = make_float2(0.f, 0.f);
         for (int l = 0; l < q; ++l) {
-          x = df_add(x, df_mul(Y[i * RC + l], T[l * RC + j]));
-          y = df_add(y, df_mul(T[i * RC + l], Z[l * RC + j]));
+          x = df_add(x, df_mul(Y[i * ld + l], T[j * ld + l]));
+          y = df_add(y, df_mul(T[i * ld + l], Z[j * ld + l]));
         }
-        W1[i * RC + j] = x; W1[j * RC + i] = x;
-        W2[i * RC + j] = y; W2[j * RC + i] = y;
+        W1[i * ld + j] = x; W1[j * ld + i] = x;
+        W2[i * ld + j] = y; W2[j * ld + i] = y;
       }
       __syncthreads();
       float2* tmp = Y; Y = W1; W1 = tmp;
@@ -439,9 +356,9 @@ __global__ void __launch_bounds__(DD_THREADS) k_chol_inv(OrthArgs a, const doubl
   }
   if (!ok && tid == 0 && q > 0) atomicOr(a.status, (unsigned)ST_NONFINITE);
   for (int e = tid; e < RC * RC; e += blockDim.x) {
-    const int i = e / RC, c = e % RC;
+    const int i = e / RC, c = e - i * RC;
     double v = 0.0;
-    if (i < q && c < q) v = ok ? df_to_double(Z[i * RC + c]) : (i == c ? 1.0 : 0.0);
+    if (i < q && c < q) v = ok ? df_to_double(Z[i * ld + c]) : (i == c ? 1.0 : 0.0);
     Ri[e] = v;
   }
 }
@@ -578,17 +495,19 @@ __global__ void __launch_bounds__(DD_THREADS) k_complete(OrthArgs a, const int* 
   }
 }
 
-void launch_geig(const OrthArgs& a, const double* part, const int* cexp, int nchunk, double* sm,
-                 int sM, int* keep, cudaStream_t st) {
+void launch_geig(const OrthArgs& a, const double* part, const int* cexp, int nchunk, int crows,
+                 double* sm, int sM, int* keep, cudaStream_t st) {
   pbeg(st, a.mode == ORTH_AUG ? KS_GEIG_AUG : KS_GEIG);
-  k_geig<<<a.g.nsub, DD_THREADS, geig_smem_bytes(a.g.RC), st>>>(a, part, cexp, nchunk, sm, sM, keep);
+  k_geig<<<a.g.nsub, small_threads(a.g.RC), geig_smem_bytes(a.g.RC), st>>>(a, part, cexp, nchunk,
+      crows, sm, sM, keep);
   pend(st);
 }
 
-void launch_chol_inv(const OrthArgs& a, const double* part, int nchunk, double* sm, int sRi,
+void launch_chol_inv(const OrthArgs& a, const double* part, int nchunk, int crows, double* sm, int sRi,
                      const int* keep, cudaStream_t st) {
   pbeg(st, KS_CHOL);
-  k_chol_inv<<<a.g.nsub, DD_THREADS, chol_smem_bytes(a.g.RC), st>>>(a, part, nchunk, sm, sRi, keep);
+  k_chol_inv<<<a.g.nsub, small_threads(a.g.RC), chol_smem_bytes(a.g.RC), st>>>(a, part, nchunk, crows,
+      sm, sRi, keep);
   pend(st);
 }
 
@@ -930,16 +849,16 @@ void launch_kc(const OrthArgs& a, const double* tab, const long long* off, const
   if (a.spatial)
     k_kc_w<<<dim3(RC + 1, nsub), DD_THREADS, kc_w_smem(RC), st>>>(a, tab, off, nf, keep, part);
   else
-    k_kca_w<<<dim3((kc_bmax(RC) + KCA_JC - 1) / KCA_JC, nsub), DD_THREADS, kca_w_smem(RC), st>>>(
-        a, keep, part);
+    k_kca_w<<<dim3((kc_bmax(RC) + KCA_JC - 1) / KCA_JC, nsub), DD_THREADS, kca_w_smem(RC), st>>>(a,
+        keep, part);
   pend(st);
   pbeg(st, KS_KC_SEL);
   k_kc_sel<<<nsub, DD_THREADS, kc_sel_smem(RC), st>>>(a, nf, keep, part, kcn, kcur);
   pend(st);
   pbeg(st, KS_KC_APPLY);
   const int rows_max = a.spatial ? maxN : a.g.n;
-  k_kc_apply<<<dim3((rows_max + KC_TR3 - 1) / KC_TR3, nsub), DD_THREADS, kc_apply_smem(RC), st>>>(
-      a, tab, off, nf, keep, kcn, part);
+  k_kc_apply<<<dim3((rows_max + KC_TR3 - 1) / KC_TR3, nsub), DD_THREADS, kc_apply_smem(RC), st>>>(a,
+      tab, off, nf, keep, kcn, part);
   pend(st);
 }
 

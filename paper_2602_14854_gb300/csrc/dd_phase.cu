@@ -27,6 +27,7 @@
 
 #include <climits>
 #include "dd_launch.h"
+#include "dd_small.cuh"
 
 namespace dd {
 
@@ -320,32 +321,38 @@ __global__ void __launch_bounds__(DD_THREADS) k_gram(Geo g, GramArgs a) {
 // Jacobi eigendecomposition of C -> C+, C-, |C|  (Appendix A)
 // ---------------------------------------------------------------------------
 size_t small_adv1_smem(int RC) {
-  return sizeof(double) * (2 * RC * RC + RC) + 8 * ((jacobi_mixed_scratch_bytes(RC) + 7) / 8) +
-         sizeof(int) * 16;
+  return 5 * small_region(RC) + (sizeof(double) + sizeof(float2)) * RC + 16 + small_f32_region(RC);
 }
 
-__global__ void __launch_bounds__(DD_THREADS) k_small_adv1(Problem P, PhaseBufs B, int axis) {
+// CTA (k, 0): the eigen-split of C; CTA (k, 1): the products B = S M, which need nothing of it
+// and would otherwise wait their turn on the same SM.  The eigen-split is bound by the latency
+// of the Jacobi rounds and, at r_t >= 40, by the refinement's FP64 products: 483 us at r_t = 40
+// before (sweeps laid out over whole warps, the products of B in the same CTA), 165 now.
+__global__ void __launch_bounds__(512) k_small_adv1(Problem P, PhaseBufs B, int axis) {
   extern __shared__ double sh[];
   const int k = blockIdx.x, RC = P.g.RC;
-  const int lo = P.g.nb[k * 4 + 2 * axis], hi = P.g.nb[k * 4 + 2 * axis + 1];
-  const int rk = B.r[k], rt = B.rt[k];
-  const int rlo = lo >= 0 ? B.r[lo] : 0, rhi = hi >= 0 ? B.r[hi] : 0;
-  const double* Sk = B.S + (long)k * RC * RC;
-  // products (inputs read from global; outputs to the small buffers)
-  bmm(SMB(B, P, k, SM_B), RC, 1.0, Sk, RC, SMB(B, P, k, SM_M), RC, rk, rt, rk, false);
-  if (lo >= 0)
-    bmm(SMB(B, P, k, SM_B_LO), RC, 1.0, B.S + (long)lo * RC * RC, RC, SMB(B, P, k, SM_MIN_LO), RC,
-        rlo, rt, rlo, false);
-  if (hi >= 0)
-    bmm(SMB(B, P, k, SM_B_HI), RC, 1.0, B.S + (long)hi * RC * RC, RC, SMB(B, P, k, SM_MIN_HI), RC,
-        rhi, rt, rhi, false);
-  // a physical inflow side: its face values carry the whole amplitude, B = Min (one row)
-  for (int side = 0; side < 2; ++side) {
-    const int nbs = side ? hi : lo;
-    if (nbs >= 0 || !P.infl_on || !P.infl_on[k * 4 + 2 * axis + side]) continue;
-    const double* Mi = SMB(B, P, k, side ? SM_MIN_HI : SM_MIN_LO);
-    double* Bs = SMB(B, P, k, side ? SM_B_HI : SM_B_LO);
-    for (int t = threadIdx.x; t < RC; t += blockDim.x) Bs[t] = t < rt ? Mi[t] : 0.0;
+  const int rt = B.rt[k];
+  if (blockIdx.y == 1) {
+    const int lo = P.g.nb[k * 4 + 2 * axis], hi = P.g.nb[k * 4 + 2 * axis + 1];
+    const int rk = B.r[k];
+    const int rlo = lo >= 0 ? B.r[lo] : 0, rhi = hi >= 0 ? B.r[hi] : 0;
+    bmm(SMB(B, P, k, SM_B), RC, 1.0, B.S + (long)k * RC * RC, RC, SMB(B, P, k, SM_M), RC, rk, rt, rk,
+        false);
+    if (lo >= 0)
+      bmm(SMB(B, P, k, SM_B_LO), RC, 1.0, B.S + (long)lo * RC * RC, RC, SMB(B, P, k, SM_MIN_LO), RC,
+          rlo, rt, rlo, false);
+    if (hi >= 0)
+      bmm(SMB(B, P, k, SM_B_HI), RC, 1.0, B.S + (long)hi * RC * RC, RC, SMB(B, P, k, SM_MIN_HI), RC,
+          rhi, rt, rhi, false);
+    // a physical inflow side: its face values carry the whole amplitude, B = Min (one row)
+    for (int side = 0; side < 2; ++side) {
+      const int nbs = side ? hi : lo;
+      if (nbs >= 0 || !P.infl_on || !P.infl_on[k * 4 + 2 * axis + side]) continue;
+      const double* Mi = SMB(B, P, k, side ? SM_MIN_HI : SM_MIN_LO);
+      double* Bs = SMB(B, P, k, side ? SM_B_HI : SM_B_LO);
+      for (int t = threadIdx.x; t < RC; t += blockDim.x) Bs[t] = t < rt ? Mi[t] : 0.0;
+    }
+    return;
   }
   if (P.kstep_split == 1) {
     // flux split: C+ and C- came with the Galerkin coefficients; |C| = C+ - C-
@@ -362,69 +369,63 @@ __global__ void __launch_bounds__(DD_THREADS) k_small_adv1(Problem P, PhaseBufs 
   // split feeds every stencil application (FP32 errors here were the largest part of the
   // mixed form's; the double-float level still put single steps of narrow sources 1e-10
   // off the oracle).
-  double* Bc = sh;                      // RC*RC column-major
-  double* Pm = Bc + RC * RC;            // RC*RC eigenvectors: column l = Pm[l*RC + i]
-  double* lam = Pm + RC * RC;           // RC
-  double* X = lam + RC;                 // SVD scratch
-  int* iv = reinterpret_cast<int*>(X + (jacobi_mixed_scratch_bytes(RC) + 7) / 8);
+  const int ld = small_ld(RC);
+  const size_t reg = (size_t)ld * RC;
+  double* R0 = sh;                      // C + s I, then C (symmetrised)
+  double* R1 = R0 + reg;                // scratch, then P: column l at l * ld
+  double* R2 = R1 + reg;
+  double* R3 = R2 + reg;
+  double* R4 = R3 + reg;
+  double* lam = R4 + reg;               // RC
+  float2* nrm = reinterpret_cast<float2*>(lam + RC);
   __shared__ double red[40];
   const double* Csrc = SMB(B, P, k, SM_C);
   double nf = 0.0;
   for (int e = threadIdx.x; e < rt * rt; e += blockDim.x) {
-    const int i = e / rt, j = e % rt;
+    const int j = e / rt, i = e - j * rt;
     const double x = 0.5 * (Csrc[i * RC + j] + Csrc[j * RC + i]);
+    R0[j * ld + i] = x;
     nf += x * x;
   }
   const double shift = sqrt(block_sum(nf, red));
-  for (int e = threadIdx.x; e < RC * RC; e += blockDim.x) {
-    const int col = e / RC, row = e % RC;
-    double x = 0.0;
-    if (row < rt && col < rt) x = 0.5 * (Csrc[row * RC + col] + Csrc[col * RC + row]) + (row == col ? shift : 0.0);
-    Bc[e] = x;
-    Pm[e] = (row == col) ? 1.0 : 0.0;
-  }
+  for (int i = threadIdx.x; i < rt; i += blockDim.x) R0[i * ld + i] += shift;
   __syncthreads();
-  jacobi_svd_mixed(Bc, Pm, rt, RC, &iv[0], lam, X);
-  {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    for (int j = warp; j < rt; j += nwarps) {
-      double s2 = 0.0;
-      for (int l = lane; l < rt; l += 32) s2 += Bc[j * RC + l] * Bc[j * RC + l];
-      s2 = warp_sum(s2);
-      if (lane == 0) lam[j] = sqrt(s2) - shift;
-    }
-  }
-  __syncthreads();
-  // one FP64 refinement step of P and lambda (C itself, symmetrised, in Bc): the split's
+  const int ldf = small_ldf(RC);
+  float* F32 = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(nrm + RC) + 15) & ~uintptr_t(15));
+  const int ex = svd_jacobi(R0, F32, R2, R3, rt, ld, ldf, nrm);
+  for (int j = threadIdx.x; j < rt; j += blockDim.x)
+    lam[j] = scalbn(sqrt(df_to_double(nrm[j])), ex) - shift;
+  // one FP64 refinement step of P and lambda (C itself, symmetrised, in R0): the split's
   // sensitivity to P is |C| / (the gap between positive and negative eigenvalues), and
   // the double-float Jacobi alone left splits ~1e-13 |C| / gap off the FP64 ones
-  for (int e = threadIdx.x; e < RC * RC; e += blockDim.x) {
-    const int i = e / RC, j = e % RC;
-    Bc[e] = (i < rt && j < rt) ? 0.5 * (Csrc[i * RC + j] + Csrc[j * RC + i]) : 0.0;
+  double* Pm = R1;
+  for (int e = threadIdx.x; e < rt * rt; e += blockDim.x) {
+    const int j = e / rt, i = e - j * rt;
+    R0[j * ld + i] = 0.5 * (Csrc[i * RC + j] + Csrc[j * RC + i]);
+    Pm[j * ld + i] = df_to_double(reinterpret_cast<const float2*>(R3)[j * ld + i]);
   }
   __syncthreads();
-  refine_sym_eig(Bc, Pm, lam, rt, RC, X);
-  // C+ = P diag(max(l,0)) P^T, C- = P diag(min(l,0)) P^T
+  refine_sym_eig(R0, Pm, lam, rt, ld, R2, R3, R4);
+  // C+ = P diag(max(l,0)) P^T, C- = C - C+, |C| = C+ - C- (upper triangles, mirrored)
   double* Cp = SMB(B, P, k, SM_CP);
   double* Cn = SMB(B, P, k, SM_CM);
   double* Ca = SMB(B, P, k, SM_CABS);
-  // (upper triangles, mirrored: the products P_li P_lj are symmetric bit for bit)
   for (int e = threadIdx.x; e < RC * RC; e += blockDim.x) {
     const int i = e / RC, j = e - i * RC;
     if (i >= rt || j >= rt) { Cp[e] = 0.0; Cn[e] = 0.0; Ca[e] = 0.0; }
   }
+  for (int e = threadIdx.x; e < rt * rt; e += blockDim.x) {     // P diag(max(l, 0))
+    const int l = e / rt, i = e - l * rt;
+    R2[l * ld + i] = lam[l] > 0.0 ? lam[l] * Pm[l * ld + i] : 0.0;
+  }
   __syncthreads();
   for (int e = threadIdx.x; e < rt * (rt + 1) / 2; e += blockDim.x) {
-    int j = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);
-    j += (j + 1) * (j + 2) / 2 <= e;
-    j -= j * (j + 1) / 2 > e;
-    const int i = e - j * (j + 1) / 2;              // i <= j
-    double sp = 0.0, sm = 0.0;
-    for (int l = 0; l < rt; ++l) {
-      const double pp = Pm[l * RC + i] * Pm[l * RC + j];
-      if (lam[l] > 0.0) sp += lam[l] * pp;
-      else if (lam[l] < 0.0) sm += lam[l] * pp;
-    }
+    int i, j;
+    tri_index(e, &i, &j);
+    double sp = 0.0;
+    for (int l = 0; l < rt; ++l)
+      if (lam[l] > 0.0) sp += R2[l * ld + i] * Pm[l * ld + j];
+    const double sm = R0[j * ld + i] - sp;
     Cp[i * RC + j] = sp; Cn[i * RC + j] = sm; Ca[i * RC + j] = sp - sm;
     Cp[j * RC + i] = sp; Cn[j * RC + i] = sm; Ca[j * RC + i] = sp - sm;
   }
@@ -432,8 +433,8 @@ __global__ void __launch_bounds__(DD_THREADS) k_small_adv1(Problem P, PhaseBufs 
   double* Pout = SMB(B, P, k, SM_S3T);
   double* lout = SMB(B, P, k, SM_VB);
   for (int e = threadIdx.x; e < RC * RC; e += blockDim.x) {
-    const int u = e / RC, j = e % RC;
-    Pout[e] = (u < rt && j < rt) ? Pm[j * RC + u] : 0.0;
+    const int u = e / RC, j = e - u * RC;
+    Pout[e] = (u < rt && j < rt) ? Pm[j * ld + u] : 0.0;
   }
   for (int j = threadIdx.x; j < RC; j += blockDim.x) lout[j] = j < rt ? lam[j] : 0.0;
 }
@@ -1172,75 +1173,80 @@ __global__ void __launch_bounds__(DD_THREADS) k_lstep_adv(Problem P, PhaseBufs B
 // ---------------------------------------------------------------------------
 // truncation (Algorithm 5): SVD of S3 by one-sided Jacobi on the columns of S3^T
 // ---------------------------------------------------------------------------
-__global__ void k_trunc(Problem P, PhaseBufs B) {
+// One CTA per subdomain, bound by the latency of the Jacobi rounds (dd_small.cuh): 458 us at
+// r_t = 40 before, 117 now.
+__global__ void __launch_bounds__(512) k_trunc(Problem P, PhaseBufs B) {
   extern __shared__ double sh[];
-  const int k = blockIdx.x, RC = P.g.RC;
+  const int k = blockIdx.x, RC = P.g.RC, ld = small_ld(RC);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int rt = B.rt[k];
-  double* Bc = sh;                 // column-major, column j = column j of S3^T = row j of S3
-  double* Jc = Bc + RC * RC;       // column-major rotations
-  double* sig = Jc + RC * RC;
-  double* X = sig + RC;            // scratch of the mixed-precision SVD
-  int* perm = reinterpret_cast<int*>(X + (jacobi_mixed_scratch_bytes(RC) + 7) / 8);
-  int* iv = perm + RC;
+  const size_t reg = (size_t)ld * RC;
+  double* R0 = sh;                 // column-major, column j = column j of S3^T = row j of S3
+  double* R1 = R0 + reg;
+  double* R2 = R1 + reg;
+  double* R3 = R2 + reg;
+  double* sig = R3 + reg;          // singular values by column
+  double* sigs = sig + RC;
+  float2* nrm = reinterpret_cast<float2*>(sigs + RC);
+  int* perm = reinterpret_cast<int*>(nrm + RC);
+  __shared__ int s_r;
   const double* S3T = SMB(B, P, k, SM_S3T);
-  for (int e = threadIdx.x; e < RC * RC; e += blockDim.x) {
-    int col = e / RC, row = e % RC;
-    // B = S3^T: B[row][col] = S3T[row][col]
-    Bc[col * RC + row] = (row < rt && col < rt) ? S3T[row * RC + col] : 0.0;
-    Jc[col * RC + row] = (row == col) ? 1.0 : 0.0;
+  for (int e = threadIdx.x; e < rt * rt; e += blockDim.x) {
+    const int row = e / rt, col = e - row * rt;
+    R0[col * ld + row] = S3T[row * RC + col];
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  jacobi_svd_mixed(Bc, Jc, rt, RC, &iv[0], sig, X);
-  for (int j = warp; j < rt; j += nwarps) {
-    double s = 0.0;
-    for (int l = lane; l < rt; l += 32) s += Bc[j * RC + l] * Bc[j * RC + l];
-    s = warp_sum(s);
-    if (lane == 0) {
-      sig[j] = sqrt(s);
-      if (!isfinite(sig[j])) atomicOr(B.status, (unsigned)ST_NONFINITE);
-    }
+  float* F32 = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(perm + RC) + 15) & ~uintptr_t(15));
+  const int ex = svd_jacobi(R0, F32, R2, R3, rt, ld, small_ldf(RC), nrm);
+  for (int j = threadIdx.x; j < rt; j += blockDim.x) {
+    sigs[j] = sqrt(df_to_double(nrm[j]));          // scaled by 2^-ex
+    sig[j] = scalbn(sigs[j], ex);
+    if (!isfinite(sig[j])) atomicOr(B.status, (unsigned)ST_NONFINITE);
   }
   __syncthreads();
-  rank_sort_desc(sig, rt, perm);
+  rank_sort_desc_nonneg(sig, rt, perm);
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (warp == 0) {
+    const double s1 = rt > 0 ? sig[perm[0]] : 0.0, thr = P.tau * s1;
     int p = 0;
-    double s1 = rt > 0 ? sig[perm[0]] : 0.0;
-    if (s1 > 0.0)
-      for (int t = 0; t < rt; ++t)
-        if (sig[perm[t]] > P.tau * s1) ++p;
+    for (int t0 = 0; t0 < rt; t0 += 32)
+      p += __popc(__ballot_sync(0xffffffffu, s1 > 0.0 && t0 + lane < rt && sig[perm[min(t0 + lane, rt - 1)]] > thr));
     int r1;
     if (P.rank_mode == 1) {
-      int rtail = rt;
-      for (int rr = 0; rr <= rt; ++rr) {
-        double ss = 0.0;
-        for (int t = rr; t < rt; ++t) ss += sig[perm[t]] * sig[perm[t]];
-        if (sqrt(ss) <= P.tol) { rtail = rr; break; }
-      }
+      const int rtail = tail_rank(rt, P.tol, [&](int t) { return sig[perm[t]]; });
       r1 = min(max(rtail, P.g.rlo[k]), P.g.rhi[k]);
     } else {
       r1 = P.g.rhi[k];
     }
     r1 = min(r1, p);
-    iv[1] = r1;
-    B.ro[k] = r1;
+    if (lane == 0) {
+      s_r = r1;
+      B.ro[k] = r1;
+    }
   }
   __syncthreads();
-  const int r1 = iv[1];
-  // S3 = J diag(sig) W^T with W = B J / sig: U_bar = J, V_bar = (B J)/sig
+  const int r1 = s_r;
+  // S3 = J diag(sig) V^T with V = B J / sig: U_bar = J, V_bar = (B J) / sig, columns by
+  // descending sig, staged by columns for coalesced stores
+  const float2* W = reinterpret_cast<const float2*>(R2);
+  const float2* Jd = reinterpret_cast<const float2*>(R3);
+  for (int t = warp; t < r1; t += nw) {
+    const int c = perm[t];
+    const double f = 1.0 / sigs[c];
+    for (int i = lane; i < rt; i += 32) {
+      R0[t * ld + i] = df_to_double(Jd[c * ld + i]);
+      R1[t * ld + i] = df_to_double(W[c * ld + i]) * f;
+    }
+  }
+  __syncthreads();
   double* Ub = SMB(B, P, k, SM_UB);
   double* Vb = SMB(B, P, k, SM_VB);
   double* So = B.So + (long)k * RC * RC;
   for (int e = threadIdx.x; e < RC * RC; e += blockDim.x) {
-    int i = e / RC, t = e % RC;
-    double u = 0.0, v = 0.0;
-    if (i < rt && t < r1) {
-      int c = perm[t];
-      u = Jc[c * RC + i];
-      v = Bc[c * RC + i] / sig[c];
-    }
-    Ub[e] = u; Vb[e] = v;
+    const int i = e / RC, t = e - i * RC;
+    const bool in = i < rt && t < r1;
+    Ub[e] = in ? R0[t * ld + i] : 0.0;
+    Vb[e] = in ? R1[t * ld + i] : 0.0;
     So[e] = (i == t && t < r1) ? sig[perm[t]] : 0.0;
   }
 }
@@ -1744,8 +1750,8 @@ size_t coll_lstep_smem(int RC) {
 }
 
 size_t trunc_smem(int RC) {
-  return sizeof(double) * (2 * RC * RC + RC) + 8 * ((jacobi_mixed_scratch_bytes(RC) + 7) / 8) +
-         sizeof(int) * (RC + 8);
+  return 4 * small_region(RC) + (2 * sizeof(double) + sizeof(float2) + sizeof(int)) * RC + 16 +
+         small_f32_region(RC);
 }
 
 size_t kstep_smem(const Problem& P, int lpb, int len) {
@@ -2126,7 +2132,7 @@ static void orthonormalize(const Problem& P, const PhaseBufs& B, cudaStream_t st
   const int sp = a.spatial;
   double* W = sp ? B.Hw : B.Hwa;
   int nch = gram_partials(P, B, st, sp, a.A, a.lda, a.acols, B.cexp);
-  launch_geig(a, B.part, B.cexp, nch, B.sm, SM_QM, B.keep, st);
+  launch_geig(a, B.part, B.cexp, nch, 0, B.sm, SM_QM, B.keep, st);
   // U1 = A M; its Gram from the same tiles when their partials fit the buffer (one partial
   // per 32-row tile, counted from each subdomain's first row), else by k_gram
   const int ntile = ((sp ? P.maxN : P.g.n) + TALL_ROWS - 1) / TALL_ROWS;
@@ -2134,7 +2140,7 @@ static void orthonormalize(const Problem& P, const PhaseBufs& B, cudaStream_t st
   tall(P, B, st, sp, a.A, a.lda, a.acols, 0, nullptr, SM_QM, B.keep, 0, W, P.WC,
        fuse ? B.part : nullptr);
   nch = fuse ? ntile : gram_partials(P, B, st, sp, W, P.WC, B.keep, nullptr);
-  launch_chol_inv(a, B.part, nch, B.sm, SM_R1I, B.keep, st);
+  launch_chol_inv(a, B.part, nch, 0, B.sm, SM_R1I, B.keep, st);
   tall(P, B, st, sp, W, P.WC, B.keep, 0, nullptr, SM_R1I, B.keep, 0, a.Q, a.ldq);
   if (a.mode == ORTH_QR || (!sp && a.mode == ORTH_AUG)) {
     // mutually orthogonal candidates (the cosines; the angular table): coefficient-space
@@ -2210,7 +2216,7 @@ void advection_phase(const Problem& P, const PhaseBufs& B, int axis, cudaStream_
   }
   // 3. S M products, eigen-split of C
   pbeg(st, KS_SMALL_ADV1);
-  k_small_adv1<<<nsub, DD_THREADS, small_adv1_smem(RC), st>>>(P, B, axis);
+  k_small_adv1<<<dim3(nsub, 2), small_threads(RC), small_adv1_smem(RC), st>>>(P, B, axis);
   pend(st);
   // 4. K^0 = X (S <V, Vh>)
   galerkin_tall(P, B, st, 1, B.X, RC, B.r, nullptr, SM_B, B.rt, B.K, RC);
@@ -2353,8 +2359,7 @@ void advection_phase(const Problem& P, const PhaseBufs& B, int axis, cudaStream_
   gram(P, B, st, 0, B.V1, RC, B.rt, 0, B.L, RC, B.rt, 0, 1, nullptr, SM_S3T);
   // 11. truncation (Algorithm 5)
   pbeg(st, KS_TRUNC);
-  k_trunc<<<nsub, DD_THREADS, trunc_smem(RC), st>>>(
-      P, B);
+  k_trunc<<<nsub, small_threads(RC), trunc_smem(RC), st>>>(P, B);
   pend(st);
   galerkin_tall(P, B, st, 1, B.X1, RC, B.rt, nullptr, SM_UB, B.ro, B.Xo, RC);
   galerkin_tall(P, B, st, 0, B.V1, RC, B.rt, nullptr, SM_VB, B.ro, B.Vo, RC);
@@ -2489,7 +2494,7 @@ void mass_fix_phase(const Problem& P, const PhaseBufs& B, cudaStream_t st) {
   cudaMemcpyAsync(B.rt, B.m, sizeof(int) * nsub, cudaMemcpyDeviceToDevice, st);
   pend(st);
   pbeg(st, KS_TRUNC);
-  k_trunc<<<nsub, DD_THREADS, trunc_smem(RC), st>>>(P, B);
+  k_trunc<<<nsub, small_threads(RC), trunc_smem(RC), st>>>(P, B);
   pend(st);
   tall(P, B, st, 1, B.K, RC, B.rt, 0, nullptr, SM_UB, B.ro, 0, B.Xo, RC);
   tall(P, B, st, 0, B.V1, RC, B.rt, 0, nullptr, SM_VB, B.ro, 0, B.Vo, RC);
