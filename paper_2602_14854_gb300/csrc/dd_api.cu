@@ -415,8 +415,9 @@ static dd_status create_impl(int ninst, const dd_grid* grids, const dd_tiling* t
   // augmentation input width both fit
   h->RC = std::max(raug_max, h->MC);
   // the tensor-core forms stage rows with TMA, which needs rows on 16-byte boundaries
-  if (opt->precision == DD_TF32 || opt->precision == DD_BF16 || opt->products != DD_PRODUCTS_FP64)
-    h->RC += h->RC & 1;
+  const bool even = opt->precision == DD_TF32 || opt->precision == DD_BF16 ||
+                    opt->products != DD_PRODUCTS_FP64;
+  if (even) h->RC += h->RC & 1;
   h->r_floor = opt->rank_mode == DD_RANK_FIXED ? opt->rank : opt->r_min;
   auto bail = [&](dd_status s, const std::string& m) {
     free_all(h);
@@ -424,6 +425,7 @@ static dd_status create_impl(int ninst, const dd_grid* grids, const dd_tiling* t
     return fail(s, m);
   };
   if (h->n < h->MC) return bail(DD_ERR_ARG, "need at least 3 * stored-rank cap directions");
+  if (even) h->MC += h->MC & 1;      // the augmentation input's rows likewise (MC <= RC still)
 
   // geometry, instance after instance
   int rowoff = 0, fbase = 0;
@@ -655,7 +657,7 @@ static dd_status create_impl(int ninst, const dd_grid* grids, const dd_tiling* t
   ok &= dalloc(&h->d_keep, nsub) == cudaSuccess;
   ok &= dalloc(&h->d_kcn, nsub) == cudaSuccess;
   ok &= dalloc(&h->d_kcur, nsub) == cudaSuccess;
-  ok &= dalloc(&h->d_cexp, (long)nsub * 16) == cudaSuccess;
+  ok &= dalloc(&h->d_cexp, (long)nsub * dd::GRAM_CHUNKS) == cudaSuccess;
   ok &= dalloc(&h->d_dm, Nt) == cudaSuccess;
   ok &= dalloc(&h->d_mvec, (long)nsub * RC) == cudaSuccess;
   ok &= dalloc(&h->d_status, 1) == cudaSuccess;
@@ -702,14 +704,38 @@ static dd_status create_impl(int ninst, const dd_grid* grids, const dd_tiling* t
   P.nchunk_ang = std::max(1, std::min(16, n / 64));
   P.ochunk_sp = P.nchunk_sp;
   P.ochunk_ang = P.nchunk_ang;
+  // rows per item of the tensor-core products: 256 (one read-out) unless that makes more than
+  // about four items per SM, or more than GRAM_CHUNKS chunks of a subdomain (half as many in
+  // angle, where a step has twice the products: the partials' memory)
+  auto crows = [&](long rows, long largest, int most) {
+    const long r = std::max(std::max(1L, std::min(16L, rows / (1024L * P.nsm))),
+                            (largest + 256L * most - 1) / (256L * most));
+    return 256 * (int)r;
+  };
+  P.crows_sp = crows(Nt, h->maxN, dd::GRAM_CHUNKS);
+  P.crows_ang = crows((long)nsub * n, n, dd::GRAM_CHUNKS / 2);
+  P.ocrows_sp = P.crows_sp;
+  P.ocrows_ang = P.crows_ang;
   if (dalloc(&h->d_part, dd::part_elems(P)) != cudaSuccess)
     return bail(DD_ERR_CUDA, "device allocation failed");
   if (dd::orth_init() != cudaSuccess || dd::phase_init() != cudaSuccess)
     return bail(DD_ERR_CUDA, "kernel attribute setup failed");
   if (opt->products == DD_PRODUCTS_AUTO) {      // the heuristic; the autotuner may revise it
+    // Per row family.  Tall products: two 128-row tiles per SM, or rows x r_cap^2 past 5.5e7 (the FP64
+    // pipe does 2 FMA per clock and SM; the tensor form costs 15 us at least).  16 x 1024
+    // cells and 16 x 512 directions: r_cap = 30, 19.4 against 18.1 us per product and a step 2.24
+    // against 2.59 ms (the Gram of an orthonormalisation comes with the FP64 product); r_cap = 60,
+    // 48.6 against 24.8 us, 6.55 against 5.93 ms; 50, but with ranks well below it, 2.33 against 2.50.
     const long tiles_sp = (long)nsub * ((h->maxN + 127) / 128), tiles_ang = (long)nsub * ((n + 127) / 128);
-    P.oz_sp = tiles_sp >= 2L * P.nsm;
-    P.oz_ang = tiles_ang >= 2L * P.nsm;
+    const long rc2 = (long)RC * RC;
+    P.oz_sp = tiles_sp >= 2L * P.nsm || Nt * rc2 >= 55000000L;
+    P.oz_ang = tiles_ang >= 2L * P.nsm || (long)nsub * n * rc2 >= 55000000L;
+    // Tall-skinny products likewise, and where the FP64 kernels' chunks (at most 16 of a subdomain)
+    // come to 2e5 row x r_cap^2 each: 4 x 4096 cells, r_cap = 30 (256 rows a chunk): spatial
+    // coefficients 104 us against 34 on the tensor cores, a Gram 26 against 33; 16384 cells (1024
+    // rows): 253 and 81 against 31; below it, at 64 rows a chunk, 42 and 17 against 36.
+    P.ozg_sp = P.oz_sp || h->maxN / P.nchunk_sp * rc2 >= 200000L;
+    P.ozg_ang = P.oz_ang || n / P.nchunk_ang * rc2 >= 200000L;
   }
   if ((P.prec >= dd::PREC_TF32 || opt->products != DD_PRODUCTS_FP64) && dd::tc_init() != cudaSuccess)
     return bail(DD_ERR_CUDA, "tensor-core setup failed (tensor-map encoder or kernel attributes)");
@@ -952,8 +978,8 @@ dd_status dd_dlra_tuning(dd_dlra_t h, int* choice, double* ms) {
   if (choice) {
     choice[0] = h->P.oz_sp;
     choice[1] = h->P.oz_ang;
-    choice[2] = h->P.ochunk_sp;
-    choice[3] = h->P.ochunk_ang;
+    choice[2] = h->P.ozg_sp ? (h->maxN + h->P.ocrows_sp - 1) / h->P.ocrows_sp : h->P.ochunk_sp;
+    choice[3] = h->P.ozg_ang ? (h->n + h->P.ocrows_ang - 1) / h->P.ocrows_ang : h->P.ochunk_ang;
     choice[4] = h->P.ozg_sp;
     choice[5] = h->P.ozg_ang;
   }

@@ -97,12 +97,15 @@ struct PhaseBufs {
   int* keep;       // per subdomain: significant columns kept by the orthonormalisation
   int* kcn;        // per subdomain: candidates accepted by the coefficient-space completion
   int* kcur;       // per subdomain: columns done before the sequential completion
-  int* cexp;       // per subdomain and row chunk: power-of-two exponent of a scaled Gram
+  int* cexp;       // per subdomain and row chunk (GRAM_CHUNKS of them): power-of-two exponent of a scaled Gram
   double* dm;      // per cell: scalar-flux change of the non-conservative parts (mass fix)
   double* mvec;    // per subdomain: RC-vector scratch of the mass bookkeeping
   unsigned* status;
 };
 
+// Most row chunks of a subdomain in an orthonormalisation's Gram (their exponents: cexp) and in the
+// tensor-core products, whose partials are kept for the largest subdomain's chunks everywhere
+constexpr int GRAM_CHUNKS = 64;
 // indices of small matrices inside a subdomain's block of NSMALL matrices
 enum Small {
   SM_C = 0, SM_MOUT_LO, SM_MOUT_HI, SM_M, SM_MIN_LO, SM_MIN_HI,   // angular Galerkin coefficients
@@ -146,6 +149,8 @@ struct Problem {
   const double* sptab; const long long* spoff; const int* spnf;
   int nchunk_sp, nchunk_ang;   // chunks of the two-stage reductions
   int ochunk_sp, ochunk_ang;   // chunks of the orthonormalisations' Grams (<= nchunk_*)
+  int crows_sp, crows_ang;     // rows per chunk of the tensor-core products
+  int ocrows_sp, ocrows_ang;   // and of the orthonormalisations' Grams there (>= crows_*)
   int nsm;                     // streaming multiprocessors of the device
   long Ntot;                   // spatial rows of all subdomains
 };
@@ -198,10 +203,36 @@ bool oz_tall(const Problem& P, unsigned* status, cudaStream_t st, int spatial, c
              int lda, const int* ninner, int ninner_fix, const double* Bm, int bsmall,
              const double* smbase, const int* ncols, int ncols_fix, double* Y, int ldy,
              int mtrans = 0, int accumulate = 0, const double* rowscale = nullptr);
-// The chunk partials of the symmetric Gram A^T A (the layout and chunk exponents of k_gram)
-// FP64-accurate on the BF16 tensor cores; false when the capacity does not fit.
-bool oz_gram(const Problem& P, unsigned* status, cudaStream_t st, int spatial, const double* A,
-             int lda, const int* acnt, double* part, int nchunk, int* cexp);
+// ---- tall-skinny products on the tensor cores, FP64-accurate (dd_tc.cu, k_oz_gram) --------
+enum OzRows { OG_CELLS = 0, OG_DIRS, OG_FACE_LO, OG_FACE_HI };   // face lines: A's rows are the
+                                 // face cells of B.X1's layout, B's the ghost rows of that side
+struct OzProd {
+  const double* A; int lda; const int* acnt; int afix;
+  const double* B; int ldb; const int* bcnt; int bfix;   // null: B = A (weights on one side)
+  int rows;                      // OzRows
+  int aside;                     // -1: own rows; 0 / 1: A holds the low / high neighbour's
+                                 // direction rows (absent: its physical inflow, or nothing)
+  int shift;                     // B's row is A's row one cell earlier along the axis (B = A's array)
+  int wsel; const double* wrow;  // weights of B's rows (GramWeight)
+  int blk;                       // partial block written
+};
+#define OG_PROD 8
+struct OzGram {
+  Geo g;
+  int axis, nprod;
+  OzProd p[OG_PROD];
+  double* part; int nchunk, nblk;   // partial of (subdomain k, chunk c, block b) at (k nchunk + c) nblk + b
+  int crows;                        // rows per chunk
+  int* cexp;                        // chunk exponents (one symmetric product), or null
+  const double* ox; const double* oy;
+  const int* infl_on; const double* infl_hw;
+  int maxlines;
+  unsigned* status;
+};
+struct OzDst { int idx[OG_PROD]; };
+// Launches the products; with dst, their reduction into the small slots dst->idx[blk] too.
+// False when the capacity does not fit (nothing launched).
+bool oz_gram(const Problem& P, cudaStream_t st, OzGram& a, const OzDst* dst, double* sm);
 void advection_phase(const Problem& P, const PhaseBufs& B, int axis, cudaStream_t st);
 void collision_phase(const Problem& P, const PhaseBufs& B, cudaStream_t st);
 void mass_fix_phase(const Problem& P, const PhaseBufs& B, cudaStream_t st);

@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(512, 1) k_geig(OrthArgs a, const double* part,
   int* perm = reinterpret_cast<int*>(nrm + RC);
   // the chunk partials are Grams of 2^-e_c A: G1 of 2^-emax A is their sum with
   // weights 4^(e_c - emax)
-  __shared__ double fac[64];
+  __shared__ double fac[GRAM_CHUNKS];
   __shared__ int s_keep;
   int emax = INT_MIN;
   bool scaled = false;

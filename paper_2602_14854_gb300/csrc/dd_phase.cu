@@ -448,6 +448,8 @@ struct TallArgs {
   const double* Bm; int bsmall;     // small matrix index inside the subdomain block (or -1: Bm is per-k RC*RC stride)
   const int* ncols; int ncols_fix;
   double* Y; int ldy;
+  int mtrans;                       // M read transposed (Y = A M^T)
+  int accumulate;                   // Y += A M on the columns < ncols only
   // optional: the Gram Y^T Y of each row tile (nc x nc, RC x RC stride) to
   // gpart[k * gridDim.x + tile], the chunk partials of the next orthonormalisation step
   double* gpart;
@@ -483,7 +485,15 @@ __global__ void __launch_bounds__(DD_THREADS) k_tall(Geo g, TallArgs a, double* 
   double* Ms = sh;                                  // RC x RC (+4 so a tile never reads past it)
   double* As = Ms + RC * RC + 4;                    // TALL_ROWS x SA
   double* Ys = As + TALL_ROWS * (RC | 1);           // TALL_ROWS x SY
-  for (int e = tid; e < RC * RC + 4; e += DD_THREADS) Ms[e] = e < ni * RC ? Bk[e] : 0.0;
+  if (a.mtrans) {
+    for (int e = tid; e < RC * RC; e += DD_THREADS) {
+      const int j = e / RC, l = e - j * RC;
+      Ms[l * RC + j] = l < ni ? Bk[e] : 0.0;
+    }
+    if (tid < 4) Ms[RC * RC + tid] = 0.0;
+  } else {
+    for (int e = tid; e < RC * RC + 4; e += DD_THREADS) Ms[e] = e < ni * RC ? Bk[e] : 0.0;
+  }
   for (int r = warp; r < nrow; r += DD_THREADS / 32)
     for (int l = lane; l < ni; l += 32) As[r * SA + l] = a.A[(rb + r0 + r) * a.lda + l];
   __syncthreads();
@@ -508,8 +518,14 @@ __global__ void __launch_bounds__(DD_THREADS) k_tall(Geo g, TallArgs a, double* 
     }
   }
   __syncthreads();
-  for (int r = warp; r < nrow; r += DD_THREADS / 32)
-    for (int j = lane; j < a.ldy; j += 32) a.Y[(rb + r0 + r) * a.ldy + j] = Ys[r * SY + j];
+  for (int r = warp; r < nrow; r += DD_THREADS / 32) {
+    double* yr = a.Y + (rb + r0 + r) * a.ldy;
+    if (a.accumulate) {
+      for (int j = lane; j < nc; j += 32) yr[j] += Ys[r * SY + j];
+    } else {
+      for (int j = lane; j < a.ldy; j += 32) yr[j] = Ys[r * SY + j];
+    }
+  }
   if (gp) {
     // the tile's Gram, pairs (i <= j) enumerated densely, rows in order
     const int npair = nc * (nc + 1) / 2;
@@ -570,13 +586,11 @@ __global__ void __launch_bounds__(DD_THREADS) k_ghost(Problem P, PhaseBufs B, in
 // K-step of the advection (Appendix A), all RK stages fused; a CTA owns whole lines
 // ---------------------------------------------------------------------------
 #define KS_EPT 24    // entries per thread of k_kstep_adv (lines x cells x r_t <= 256 x 24)
-#define KE_EPT 16    // entries per thread of k_kstep_eig (<= 256 x 16)
+// The matrix stencil with C+ and C-, for the flux-split form (no eigenbasis there).
 // TC: arithmetic type (double for the FP64 path, float for the mixed path); the
-// factors stay FP64 in memory.  big_only: only the subdomains whose line does not fit
-// k_kstep_eig's tile (len r_t > 256 KE_EPT; that kernel skips them).
+// factors stay FP64 in memory.
 template <typename TC>
-__global__ void __launch_bounds__(DD_THREADS) k_kstep_adv(Problem P, PhaseBufs B, int axis, int lpb,
-                                                          int big_only) {
+__global__ void __launch_bounds__(DD_THREADS) k_kstep_adv(Problem P, PhaseBufs B, int axis, int lpb) {
   extern __shared__ double sh_raw[];
   TC* sh = reinterpret_cast<TC*>(sh_raw);
   const int k = blockIdx.y, RC = P.g.RC;
@@ -586,7 +600,6 @@ __global__ void __launch_bounds__(DD_THREADS) k_kstep_adv(Problem P, PhaseBufs B
   const int nl = min(lpb, L.nlines - l0);
   const int rt = B.rt[k];
   const int len = L.len;
-  if (big_only && (long)len * rt <= (long)DD_THREADS * KE_EPT) return;
   count_work(P.g, KS_KSTEP_ADV, (double)nl * len * rt * (6.0 * rt + 4.0) * (P.integrator == 1 ? 4 : 1));
   TC* Cp = sh;
   TC* Cn = Cp + RC * RC;
@@ -664,200 +677,67 @@ __global__ void __launch_bounds__(DD_THREADS) k_kstep_adv(Problem P, PhaseBufs B
   }
 }
 
-// K-step of the advection in the eigenbasis of C, where Appendix A's upwinding acts
-// column by column: with K~ = K P (ghost rows likewise) each RK stage is
-//   R~_ij = coef (lambda+_j (K~_ij - K~_(i-1)j) + lambda-_j (K~_(i+1)j - K~_ij)),
-// O(1) per entry instead of the 3 r_t products of the matrix stencil; the increment
-// dt sum_s b_s R~_s is rotated back with P^T and added to the FP64 state.  P and lambda
-// come from k_small_adv1 (small slots S3T and VB, free until the S-step).  Same lines-
-// per-CTA layout as k_kstep_adv; the entry indices are decoded once.
-// The explicit-Euler K-step in the eigenbasis, the stencil alone: on K~ = K P (in X1, formed
-// by a tall product) along the lines of the sweep, with the ghosts K^b P at the line ends,
-// the increment dt coef (lambda+_j (K~_c - K~_p) + lambda-_j (K~_n - K~_c)) of column j
-// (Appendix A's per-eigenvector upwinding) into Hw (zero in the columns from r_t; rotated
-// back and added to K by the next tall product).  One line per CTA: warp w takes the
-// columns 32 (w % 2) .. + 31 of the line's segment w / 2 (of KE1_SEGS), each thread walking
-// its column along the segment with the previous and current entries in registers.  The
-// one-stage form of k_kstep_eig's stencil, expanded into one coefficient per neighbour.
-#define KE1_SEGS 4
-static_assert(DD_THREADS == 64 * KE1_SEGS, "k_kstep_eig1: two warps per segment");
-__global__ void __launch_bounds__(DD_THREADS) k_kstep_eig1(Problem P, PhaseBufs B, int axis) {
-  __shared__ double gh[2][DD_MAXC];
-  const int k = blockIdx.y, RC = P.g.RC, line = blockIdx.x;
+// K-step of the advection in the eigenbasis of C, where Appendix A's upwinding acts column by
+// column: with K~ = K P (in X1, formed by a tall product) and the ghosts K^b P at the line
+// ends, the RK increment of
+//   dK~_ij/dt = coef (lambda+_j (K~_ij - K~_(i-1)j) + lambda-_j (K~_(i+1)j - K~_ij))
+// into Hw (rotated back with P^T and added to K by the next tall product).  A column has one
+// upwind side, so a thread walks one column of one line segment downwind and carries the
+// stage values of the cell behind it in registers: nothing is staged, a line may have any
+// length, and an entry costs 15 FP64 operations (RK4; 2 with Euler).  Stage s of a cell needs
+// stage s - 1 of the cell behind, so a segment that does not start at the line's end begins
+// three cells early (RK4).  seg: cells per segment (lines are cut where there are too few of
+// them to fill the GPU).  P and lambda come from k_small_adv1 (small slots S3T and VB, free
+// until the S-step).  Bound by the FP64 pipe: 512 lines x 32 cells x 20 columns, RK4, 115 us
+// with the stages in shared memory and both basis changes in the same kernel, 9 now (and two
+// products of 12 each).
+__global__ void __launch_bounds__(DD_THREADS) k_kstep_line(Problem P, PhaseBufs B, int axis, int seg) {
+  const int k = blockIdx.y, RC = P.g.RC, rt = B.rt[k];
   const Lines L = lines_of(P.g, k, axis);
-  if (line >= L.nlines) return;
-  const int len = L.len, rt = B.rt[k];
-  count_work(P.g, KS_KSTEP_ADV, (double)len * rt * 8.0);
-  const double* Pg = SMB(B, P, k, SM_S3T);
-  const double* lam = SMB(B, P, k, SM_VB);
-  for (int e = threadIdx.x; e < 2 * rt; e += blockDim.x) {     // ghosts in the eigenbasis
-    const int side = e >= rt, j = e - side * rt;
-    const double* kb = B.Kb + (((long)k * 2 + side) * P.maxlines + line) * RC;
-    double x = 0.0;
-    for (int u = 0; u < rt; ++u) x += kb[u] * Pg[u * RC + j];
-    gh[side][j] = x;
+  const int len = L.len, nseg = (len + seg - 1) / seg;
+  const int e = blockIdx.x * DD_THREADS + threadIdx.x, tot = L.nlines * nseg * rt;
+  const bool rk4 = P.integrator == 1;
+  if (blockIdx.x == 0) count_work(P.g, KS_KSTEP_ADV, (double)L.nlines * len * rt * (rk4 ? 32.0 : 8.0));
+  if (e >= tot) return;
+  const int j = e % rt, u = e / rt, line = u % L.nlines, t0 = (u / L.nlines) * seg;
+  const int t1 = min(len, t0 + seg);
+  const double lam = SMB(B, P, k, SM_VB)[j];
+  const bool up = lam >= 0.0;                        // downwind = ascending positions
+  const long step = (up ? 1 : -1) * (long)L.stride_pos * RC;
+  const long base = ((long)P.g.rowoff[k] + cell_of(L, line, up ? 0 : len - 1)) * RC + j;
+  const double* x = B.X1 + base;
+  double* out = B.Hw + base;
+  const double b = -P.g.dtk[k] * P.c_adv / (axis == 0 ? P.g.hxk[k] : P.g.hyk[k]) * fabs(lam);
+  int t = rk4 ? t0 - 3 : t0;
+  double kp;                                         // the cell behind t
+  if (t <= 0) {
+    t = 0;
+    const double* kb = B.Kb + (((long)k * 2 + (up ? 0 : 1)) * P.maxlines + line) * RC;
+    const double* Pj = SMB(B, P, k, SM_S3T) + j;
+    kp = 0.0;
+    for (int i = 0; i < rt; ++i) kp += kb[i] * Pj[i * RC];
+  } else {
+    kp = x[(t - 1) * step];
   }
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, j = (warp & 1) * 32 + (threadIdx.x & 31);
-  const int sl = (len + KE1_SEGS - 1) / KE1_SEGS, p0 = (warp >> 1) * sl, p1 = min(len, p0 + sl);
-  if (j >= RC || p0 >= p1) return;
-  const double coef = -P.c_adv / (axis == 0 ? P.g.hxk[k] : P.g.hyk[k]);
-  const double dt = P.g.dtk[k];
-  const long base = ((long)P.g.rowoff[k] + cell_of(L, line, 0)) * RC + j;
-  const long step = (long)L.stride_pos * RC;
-  if (j >= rt) {                                 // whole rows: the product reads pairs of columns
-    for (int pos = p0; pos < p1; ++pos) B.Hw[base + pos * step] = 0.0;
-    return;
-  }
-  // inc = cc kc + cp kp + cn kn with the column's coefficients (three FP64 operations per
-  // entry: the kernel is bound by the FP64 pipe, whose warp instructions cost the same
-  // however many lanes are active)
-  const double l = lam[j], lp = l > 0.0 ? l : 0.0, ln = l < 0.0 ? l : 0.0;
-  const double cpk = -dt * coef * lp, cnk = dt * coef * ln, cck = dt * coef * (lp - ln);
-  double kp = p0 > 0 ? B.X1[base + (p0 - 1) * step] : gh[0][j], kc = B.X1[base + p0 * step];
+  if (!rk4) {
 #pragma unroll 4
-  for (int pos = p0; pos < p1; ++pos) {
-    const double kn = pos < len - 1 ? B.X1[base + (pos + 1) * step] : gh[1][j];
-    B.Hw[base + pos * step] = fma(cnk, kn, fma(cpk, kp, cck * kc));
-    kp = kc;
-    kc = kn;
-  }
-}
-
-template <typename TC>
-__global__ void __launch_bounds__(DD_THREADS) k_kstep_eig(Problem P, PhaseBufs B, int axis, int lpb,
-                                                      int ebasis) {
-  extern __shared__ double sh_raw[];
-  TC* sh = reinterpret_cast<TC*>(sh_raw);
-  const int k = blockIdx.y, RC = P.g.RC;
-  const Lines L = lines_of(P.g, k, axis);
-  const int l0 = blockIdx.x * lpb;
-  if (l0 >= L.nlines) return;
-  const int nl = min(lpb, L.nlines - l0);
-  const int rt = B.rt[k];
-  const int len = L.len;
-  // a tile larger than the register tile (only with lpb = 1: a line longer than
-  // 256 KE_EPT / r_t) is left to k_kstep_adv, launched after this kernel for exactly these
-  if ((long)nl * len * rt > (long)DD_THREADS * KE_EPT) return;
-  count_work(P.g, KS_KSTEP_ADV,
-             (double)nl * len * rt * ((ebasis ? 0.0 : 4.0 * rt) + 8.0 * (P.integrator == 1 ? 4 : 1)));
-  // ebasis: K~ = K P was formed outside (in X1, by the tall products); the stages run on it
-  // and the increment dt sum_s b_s R~_s is written back there (rotated back and added to K
-  // outside)
-  const double* Ksrc = ebasis ? B.X1 : B.K;
-  TC* Pm = sh;                     // Pm[u * RC + j]: component u of eigenvector j
-  TC* lp = Pm + RC * RC;           // max(lambda, 0)
-  TC* ln = lp + RC;                // min(lambda, 0)
-  TC* Glo = ln + RC;               // lpb x RC ghost rows in the eigenbasis
-  TC* Ghi = Glo + lpb * RC;
-  TC* Kst = Ghi + lpb * RC;        // lpb x len x rt
-  const double* Pg = SMB(B, P, k, SM_S3T);
-  const double* lam = SMB(B, P, k, SM_VB);
-  for (int e = threadIdx.x; e < RC * RC; e += blockDim.x) Pm[e] = (TC)Pg[e];
-  for (int j = threadIdx.x; j < RC; j += blockDim.x) {
-    const double l = j < rt ? lam[j] : 0.0;
-    lp[j] = (TC)(l > 0.0 ? l : 0.0);
-    ln[j] = (TC)(l < 0.0 ? l : 0.0);
-  }
-  const int tot = nl * len * rt;
-  int code[KE_EPT];                // li << 20 | pos << 8 | t (li < 2^11, pos < 2^12, t < 2^8)
-#pragma unroll
-  for (int i = 0; i < KE_EPT; ++i) {
-    const int e = threadIdx.x + i * blockDim.x;
-    code[i] = 0;
-    if (e < tot) {
-      const int li = e / (len * rt), pos = (e / rt) % len, t = e % rt;
-      code[i] = (li << 20) | (pos << 8) | t;
-      Kst[e] = (TC)Ksrc[((long)P.g.rowoff[k] + cell_of(L, l0 + li, pos)) * RC + t];
-    }
-  }
-  __syncthreads();
-  // ghosts and K into the eigenbasis
-  for (int e = threadIdx.x; e < 2 * nl * rt; e += blockDim.x) {
-    const int side = e >= nl * rt, r = e - side * nl * rt, li = r / rt, j = r - li * rt;
-    const double* kb = B.Kb + (((long)k * 2 + side) * P.maxlines + l0 + li) * RC;
-    TC x = 0;
-    for (int u = 0; u < rt; ++u) x += (TC)kb[u] * Pm[u * RC + j];
-    (side ? Ghi : Glo)[li * RC + j] = x;
-  }
-  TC k0[KE_EPT], acc[KE_EPT];
-#pragma unroll
-  for (int i = 0; i < KE_EPT; ++i) {
-    const int e = threadIdx.x + i * blockDim.x;
-    k0[i] = 0; acc[i] = 0;
-    if (e < tot) {
-      if (ebasis) {
-        k0[i] = Kst[e];
-      } else {
-        const int t = code[i] & 255, rowe = e - t;   // entry of column 0 of this cell
-        TC x = 0;
-        for (int u = 0; u < rt; ++u) x += Kst[rowe + u] * Pm[u * RC + t];
-        k0[i] = x;
-      }
-    }
-  }
-  __syncthreads();
-  if (!ebasis) {
-#pragma unroll
-    for (int i = 0; i < KE_EPT; ++i) {
-      const int e = threadIdx.x + i * blockDim.x;
-      if (e < tot) Kst[e] = k0[i];
-    }
-  }
-  __syncthreads();
-  const TC coef = (TC)(-P.c_adv / (axis == 0 ? P.g.hxk[k] : P.g.hyk[k]));
-  const TC dt = (TC)P.g.dtk[k];
-  const int nst = P.integrator == 1 ? 4 : 1;
-  for (int s = 0; s < nst; ++s) {
-    TC kv[KE_EPT];
-  #pragma unroll
-  for (int i = 0; i < KE_EPT; ++i) {
-      const int e = threadIdx.x + i * blockDim.x;
-      kv[i] = 0;
-      if (e < tot) {
-        const int li = code[i] >> 20, pos = (code[i] >> 8) & 4095, j = code[i] & 255;
-        const TC kc = Kst[e];
-        const TC kp = pos > 0 ? Kst[e - rt] : Glo[li * RC + j];
-        const TC kn = pos < len - 1 ? Kst[e + rt] : Ghi[li * RC + j];
-        kv[i] = coef * (lp[j] * (kc - kp) + ln[j] * (kn - kc));
-      }
-    }
-    __syncthreads();
-    const TC bs = (TC)((nst == 4) ? c_rk_b[s] : 1.0);
-    const TC an = (TC)((s + 1 < nst) ? c_rk_a[s + 1] : 0.0);
-  #pragma unroll
-  for (int i = 0; i < KE_EPT; ++i) {
-      const int e = threadIdx.x + i * blockDim.x;
-      if (e < tot) {
-        acc[i] += bs * kv[i];
-        Kst[e] = (s + 1 < nst) ? k0[i] + an * dt * kv[i] : acc[i];
-      }
-    }
-    __syncthreads();
-  }
-  if (ebasis) {                     // the increment dt acc~, in the eigenbasis
-#pragma unroll
-    for (int i = 0; i < KE_EPT; ++i) {
-      const int e = threadIdx.x + i * blockDim.x;
-      if (e < tot) {
-        const int li = code[i] >> 20, pos = (code[i] >> 8) & 4095, t = code[i] & 255;
-        B.X1[((long)P.g.rowoff[k] + cell_of(L, l0 + li, pos)) * RC + t] = (double)(dt * Kst[e]);
-      }
+    for (; t < t1; ++t) {
+      const double kc = x[t * step];
+      out[t * step] = b * (kc - kp);
+      kp = kc;
     }
     return;
   }
-  // back to the original basis: increment_t = dt sum_j acc~_j P_tj, added in FP64
-#pragma unroll
-  for (int i = 0; i < KE_EPT; ++i) {
-    const int e = threadIdx.x + i * blockDim.x;
-    if (e < tot) {
-      const int li = code[i] >> 20, pos = (code[i] >> 8) & 4095, t = code[i] & 255;
-      const int rowe = e - t;
-      TC x = 0;
-      for (int j = 0; j < rt; ++j) x += Kst[rowe + j] * Pm[t * RC + j];
-      double* Ke = B.K + ((long)P.g.rowoff[k] + cell_of(L, l0 + li, pos)) * RC + t;
-      *Ke = *Ke + (double)(dt * x);
-    }
+  double p1 = kp, p2 = kp, p3 = kp;                  // stage values of the cell behind
+#pragma unroll 4
+  for (; t < t1; ++t) {
+    const double kc = x[t * step];
+    const double d1 = b * (kc - kp), y1 = fma(0.5, d1, kc);
+    const double d2 = b * (y1 - p1), y2 = fma(0.5, d2, kc);
+    const double d3 = b * (y2 - p2), y3 = kc + d3;
+    const double d4 = b * (y3 - p3);
+    if (t >= t0) out[t * step] = fma(2.0, d2 + d3, d1 + d4) * (1.0 / 6.0);
+    kp = kc; p1 = y1; p2 = y2; p3 = y3;
   }
 }
 
@@ -1759,18 +1639,12 @@ size_t kstep_smem(const Problem& P, int lpb, int len) {
   return sizeof(double) * (3 * RC * RC + 2 * lpb * RC + (size_t)lpb * len * RC);
 }
 
-size_t kstep_eig_smem(const Problem& P, int lpb, int len) {
-  const int RC = P.g.RC;
-  return sizeof(double) * ((size_t)RC * RC + 2 * RC + 2 * lpb * RC + (size_t)lpb * len * RC);
-}
-
-int kstep_eig_lpb(const Problem& P, int len) {
-  const int RC = P.g.RC;
-  int lpb = max(1, (DD_THREADS * KE_EPT) / (len * RC));
-  while (lpb > 1 && kstep_eig_smem(P, lpb, len) > 200 * 1024) --lpb;
-  const long lines = (long)P.maxlines * P.g.nsub;
-  while (lpb > 1 && (lines + lpb - 1) / lpb < 2L * P.nsm) --lpb;
-  return lpb;
+// cells per segment of k_kstep_line: whole lines, unless they are fewer than two warps per
+// scheduler of every SM; then segments of at least 16 cells
+int kstep_seg(const Problem& P) {
+  const long threads = (long)P.maxlines * P.g.nsub * std::max(1, P.g.RC / 2);
+  const int cut = (int)std::max(1L, (256L * P.nsm + threads - 1) / threads);
+  return std::max(16, (P.maxlines + cut - 1) / cut);
 }
 
 int kstep_lpb(const Problem& P, int len) {
@@ -1795,9 +1669,17 @@ const char* const kSlotNames[NSLOT] = {
     "k_kc_apply", "k_tc_tall", "k_tc_gram", "k_lstep_prod", "k_oz_tall", "k_oz_gram"};
 thread_local Prof* g_prof = nullptr;
 
+// chunks of the largest subdomain's spatial rows (of the direction rows) in the tensor-core
+// products
+static int oz_chunks(const Problem& P, int spatial) {
+  return spatial ? (P.maxN + P.crows_sp - 1) / P.crows_sp : (P.g.n + P.crows_ang - 1) / P.crows_ang;
+}
+
 size_t part_elems(const Problem& P) {
   const int nc = P.nchunk_sp > P.nchunk_ang ? P.nchunk_sp : P.nchunk_ang;
-  const size_t grams = (size_t)P.g.nsub * nc * 8 * P.g.RC * P.g.RC;
+  const size_t fp64 = (size_t)P.g.nsub * nc * 8 * P.g.RC * P.g.RC;
+  const size_t oz = (size_t)P.g.nsub * std::max(4 * oz_chunks(P, 1), 8 * oz_chunks(P, 0)) * P.g.RC * P.g.RC;
+  const size_t grams = std::max(fp64, oz);
   const size_t kc = (size_t)P.g.nsub * kc_region(P.g.RC);   // the spatial completion's scratch
   return grams > kc ? grams : kc;
 }
@@ -1810,8 +1692,6 @@ cudaError_t phase_init() {
   e = cudaFuncSetAttribute(k_kstep_adv<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_kstep_adv<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_kstep_eig<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_sstep_adv, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)sstep_smem(RC));
@@ -1853,9 +1733,39 @@ static dim3 reduce_grid(const Geo& g, int nblk) {
   return dim3((nblk * g.RC * g.RC + DD_THREADS - 1) / DD_THREADS, g.nsub);
 }
 
+// ---- tall-skinny products on the tensor cores (k_oz_gram) --------------------------------
+static OzGram oz_products(const Problem& P, const PhaseBufs& B, int spatial, int axis, int nblk) {
+  OzGram a{};
+  a.axis = axis; a.nprod = 0; a.nblk = nblk;
+  a.part = B.part; a.nchunk = oz_chunks(P, spatial);
+  a.crows = spatial ? P.crows_sp : P.crows_ang;
+  a.cexp = nullptr; a.status = B.status;
+  return a;
+}
+// adds A^T B (b null: A^T A) over the rows of the family; returns it for further options
+static OzProd& oz_add(OzGram& a, OzRows rows, const double* A, int lda, const int* acnt,
+                      const double* b, int ldb, const int* bcnt, int bfix, int wsel = W_NONE,
+                      const double* wrow = nullptr) {
+  OzProd& p = a.p[a.nprod];
+  p.A = A; p.lda = lda; p.acnt = acnt; p.afix = 0;
+  p.B = b; p.ldb = ldb; p.bcnt = bcnt; p.bfix = bfix;
+  p.rows = rows; p.aside = -1; p.shift = 0; p.wsel = wsel; p.wrow = wrow;
+  p.blk = a.nprod++;
+  return p;
+}
+
 static void gram(const Problem& P, const PhaseBufs& B, cudaStream_t st, int spatial,
                  const double* A, int lda, const int* acnt, int afix, const double* Bm, int ldb,
                  const int* bcnt, int bfix, int b_per_sub, const double* wrow, int dst_small) {
+  if ((spatial ? P.ozg_sp : P.ozg_ang) && b_per_sub && acnt) {
+    OzGram o = oz_products(P, B, spatial, 0, 1);
+    const bool sym = A == Bm && lda == ldb && acnt == bcnt && !wrow;   // a weight goes on one side only
+    oz_add(o, spatial ? OG_CELLS : OG_DIRS, A, lda, acnt, sym ? nullptr : Bm, ldb, bcnt, bfix,
+           wrow ? W_ROW : W_NONE, wrow);
+    OzDst d;
+    d.idx[0] = dst_small;
+    if (oz_gram(P, st, o, &d, B.sm)) return;
+  }
   GramArgs a;
   a.spatial = spatial; a.A = A; a.lda = lda; a.acnt = acnt; a.afix = afix;
   a.Bm = Bm; a.ldb = ldb; a.bcnt = bcnt; a.bfix = bfix; a.b_per_sub = b_per_sub;
@@ -1873,18 +1783,28 @@ static void gram(const Problem& P, const PhaseBufs& B, cudaStream_t st, int spat
 }
 
 // chunked Gram A^T A left as partial sums in B.part (summed by the consumer); returns
-// the number of chunks
+// the number of chunks (their stride), *crows the rows of one (0: the chunks divide every
+// subdomain's rows)
 static int gram_partials(const Problem& P, const PhaseBufs& B, cudaStream_t st, int spatial,
-                         const double* A, int lda, const int* acnt, int* cexp) {
+                         const double* A, int lda, const int* acnt, int* cexp, int* crows) {
+  if (spatial ? P.ozg_sp : P.ozg_ang) {
+    OzGram o = oz_products(P, B, spatial, 0, 1);
+    o.cexp = cexp;
+    o.crows = spatial ? P.ocrows_sp : P.ocrows_ang;
+    o.nchunk = ((spatial ? P.maxN : P.g.n) + o.crows - 1) / o.crows;
+    oz_add(o, spatial ? OG_CELLS : OG_DIRS, A, lda, acnt, nullptr, 0, nullptr, 0);
+    if (oz_gram(P, st, o, nullptr, nullptr)) {
+      *crows = o.crows;
+      return o.nchunk;
+    }
+  }
+  *crows = 0;
   GramArgs a;
   a.spatial = spatial; a.A = A; a.lda = lda; a.acnt = acnt; a.afix = 0;
   a.Bm = A; a.ldb = lda; a.bcnt = acnt; a.bfix = 0; a.b_per_sub = 1;
   a.wrow = nullptr; a.part = B.part; a.nchunk = spatial ? P.ochunk_sp : P.ochunk_ang;
   a.cexp = cexp;
   a.sym = 1;
-  if ((spatial ? P.ozg_sp : P.ozg_ang) &&
-      oz_gram(P, B.status, st, spatial, A, lda, acnt, B.part, a.nchunk, cexp))
-    return a.nchunk;
   pbeg(st, KS_GRAM);
   k_gram<<<dim3(a.nchunk, P.g.nsub), DD_THREADS, sizeof(double) * P.g.RC * P.g.RC, st>>>(P.g, a);
   pend(st);
@@ -1897,7 +1817,7 @@ static int gram_partials(const Problem& P, const PhaseBufs& B, cudaStream_t st, 
 static void tall(const Problem& P, const PhaseBufs& B, cudaStream_t st, int spatial,
                  const double* A, int lda, const int* ninner, int ninner_fix, const double* Bm,
                  int bsmall, const int* ncols, int ncols_fix, double* Y, int ldy,
-                 double* gpart = nullptr);
+                 double* gpart = nullptr, int mtrans = 0, int accumulate = 0);
 static void galerkin_tall(const Problem& P, const PhaseBufs& B, cudaStream_t st, int spatial,
                           const double* A, int lda, const int* ninner, const double* Bm,
                           int bsmall, const int* ncols, double* Y, int ldy) {
@@ -1910,15 +1830,15 @@ static void galerkin_tall(const Problem& P, const PhaseBufs& B, cudaStream_t st,
 static void tall(const Problem& P, const PhaseBufs& B, cudaStream_t st, int spatial,
                  const double* A, int lda, const int* ninner, int ninner_fix, const double* Bm,
                  int bsmall, const int* ncols, int ncols_fix, double* Y, int ldy,
-                 double* gpart) {
+                 double* gpart, int mtrans, int accumulate) {
   if ((spatial ? P.oz_sp : P.oz_ang) && !gpart &&
       oz_tall(P, B.status, st, spatial, A, lda, ninner, ninner_fix, Bm, bsmall,
-                                B.sm, ncols, ncols_fix, Y, ldy))
+                                B.sm, ncols, ncols_fix, Y, ldy, mtrans, accumulate))
     return;
   TallArgs a;
   a.spatial = spatial; a.A = A; a.lda = lda; a.ninner = ninner; a.ninner_fix = ninner_fix;
   a.Bm = Bm; a.bsmall = bsmall; a.ncols = ncols; a.ncols_fix = ncols_fix; a.Y = Y; a.ldy = ldy;
-  a.gpart = gpart;
+  a.gpart = gpart; a.mtrans = mtrans; a.accumulate = accumulate;
   const int rows = spatial ? P.maxN : P.g.n;
   dim3 grid((rows + TALL_ROWS - 1) / TALL_ROWS, P.g.nsub);
   pbeg(st, KS_TALL);
@@ -1959,7 +1879,7 @@ __global__ void k_trial_fill(double* a, long n) {
 
 namespace {
 struct TuneChoice {
-  int oz_sp, oz_ang, nch_sp, nch_ang, ozg_sp, ozg_ang;
+  int oz_sp, oz_ang, nch_sp, nch_ang, ozg_sp, ozg_ang, crows_sp, crows_ang;
   double ms[8];
 };
 std::mutex g_tune_mu;
@@ -1998,7 +1918,11 @@ cudaError_t autotune(Problem& P, const PhaseBufs& B, cudaStream_t st, int tune_p
       if (tune_products) {
         P.oz_sp = c.oz_sp; P.oz_ang = c.oz_ang; P.ozg_sp = c.ozg_sp; P.ozg_ang = c.ozg_ang;
       }
-      if (tune_chunks) { P.ochunk_sp = c.nch_sp; P.ochunk_ang = c.nch_ang; }
+      if (tune_chunks) {
+        P.ochunk_sp = c.nch_sp; P.ochunk_ang = c.nch_ang;
+        P.ocrows_sp = std::max(P.ocrows_sp, c.crows_sp);       // (at most GRAM_CHUNKS chunks)
+        P.ocrows_ang = std::max(P.ocrows_ang, c.crows_ang);
+      }
       for (int i = 0; i < 8; ++i) ms[i] = c.ms[i];
       return cudaSuccess;
     }
@@ -2035,10 +1959,7 @@ cudaError_t autotune(Problem& P, const PhaseBufs& B, cudaStream_t st, int tune_p
       Qg.ozg_sp = Qg.ozg_ang = 1;
       auto gram_trial = [&](const Problem& R) {
         return time_on(st, REPS, [&] {
-          const int n = gram_partials(R, B, st, sp, A, RC, B.keep, nullptr);
-          Dst d;
-          for (int i = 0; i < 8; ++i) d.idx[i] = SM_QM;
-          reduce_to(R, B, st, n, 1, d);
+          gram(R, B, st, sp, A, RC, B.keep, 0, A, RC, B.keep, 0, 1, nullptr, SM_QM);
         });
       };
       const double tg64 = gram_trial(Q), tgoz = gram_trial(Qg);
@@ -2061,7 +1982,26 @@ cudaError_t autotune(Problem& P, const PhaseBufs& B, cudaStream_t st, int tune_p
       const int pick = oz_ok && toz > 0.0 && toz < t64 ? 1 : 0;
       if (sp) P.oz_sp = pick; else P.oz_ang = pick;
     }
-    if (tune_chunks) {
+    if (tune_chunks && (sp ? P.ozg_sp : P.ozg_ang)) {
+      // the rows per item of the tensor-core Gram: the heuristic's, twice and four times that
+      int& rows = sp ? P.ocrows_sp : P.ocrows_ang;
+      const int h = rows;
+      double best = -1.0, worst = -1.0;
+      int pick = h;
+      for (int cand : {h, 2 * h, 4 * h}) {
+        Problem Q = P;
+        (sp ? Q.ocrows_sp : Q.ocrows_ang) = cand;
+        const double t = time_on(st, REPS, [&] {
+          int crows;
+          (void)gram_partials(Q, B, st, sp, A, RC, B.keep, nullptr, &crows);
+        });
+        if (t > 0.0 && (best < 0.0 || t < 0.97 * best)) { best = t; pick = cand; }
+        worst = std::max(worst, t);
+      }
+      rows = pick;
+      ms[4 * f + 2] = best;
+      ms[4 * f + 3] = worst;
+    } else if (tune_chunks) {
       // the orthonormalisations' Gram A^T A with its fixed-order reduction, at the
       // heuristic's chunk count and at a half and a quarter of it (the partials buffer is
       // sized for the heuristic's; the Galerkin products keep it)
@@ -2074,7 +2014,8 @@ cudaError_t autotune(Problem& P, const PhaseBufs& B, cudaStream_t st, int tune_p
         Problem Q = P;
         (sp ? Q.ochunk_sp : Q.ochunk_ang) = cand;
         const double t = time_on(st, REPS, [&] {
-          const int n = gram_partials(Q, B, st, sp, A, RC, B.keep, nullptr);
+          int crows;
+          const int n = gram_partials(Q, B, st, sp, A, RC, B.keep, nullptr, &crows);
           Dst d;
           for (int i = 0; i < 8; ++i) d.idx[i] = SM_QM;
           reduce_to(Q, B, st, n, 1, d);
@@ -2096,6 +2037,7 @@ cudaError_t autotune(Problem& P, const PhaseBufs& B, cudaStream_t st, int tune_p
     TuneChoice c;
     c.oz_sp = P.oz_sp; c.oz_ang = P.oz_ang; c.nch_sp = P.ochunk_sp; c.nch_ang = P.ochunk_ang;
     c.ozg_sp = P.ozg_sp; c.ozg_ang = P.ozg_ang;
+    c.crows_sp = P.ocrows_sp; c.crows_ang = P.ocrows_ang;
     for (int i = 0; i < 8; ++i) c.ms[i] = ms[i];
     g_tune_cache[key] = c;
   }
@@ -2108,8 +2050,8 @@ static void mass_acc(const Problem& P, const PhaseBufs& B, cudaStream_t st, cons
                      const double* V, const double* S, const int* cnt, double sign) {
   pbeg(st, KS_MASS);
   k_mf_vec<<<P.g.nsub, DD_THREADS, 0, st>>>(P, V, S, cnt, B.mvec);
-  k_mf_acc<<<dim3((P.maxN + DD_THREADS - 1) / DD_THREADS, P.g.nsub), DD_THREADS, 0, st>>>(
-      P, A, cnt, B.mvec, sign, B.dm);
+  k_mf_acc<<<dim3((P.maxN + DD_THREADS - 1) / DD_THREADS, P.g.nsub), DD_THREADS, 0, st>>>(P, A, cnt,
+      B.mvec, sign, B.dm);
   pend(st);
 }
 
@@ -2131,16 +2073,17 @@ static OrthArgs orth_args(const Problem& P, const PhaseBufs& B, int spatial, int
 static void orthonormalize(const Problem& P, const PhaseBufs& B, cudaStream_t st, OrthArgs a) {
   const int sp = a.spatial;
   double* W = sp ? B.Hw : B.Hwa;
-  int nch = gram_partials(P, B, st, sp, a.A, a.lda, a.acols, B.cexp);
-  launch_geig(a, B.part, B.cexp, nch, 0, B.sm, SM_QM, B.keep, st);
+  int crows, nch = gram_partials(P, B, st, sp, a.A, a.lda, a.acols, B.cexp, &crows);
+  launch_geig(a, B.part, B.cexp, nch, crows, B.sm, SM_QM, B.keep, st);
   // U1 = A M; its Gram from the same tiles when their partials fit the buffer (one partial
   // per 32-row tile, counted from each subdomain's first row), else by k_gram
   const int ntile = ((sp ? P.maxN : P.g.n) + TALL_ROWS - 1) / TALL_ROWS;
   const bool fuse = !(sp ? P.oz_sp : P.oz_ang) && ntile <= 8 * std::max(P.nchunk_sp, P.nchunk_ang);
   tall(P, B, st, sp, a.A, a.lda, a.acols, 0, nullptr, SM_QM, B.keep, 0, W, P.WC,
        fuse ? B.part : nullptr);
-  nch = fuse ? ntile : gram_partials(P, B, st, sp, W, P.WC, B.keep, nullptr);
-  launch_chol_inv(a, B.part, nch, 0, B.sm, SM_R1I, B.keep, st);
+  crows = 0;
+  nch = fuse ? ntile : gram_partials(P, B, st, sp, W, P.WC, B.keep, nullptr, &crows);
+  launch_chol_inv(a, B.part, nch, crows, B.sm, SM_R1I, B.keep, st);
   tall(P, B, st, sp, W, P.WC, B.keep, 0, nullptr, SM_R1I, B.keep, 0, a.Q, a.ldq);
   if (a.mode == ORTH_QR || (!sp && a.mode == ORTH_AUG)) {
     // mutually orthogonal candidates (the cosines; the angular table): coefficient-space
@@ -2176,8 +2119,27 @@ void advection_phase(const Problem& P, const PhaseBufs& B, int axis, cudaStream_
   // twice the angular chunks (more blocks than SMs), as far as the partial buffer holds
   const int nch_ac = std::min(2 * P.nchunk_ang, std::max(P.nchunk_sp, P.nchunk_ang));
   const int nblk_ac = P.kstep_split == 1 ? 8 : 6;
-  bool tc_done = false;
-  if (P.prec >= PREC_TF32 && !P.infl_on) {
+  bool oz_done = false, tc_done = false;
+  if (P.ozg_ang) {
+    // FP64-accurate on the tensor cores in every precision (faster than the split TF32 / BF16
+    // products too: one read of the rows per block instead of a double-float read-out per 32)
+    OzGram o = oz_products(P, B, 0, axis, nblk_ac);
+    oz_add(o, OG_DIRS, B.Vh, RC, B.rt, B.Vh, RC, B.rt, 0, W_OMEGA);                   // C
+    oz_add(o, OG_DIRS, B.Vh, RC, B.rt, nullptr, 0, nullptr, 0, W_NEG);                // Mout_lo
+    oz_add(o, OG_DIRS, B.Vh, RC, B.rt, nullptr, 0, nullptr, 0, W_NONNEG);             // Mout_hi
+    oz_add(o, OG_DIRS, B.V, RC, B.r, B.Vh, RC, B.rt, 0);                              // M
+    oz_add(o, OG_DIRS, B.V, RC, B.r, B.Vh, RC, B.rt, 0, W_NONNEG).aside = 0;          // Min_lo
+    oz_add(o, OG_DIRS, B.V, RC, B.r, B.Vh, RC, B.rt, 0, W_NEG).aside = 1;             // Min_hi
+    if (nblk_ac == 8) {
+      oz_add(o, OG_DIRS, B.Vh, RC, B.rt, B.Vh, RC, B.rt, 0, W_OMEGA_POS);             // C+
+      oz_add(o, OG_DIRS, B.Vh, RC, B.rt, B.Vh, RC, B.rt, 0, W_OMEGA_NEG);             // C-
+    }
+    OzDst d;
+    const int slots[8] = {SM_C, SM_MOUT_LO, SM_MOUT_HI, SM_M, SM_MIN_LO, SM_MIN_HI, SM_CP, SM_CM};
+    for (int i = 0; i < 8; ++i) d.idx[i] = slots[i];
+    oz_done = oz_gram(P, st, o, &d, B.sm);
+  }
+  if (!oz_done && P.prec >= PREC_TF32 && !P.infl_on) {
     // the six (eight) blocks as weighted Grams against Vh; the sources that read Vh itself
     // take the even slots, the own and neighbour V the odd ones
     TcGram a = tgram(P, B, 0, axis, B.Vh, B.rt, nch_ac, nblk_ac);
@@ -2198,14 +2160,14 @@ void advection_phase(const Problem& P, const PhaseBufs& B, int axis, cudaStream_
     }
     tc_done = tc_gram(P, st, a);
   }
-  if (!tc_done) {
+  if (!oz_done && !tc_done) {
     pbeg(st, KS_ANG_COEFFS);
     k_ang_coeffs<<<dim3(nch_ac, nsub), DD_THREADS, 0, st>>>(
         g, axis == 0 ? P.ox : P.oy, B.Vh, B.V, B.r, B.rt, axis, nch_ac, nblk_ac, B.part,
         P.infl_on, P.infl_hw);
     pend(st);
   }
-  {
+  if (!oz_done) {
     Dst d;
     d.idx[0] = SM_C; d.idx[1] = SM_MOUT_LO; d.idx[2] = SM_MOUT_HI;
     d.idx[3] = SM_M; d.idx[4] = SM_MIN_LO; d.idx[5] = SM_MIN_HI;
@@ -2227,55 +2189,29 @@ void advection_phase(const Problem& P, const PhaseBufs& B, int axis, cudaStream_
   // 6. K-step
   {
     const int len = P.maxlines;
-    // with the spatial tall products on the tensor cores (and, for RK4, every line within
-    // the eigenbasis tile): the two basis changes as tall products (K~ = K P into X1, free
-    // until the QR; K += increment P^T, accumulated in FP64 by the product's epilogue:
-    // rotating the whole K back would put rounding of K's size on entries whose increment is
-    // tiny), the stages in the eigenbasis in between
-    const bool euler = P.integrator == 0;
-    const bool ebasis = P.kstep_split == 0 && P.oz_sp &&
-                        (euler || (long)len * g.RC <= (long)DD_THREADS * KE_EPT);
-    if (ebasis && oz_tall(P, B.status, st, 1, B.K, RC, B.rt, 0, nullptr, SM_S3T, B.sm, B.rt, 0,
-                          B.X1, RC, 0)) {
-      // the stages on K~ (the increment into Hw with Euler, in place in X1 with RK4), then
-      // K += increment P^T by the second product (the same shape as the first: it cannot be
-      // refused where that one was not)
+    if (P.kstep_split == 0) {
+      // FP64 eigen-split in the eigenbasis, in every precision (an FP32 matrix stencil rounds
+      // |C| K_i, C+ K_i-1 and C- K_i+1, which cancel to the much smaller increment, and its
+      // error grew to 1e-4..1e-3 of the flux on narrow sources): K~ = K P into X1 (free until
+      // the QR), the stages into Hw, K += increment P^T by the accumulating product (rotating
+      // the whole K back would put rounding of K's size on entries whose increment is tiny)
+      tall(P, B, st, 1, B.K, RC, B.rt, 0, nullptr, SM_S3T, B.rt, 0, B.X1, RC);
+      const int seg = kstep_seg(P);
+      const long per = (long)P.maxlines * ((len + seg - 1) / seg) * RC;
       pbeg(st, KS_KSTEP_ADV);
-      if (euler) {
-        k_kstep_eig1<<<dim3(P.maxlines, nsub), DD_THREADS, 0, st>>>(P, B, axis);
-      } else {
-        const int lpb = kstep_eig_lpb(P, len);
-        dim3 grid((P.maxlines + lpb - 1) / lpb, nsub);
-        k_kstep_eig<double><<<grid, DD_THREADS, kstep_eig_smem(P, lpb, len), st>>>(P, B, axis, lpb, 1);
-      }
+      k_kstep_line<<<dim3((unsigned)((per + DD_THREADS - 1) / DD_THREADS), nsub), DD_THREADS, 0, st>>>(
+          P, B, axis, seg);
       pend(st);
-      (void)oz_tall(P, B.status, st, 1, euler ? B.Hw : B.X1, RC, B.rt, 0, nullptr, SM_S3T, B.sm,
-                    B.rt, 0, B.K, RC, 1, 1);
-    } else {
-    pbeg(st, KS_KSTEP_ADV);
-    if (P.kstep_split == 0 && len < 4096) {
-      // FP64 eigen-split in the eigenbasis, in the mixed form too: the FP32 matrix
-      // stencil rounds |C| K_i, C+ K_i-1 and C- K_i+1, which cancel to the much smaller
-      // increment, and its error grew to 1e-4..1e-3 of the flux on narrow sources
-      const int lpb = kstep_eig_lpb(P, len);
-      dim3 grid((P.maxlines + lpb - 1) / lpb, nsub);
-      k_kstep_eig<double><<<grid, DD_THREADS, kstep_eig_smem(P, lpb, len), st>>>(P, B, axis, lpb, 0);
-      if ((long)len * g.RC > (long)DD_THREADS * KE_EPT) {
-        // subdomains whose line exceeds the eigenbasis kernel's tile: the FP64 matrix
-        // stencil (the same discrete operator)
-        const int lpb2 = kstep_lpb(P, len);
-        dim3 grid2((P.maxlines + lpb2 - 1) / lpb2, nsub);
-        k_kstep_adv<double><<<grid2, DD_THREADS, kstep_smem(P, lpb2, len), st>>>(P, B, axis, lpb2, 1);
-      }
+      tall(P, B, st, 1, B.Hw, P.WC, B.rt, 0, nullptr, SM_S3T, B.rt, 0, B.K, RC, nullptr, 1, 1);
     } else {
       const int lpb = kstep_lpb(P, len);
       dim3 grid((P.maxlines + lpb - 1) / lpb, nsub);
+      pbeg(st, KS_KSTEP_ADV);
       if (P.prec >= PREC_MIXED)
-        k_kstep_adv<float><<<grid, DD_THREADS, kstep_smem(P, lpb, len), st>>>(P, B, axis, lpb, 0);
+        k_kstep_adv<float><<<grid, DD_THREADS, kstep_smem(P, lpb, len), st>>>(P, B, axis, lpb);
       else
-        k_kstep_adv<double><<<grid, DD_THREADS, kstep_smem(P, lpb, len), st>>>(P, B, axis, lpb, 0);
-    }
-    pend(st);
+        k_kstep_adv<double><<<grid, DD_THREADS, kstep_smem(P, lpb, len), st>>>(P, B, axis, lpb);
+      pend(st);
     }
   }
   if (P.mass_fix) mass_acc(P, B, st, B.K, B.Vh, nullptr, B.rt, 1.0);
@@ -2286,13 +2222,23 @@ void advection_phase(const Problem& P, const PhaseBufs& B, int axis, cudaStream_
     orthonormalize(P, B, st, a);
   }
   // 8. S-step coefficients and S-step
-  bool sp_tc = false;
-  {
+  oz_done = false;
+  if (P.ozg_sp) {
+    OzGram o = oz_products(P, B, 1, axis, 4);
+    oz_add(o, OG_CELLS, B.X1, RC, B.rt, B.K, RC, B.rt, 0);                            // S1
+    oz_add(o, OG_CELLS, B.X1, RC, B.rt, B.X1, RC, B.rt, 0).shift = 1;                 // T
+    oz_add(o, OG_FACE_LO, B.X1, RC, B.rt, B.Kb, RC, B.rt, 0);                         // G_lo
+    oz_add(o, OG_FACE_HI, B.X1, RC, B.rt, B.Kb, RC, B.rt, 0);                         // G_hi
+    OzDst d;
+    d.idx[0] = SM_S1; d.idx[1] = SM_T; d.idx[2] = SM_G_LO; d.idx[3] = SM_G_HI;
+    oz_done = oz_gram(P, st, o, &d, B.sm);
+  }
+  if (!oz_done) {
     // the spatial coefficient T = X1^T shift(X1) on the tensor cores in its difference form
     // E = X1^T (X1 - shift(X1)) = I - T (a Gram against X1, written transposed; the
     // reduction forms T = I - E); S1 = X1^T K (the R factor of the QR of K) and the face
     // products G_lo, G_hi in FP64
-    bool& tcd = sp_tc;
+    bool tcd = false;
     if (P.prec >= PREC_TF32) {
       TcGram a = tgram(P, B, 1, axis, B.X1, B.rt, P.nchunk_sp, 4);
       a.src[0] = gsrc(B.X1, RC, B.rt, 1, W_NONE, nullptr, 1);
@@ -2303,11 +2249,9 @@ void advection_phase(const Problem& P, const PhaseBufs& B, int axis, cudaStream_
     pbeg(st, KS_SP_COEFFS);
     k_sp_coeffs<<<dim3(P.nchunk_sp, nsub), DD_THREADS, 0, st>>>(P, B, axis, tcd ? 1 : 0);
     pend(st);
-  }
-  {
     Dst d;
     d.idx[0] = SM_S1; d.idx[1] = SM_T; d.idx[2] = SM_G_LO; d.idx[3] = SM_G_HI;
-    d.ident = sp_tc ? 2 : 0;
+    d.ident = tcd ? 2 : 0;
     pbeg(st, KS_REDUCE);
     k_reduce<<<reduce_grid(g, 4), DD_THREADS, 0, st>>>(B.part, P.nchunk_sp, 4, d, B.sm, RC);
     pend(st);
@@ -2396,59 +2340,69 @@ void collision_phase(const Problem& P, const PhaseBufs& B, cudaStream_t st) {
     a.A = B.K; a.lda = RC; a.acols = B.rc; a.Q = B.Xo; a.ldq = RC; a.rout = B.rc;
     orthonormalize(P, B, st, a);
   }
-  // S1 = Xo^T K (the R factor of the QR of K) in FP64; the Galerkin contractions
-  // Ms = Xo^T diag(sigma_s) Xo, Mt = Xo^T diag(sigma_t) Xo on the tensor cores in the
-  // DD_TF32 / DD_BF16 forms
-  gram(P, B, st, 1, B.Xo, RC, B.rc, 0, B.K, RC, B.rc, 0, 1, nullptr, SM_S1);
-  {
-    bool tcd = false;
-    if (P.prec >= PREC_TF32) {
-      TcGram a = tgram(P, B, 1, 0, B.Xo, B.rc, P.nchunk_sp, 2);
-      a.src[0] = gsrc(nullptr, RC, B.rc, 0, W_ROW, P.sig_s);
-      a.src[0].same_as_b = 1;
-      a.src[1] = a.src[0];
-      a.src[1].blk = 1;
-      a.src[1].wrow = P.sig_t;
-      a.nsrc = 2;
-      if ((tcd = tc_gram(P, st, a))) {
-        Dst d;
-        d.idx[0] = SM_MS; d.idx[1] = SM_MT;
-        reduce_to(P, B, st, P.nchunk_sp, 2, d);
+  // S1 = Xo^T K (the R factor of the QR of K), Ms = Xo^T diag(sigma_s) Xo,
+  // Mt = Xo^T diag(sigma_t) Xo and q = Xo^T sQ (column 0 of a scratch block)
+  bool oz_done = false;
+  if (P.ozg_sp) {
+    OzGram o = oz_products(P, B, 1, 0, 4);
+    oz_add(o, OG_CELLS, B.Xo, RC, B.rc, B.K, RC, B.rc, 0);
+    oz_add(o, OG_CELLS, B.Xo, RC, B.rc, B.Xo, RC, B.rc, 0, W_ROW, P.sig_s);
+    oz_add(o, OG_CELLS, B.Xo, RC, B.rc, B.Xo, RC, B.rc, 0, W_ROW, P.sig_t);
+    oz_add(o, OG_CELLS, B.Xo, RC, B.rc, P.sQ, 1, nullptr, 1);
+    OzDst d;
+    d.idx[0] = SM_S1; d.idx[1] = SM_MS; d.idx[2] = SM_MT; d.idx[3] = SM_UB;
+    oz_done = oz_gram(P, st, o, &d, B.sm);
+  }
+  if (!oz_done) {
+    gram(P, B, st, 1, B.Xo, RC, B.rc, 0, B.K, RC, B.rc, 0, 1, nullptr, SM_S1);
+    {
+      bool tcd = false;
+      if (P.prec >= PREC_TF32) {
+        TcGram a = tgram(P, B, 1, 0, B.Xo, B.rc, P.nchunk_sp, 2);
+        a.src[0] = gsrc(nullptr, RC, B.rc, 0, W_ROW, P.sig_s);
+        a.src[0].same_as_b = 1;
+        a.src[1] = a.src[0];
+        a.src[1].blk = 1;
+        a.src[1].wrow = P.sig_t;
+        a.nsrc = 2;
+        if ((tcd = tc_gram(P, st, a))) {
+          Dst d;
+          d.idx[0] = SM_MS; d.idx[1] = SM_MT;
+          reduce_to(P, B, st, P.nchunk_sp, 2, d);
+        }
+      }
+      if (!tcd) {
+        gram(P, B, st, 1, B.Xo, RC, B.rc, 0, B.Xo, RC, B.rc, 0, 1, P.sig_s, SM_MS);
+        gram(P, B, st, 1, B.Xo, RC, B.rc, 0, B.Xo, RC, B.rc, 0, 1, P.sig_t, SM_MT);
       }
     }
-    if (!tcd) {
-      gram(P, B, st, 1, B.Xo, RC, B.rc, 0, B.Xo, RC, B.rc, 0, 1, P.sig_s, SM_MS);
-      gram(P, B, st, 1, B.Xo, RC, B.rc, 0, B.Xo, RC, B.rc, 0, 1, P.sig_t, SM_MT);
+    // q = X1^T sQ  -> row 1 of the vector block (reduce into a scratch small, then copy)
+    {
+      GramArgs a;
+      a.spatial = 1; a.A = B.Xo; a.lda = RC; a.acnt = B.rc; a.afix = 0;
+      a.Bm = P.sQ; a.ldb = 1; a.bcnt = nullptr; a.bfix = 1; a.b_per_sub = 1;
+      a.wrow = nullptr; a.part = B.part; a.nchunk = P.nchunk_sp; a.cexp = nullptr; a.sym = 0;
+      pbeg(st, KS_GRAM);
+      k_gram<<<dim3(a.nchunk, nsub), DD_THREADS, sizeof(double) * RC * RC, st>>>(g, a);
+      pend(st);
+      Dst d;
+      d.idx[0] = SM_UB;   // scratch: column 0 holds q
+      pbeg(st, KS_REDUCE);
+      k_reduce<<<reduce_grid(g, 1), DD_THREADS, 0, st>>>(B.part, a.nchunk, 1, d, B.sm, RC);
+      pend(st);
     }
-  }
-  // q = X1^T sQ  -> row 1 of the vector block (reduce into a scratch small, then copy)
-  {
-    GramArgs a;
-    a.spatial = 1; a.A = B.Xo; a.lda = RC; a.acnt = B.rc; a.afix = 0;
-    a.Bm = P.sQ; a.ldb = 1; a.bcnt = nullptr; a.bfix = 1; a.b_per_sub = 1;
-    a.wrow = nullptr; a.part = B.part; a.nchunk = P.nchunk_sp; a.cexp = nullptr; a.sym = 0;
-    pbeg(st, KS_GRAM);
-    k_gram<<<dim3(a.nchunk, nsub), DD_THREADS, sizeof(double) * RC * RC, st>>>(g, a);
-    pend(st);
-    Dst d;
-    d.idx[0] = SM_UB;   // scratch: column 0 holds q
-    pbeg(st, KS_REDUCE);
-    k_reduce<<<reduce_grid(g, 1), DD_THREADS, 0, st>>>(B.part, a.nchunk, 1, d, B.sm, RC);
-    pend(st);
   }
   pbeg(st, KS_COLL_SMALL);
   k_coll_small<<<nsub, DD_THREADS, sizeof(double) * (4 * RC * RC + 5 * RC), st>>>(P, B);
   pend(st);
   pbeg(st, KS_COLL_LSTEP);
   if (P.prec >= PREC_MIXED) {
-    k_coll_lstep<float><<<dim3((g.n + 31) / 32, nsub), DD_THREADS,
-                   coll_lstep_smem(RC), st>>>(P, B);
+    k_coll_lstep<float><<<dim3((g.n + 31) / 32, nsub), DD_THREADS, coll_lstep_smem(RC), st>>>(P, B);
   } else if (P.integrator == 0) {
-    k_coll_lstep1<<<dim3((g.n + DD_THREADS - 1) / DD_THREADS, nsub), DD_THREADS,
-                    coll_lstep1_smem(RC), st>>>(P, B);
+    k_coll_lstep1<<<dim3((g.n + DD_THREADS - 1) / DD_THREADS, nsub), DD_THREADS, coll_lstep1_smem(RC), st>>>(
+        P, B);
   } else {
-    k_coll_lstep<double><<<dim3((g.n + 31) / 32, nsub), DD_THREADS,
-                   coll_lstep_smem(RC), st>>>(P, B);
+    k_coll_lstep<double><<<dim3((g.n + 31) / 32, nsub), DD_THREADS, coll_lstep_smem(RC), st>>>(P, B);
   }
   pend(st);
   {

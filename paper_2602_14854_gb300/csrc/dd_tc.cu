@@ -106,6 +106,9 @@ struct TcTall {
   int tps;                          // 128-row tiles per subdomain (of the largest)
   unsigned* status;
   const double* A;                  // A itself (the kernels that load it without a tensor map)
+  long nrows;                       // rows of A (the Ozaki kernel's prefetch)
+  int zfill;                        // columns nc .. ldy - 1 of Y set to zero (the Ozaki kernel; k_tc_*
+                                    // load whole rows)
   int mtrans;                       // M read transposed (the Ozaki kernel)
   const double* rowscale;           // accumulate: Y_r += rowscale_r (A M)_r (the Ozaki kernel; null: 1)
 };
@@ -497,44 +500,11 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_tc_gram(const __grid_constant
 // |M'[k][n]| per entry (the FP64 rounding of each product is 2^-53 of the product).  No FP64
 // arithmetic runs in the kernel.
 //
-// A CTA (one per SM: 16 worker warps and one warp that issues the MMAs) walks a contiguous
-// range of 128-row tiles.  M's digit planes
-// are formed once per subdomain.  Per tile, each warp loads 8 rows straight into registers
-// (16-byte loads, 8 rows x 64 bytes per instruction), takes the row bounds by shuffles and
-// writes the digit planes (two digits per 32-bit shared store); one thread then issues the
-// 28 x (K / 16) MMAs.  The planes are double-buffered: tile i's MMAs run while the warps
-// convert tile i + 1, and tile i's epilogue (TMEM -> registers -> FP64 -> a per-warp
-// transposition buffer -> whole-row stores) follows.  When two buffers of a whole row's
-// planes do not fit beside M's (lda > 48), K runs in two passes of 32: the stages (one pass
-// of one tile each) alternate between the two buffers all the same.
 #define OZ_DIG 7
 #define OZ_WORKERS 512                       // 16 warps: loads, digits, epilogue
 #define OZ_THREADS (OZ_WORKERS + 32)         // + one warp that issues the MMAs
 #define OZ_WARPS (OZ_WORKERS / 32)
 #define OZ_NONE (-(1 << 20))                 // exponent of an all-zero row / column
-#define OZ_EPI (OZ_WARPS * 32 * 5 * 8)       // epilogue buffers: 32 rows x 4 (+1) per warp
-#define OZ_SMEM_LIMIT (227 * 1024 - 4096)    // dynamic shared memory (the static part is < 4 KiB)
-
-struct OzPlan {
-  int KP, KA, npass, nbuf;                   // K extent of M's planes, of a pass; passes; buffers (2)
-  size_t mpl, apl, abuf, total;              // bytes: one M plane, one A plane, one A buffer, all
-};
-// the shared-memory plan for inner dimensions up to lda (even, <= 64)
-OzPlan oz_plan(int lda, size_t limit) {
-  OzPlan p;
-  p.KP = (lda + 15) / 16 * 16;
-  p.mpl = (size_t)DD_MAXC * 2 * p.KP;
-  for (int mode = 0; mode < 2; ++mode) {
-    p.KA = mode ? 32 : p.KP;
-    p.nbuf = 2;
-    p.npass = (p.KP + p.KA - 1) / p.KA;
-    p.apl = (size_t)TT_ROWS * 2 * p.KA;
-    p.abuf = std::max((size_t)OZ_DIG * p.apl, (size_t)OZ_EPI);
-    p.total = 128 + OZ_DIG * p.mpl + p.nbuf * p.abuf;
-    if (p.total <= limit) break;
-  }
-  return p;
-}
 
 // biased FP64 exponent of x (0 for zero and subnormals)
 __device__ __forceinline__ int f64_bexp(double x) {
@@ -571,603 +541,1112 @@ __device__ __forceinline__ void oz_digits(double x, int e, float* d) {
 __device__ __forceinline__ uint32_t oz_pack(float lo, float hi) {
   return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
 }
-// J * 2^sc as an FP64 (round to nearest even), by integer operations
-__device__ __forceinline__ double oz_to_f64(long long J, int sc) {
-  if (J == 0) return 0.0;
-  const unsigned long long sg = J < 0 ? 0x8000000000000000ull : 0ull;
-  unsigned long long u = J < 0 ? (unsigned long long)(-J) : (unsigned long long)J;
-  int msb = 63 - __clzll((long long)u);
-  unsigned long long r;
-  if (msb > 52) {
-    const int sh = msb - 52;
-    r = u >> sh;
-    const unsigned long long rem = u & ((1ull << sh) - 1ull), half = 1ull << (sh - 1);
-    if (rem > half || (rem == half && (r & 1ull))) ++r;
-    if (r >> 53) { r >>= 1; ++msb; }
-  } else {
-    r = u << (52 - msb);
-  }
-  const int be = 1023 + msb + sc;
-  if (be <= 0) return __longlong_as_double((long long)sg);
-  if (be >= 2047) return __longlong_as_double((long long)(sg | 0x7ff0000000000000ull));
-  return __longlong_as_double((long long)(sg | ((unsigned long long)be << 52) | (r & 0xfffffffffffffull)));
+// ---- roles of a CTA of k_oz_tall --------------------------------------------------------
+// One CTA per SM, its warps specialised, handing 128-row tiles over through mbarriers:
+//   16 converter warps  8 rows of A each -> registers -> digit planes of A' in shared memory,
+//                       M's digit planes once per subdomain;
+//   1 MMA warp          one thread issues the digit products of a tile, 16 columns of Y at a
+//                       time, into one of four TMEM buffers (7 accumulators of 16 columns);
+//   8 epilogue warps    TMEM -> registers (the buffer is free again at once) -> FP64 -> Y.
+// Conversion (integer and FP32 issue), the tensor cores and the epilogue (integer issue) of
+// different tiles overlap; before, all 16 worker warps converted a tile's digits, then all of
+// them ran the previous tile's epilogue, with CTA-wide barriers between, and issued on 40% of
+// the cycles.  262144 x 40 x 40 (64 subdomains, lda 60), per launch: 166 us before, 47 now.
+//
+// Digit planes of A: rows of 2 KP bytes (KP = the inner dimension rounded up to 16), plane s
+// of a stage at s APL; two stages while KP <= 48, one for KP = 64.  M: for column chunk c of
+// 16, plane u: rows (7 c + u) 16 + n, so the planes a product needs are adjacent along N: A's
+// plane s times M's planes 0 .. 6 - s is one MMA of N = 16 (7 - s) into the accumulators
+// s .. 6 of the buffer.
+#define OT_CONV 16
+#define OT_EPI 8
+#define OT_THREADS ((OT_CONV + OT_EPI + 1) * 32)
+#define OT_NB 4                              // TMEM buffers of 128 columns (7 x 16 in use)
+// tiles whose row and column exponents are kept: a converter is at most 5 tiles ahead of the
+// epilogue (2 stages, and the MMAs of the tile before them wait for one of 4 TMEM buffers)
+#define OT_RING 8
+#define OT_AHEAD 3                           // tiles of A on their way into L2 ahead of the converters
+
+static uint32_t ot_mpl(int KP) { return (uint32_t)OZ_DIG * DD_MAXC * 2 * KP; }
+static uint32_t ot_apl(int KP) { return (uint32_t)OZ_DIG * TT_ROWS * 2 * KP; }
+// dynamic shared memory for inner dimensions up to lda (<= 64): the largest plan among them
+static size_t ot_smem(int lda) {
+  size_t most = 0;
+  for (int KP = 16; KP <= (lda + 15) / 16 * 16; KP += 16)
+    most = std::max(most, (size_t)ot_mpl(KP) + (KP <= 48 ? 2 : 1) * (size_t)ot_apl(KP));
+  return most + 128;
 }
-// tcgen05.ld of 4 columns without the wait (the caller waits once for several)
+
+// Converter warps only: barrier, and barrier returning whether all of them pass true
+__device__ __forceinline__ void ot_conv_sync() { asm volatile("bar.sync 2, %0;" ::"n"(OT_CONV * 32) : "memory"); }
+__device__ __forceinline__ bool ot_conv_all(bool p) {
+  int r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\t"
+      "bar.red.and.pred q, 2, %2, p;\n\tselp.b32 %0, 1, 0, q;\n\t}\n"
+      : "=r"(r)
+      : "r"((int)p), "n"(OT_CONV * 32)
+      : "memory");
+  return r != 0;
+}
+
+// The digits of oz_digits for two values, packed: word s holds the BF16 digits s of x0 (low
+// half) and x1.  A low byte b = d + 128 becomes d in BF16 by two logic operations and one
+// packed subtraction: 128 + (b & 127) is 0x4300 | (b & 127), and what has to come off it is
+// 128 where bit 7 of b is set, else 256: 0x4300 | (~b & 128).
+__device__ __forceinline__ void oz_digits2(double x0, int e0, double x1, int e1, uint32_t* w) {
+  uint32_t vl[2], vh[2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(i ? x1 : x0);
+    const unsigned hi = (unsigned)(u >> 32);
+    const int E = (int)((hi >> 20) & 0x7ffu);
+    const int sh = 1030 + (i ? e1 : e0) - E;                 // >= 8
+    const unsigned long long m = (u << 11) | 0x8000000000000000ull;
+    long long T = (E != 0 && sh < 64) ? (long long)(m >> sh) : 0ll;
+    if (hi >> 31) T = -T;
+    const unsigned long long V = (unsigned long long)T + 0x808080808080ull;
+    vl[i] = (unsigned)V;
+    vh[i] = (unsigned)(V >> 32);
+  }
+#pragma unroll
+  for (int s = 1; s < OZ_DIG; ++s) {
+    const int b = (6 - s) & 3;                               // byte of the word
+    const uint32_t sel = (uint32_t)(b | (b << 4) | ((4 + b) << 8) | ((4 + b) << 12));
+    const uint32_t p = s <= 2 ? __byte_perm(vh[0], vh[1], sel) : __byte_perm(vl[0], vl[1], sel);
+    const uint32_t X = (p & 0x007f007fu) | 0x43004300u, Y = (~p & 0x00800080u) | 0x43004300u;
+    asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(w[s]) : "r"(X), "r"(Y));
+  }
+  w[0] = oz_pack(__int_as_float(0x4B400000 + ((int)vh[0] >> 16)) - 12582912.0f,
+                 __int_as_float(0x4B400000 + ((int)vh[1] >> 16)) - 12582912.0f);
+}
+
+// starts bringing rows [row, row + n) of the row-major A (rows x lda, lda even) into L2, none
+// past the last; one thread
+__device__ __forceinline__ void prefetch_rows(const double* A, long lda, long row, long n, long rows) {
+  n = min(n, rows - row);
+  if (n > 0)
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(A + row * lda),
+                 "r"((unsigned)(n * lda * 8))
+                 : "memory");
+}
+
+// 4 consecutive FP32 columns of this warp's 32 lanes, without the wait
 __device__ __forceinline__ void oz_tmem_ld4(uint32_t taddr, uint32_t* r) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(taddr));
 }
 
-// one tile's shape
-struct OzTile {
-  int k, nrow, ni, nc, N;
-  long row0;
-};
-// a warp's 8 rows of the tile: lane (rho, q) loads row 8 w + rho, columns 8 c + 2 q and
-// 8 c + 2 q + 1 (c < KP / 8) with 16-byte loads (8 rows x 64 bytes per instruction)
-__device__ __forceinline__ void oz_load_rows(double2 (&x)[8], const double* A, int lda,
-                                             const OzTile& t, int r, int q, int KP) {
+// The value sum_g D_g 2^(-8 g) of the seven accumulators (exact integers as FP32) as an
+// integer in units of 2^-40.  |D_0|, |D_1| <= 2^22 for at most 64 terms (digit 0 is at most
+// 256, the others 128 in magnitude): their integer is in the low bits of D + 1.5 2^23.  The
+// others take the conversion instruction.
+__device__ __forceinline__ long long oz_combine(const uint32_t* D, int stride) {
+  auto f = [&](int g) { return __uint_as_float(D[g * stride]); };
+  const int d0 = __float_as_int(f(0) + 12582912.0f) - 0x4B400000;
+  const int d1 = __float_as_int(f(1) + 12582912.0f) - 0x4B400000;
+  const int d2 = __float2int_rn(f(2)), d3 = __float2int_rn(f(3)), d4 = __float2int_rn(f(4));
+  const int d5 = __float2int_rn(f(5)), d6 = __float2int_rn(f(6));
+  long long J = (long long)(d5 + (d6 >> 8));
+  J += (long long)d4 * 256;
+  J += (long long)d3 * 65536;
+  J += (long long)d2 * 16777216;
+  J += (long long)((unsigned long long)(unsigned)(d1 + d0 * 256) << 32);
+  return J;
+}
+// J 2^sc as an FP64 (rounded to nearest), by integer operations; |J| < 2^62
+__device__ __forceinline__ double oz_round(long long J, int sc) {
+  const unsigned sg = (unsigned)(J >> 63) & 0x80000000u;
+  const unsigned long long u = (unsigned long long)(J < 0 ? -J : J);
+  const int lz = __clzll((long long)u);
+  // mantissa left-aligned at bit 62 (bit 63 free for the carry of the rounding)
+  const unsigned long long n = (u << (lz & 63)) >> 1;
+  const unsigned long long r = n + 0x1ffull + ((n >> 10) & 1ull);
+  const int be = 1023 + 63 - lz + sc;                 // exponent of the leading bit
+  unsigned long long b = (r >> 10) + ((unsigned long long)(unsigned)(be - 1) << 52);
+  if (be <= 0) b = 0ull;
+  if (be >= 2047) b = 0x7ff0000000000000ull;
+  if (u == 0ull) return 0.0;
+  return __longlong_as_double((long long)(b | ((unsigned long long)sg << 32)));
+}
+
+// 8 rows of a tile, KP = 8 C columns: lane (rho, q) loads row `row`, columns 8 c + 2 q and
+// 8 c + 2 q + 1.  The loads are unconditional (columns past the array's read its last pair; what is
+// not wanted is dropped where it is used): the compiler waits for a load under its own condition
+// before the next one.
+template <int C>
+__device__ __forceinline__ void ot_load(double2 (&d)[8], const double* row, int q, int lda) {
 #pragma unroll
-  for (int c = 0; c < 8; ++c) {
+  for (int c = 0; c < C; ++c)
+    d[c] = __ldg(reinterpret_cast<const double2*>(row + min(8 * c + 2 * q, lda - 2)));
+}
+__device__ __forceinline__ void ot_load(double2 (&d)[8], const double* row, int q, int lda, int KP) {
+  if (KP <= 16) ot_load<2>(d, row, q, lda);
+  else if (KP <= 32) ot_load<4>(d, row, q, lda);
+  else if (KP <= 48) ot_load<6>(d, row, q, lda);
+  else ot_load<8>(d, row, q, lda);
+}
+// Their digit planes (row r of the stage asl, planes APL apart) and the row bound (lanes q = 0).
+// One body per KP: with the column count a run-time bound every pair of values sat in a branch
+// of its own and waited for the one before (7 clocks per instruction and warp; the converters
+// took 12000 clocks per tile).
+template <int C>
+__device__ __forceinline__ void ot_convert(const double2 (&x)[8], const int* mexp, int ni, int q, int r,
+                                           uint8_t* asl, uint32_t APL, int* rexp) {
+  int2 me[C];
+  int mx = OZ_NONE;
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
     const int kk = 8 * c + 2 * q;
-    x[c] = make_double2(0.0, 0.0);
-    if (c < KP / 8 && r < t.nrow && kk < t.ni)
-      x[c] = __ldg(reinterpret_cast<const double2*>(A + (t.row0 + r) * lda + kk));
+    me[c] = *reinterpret_cast<const int2*>(mexp + kk);
+    if (kk >= ni) me[c].x = OZ_NONE;             // past ni, or zero rows of M: the digits are zero
+    if (kk + 1 >= ni) me[c].y = OZ_NONE;
+    const int E0 = f64_bexp(x[c].x), E1 = f64_bexp(x[c].y);
+    mx = max(mx, E0 && me[c].x != OZ_NONE ? E0 - 1022 + me[c].x : OZ_NONE);
+    mx = max(mx, E1 && me[c].y != OZ_NONE ? E1 - 1022 + me[c].y : OZ_NONE);
+  }
+  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+  if (q == 0) rexp[r] = mx;
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
+    uint32_t w[OZ_DIG];
+    oz_digits2(me[c].x != OZ_NONE ? x[c].x : 0.0, mx - me[c].x, me[c].y != OZ_NONE ? x[c].y : 0.0,
+               mx - me[c].y, w);
+    uint8_t* p = asl + tc::op_off(r, (8 * c + 2 * q) * 2, 16 * C);
+#pragma unroll
+    for (int d = 0; d < OZ_DIG; ++d) *reinterpret_cast<uint32_t*>(p + d * APL) = w[d];
   }
 }
 
-__global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_tall(TcTall a, int KP, int KA, int npass,
-                                                           int nbuf) {
+struct OtShape {
+  int rows, ni, nc, KP, nch;
+  long row0;                        // first row of the subdomain
+};
+
+__global__ void __launch_bounds__(OT_THREADS, 1) k_oz_tall(TcTall a) {
   extern __shared__ uint8_t raw_oz[];
   uint8_t* msl = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw_oz) + 127) &
-                                            ~uintptr_t(127));   // OZ_DIG planes DD_MAXC x KP
-  const uint32_t MPL = DD_MAXC * 2 * KP, APL = TT_ROWS * 2 * KA;
-  const uint32_t ABUF = max(OZ_DIG * APL, (uint32_t)OZ_EPI);
-  uint8_t* asl0 = msl + OZ_DIG * MPL;                          // 2 x (OZ_DIG planes 128 x KA)
-  __shared__ uint64_t bar_mma[2];                              // MMAs of the stages in buffer 0 / 1
+                                            ~uintptr_t(127));
+  __shared__ uint64_t full[2], empty[2], tfull[OT_NB], tempty[OT_NB], meta[OT_RING];
   __shared__ uint32_t tmem_s;
-  __shared__ int mexp[DD_MAXC], fexp[DD_MAXC], rexp[2][TT_ROWS], red[8][DD_MAXC];
+  __shared__ __align__(8) int mexp[DD_MAXC];
+  __shared__ int fnow[DD_MAXC], red[OT_CONV / 2][DD_MAXC];
+  __shared__ int rexp[OT_RING][TT_ROWS], fexp[OT_RING][DD_MAXC];
+  __shared__ int part_w[32], range[4];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const bool worker = warp < OZ_WARPS;
-  const int RC = a.g.RC, tps = a.tps;
-  const int ntot = a.g.nsub * tps;
-  const int f0 = (int)((long)blockIdx.x * ntot / gridDim.x);
-  const int f1 = (int)((long)(blockIdx.x + 1) * ntot / gridDim.x);
+  const int RC = a.g.RC, nsub = a.g.nsub;
   auto rows_of = [&](int k) { return a.spatial ? a.g.N[k] : a.g.n; };
-  auto next_valid = [&](int f) {
-    while (f < f1 && (f % tps) * TT_ROWS >= rows_of(f / tps)) ++f;
-    return f;
+  auto shape = [&](int k) {
+    OtShape s;
+    s.rows = rows_of(k);
+    s.ni = a.ninner ? a.ninner[k] : a.ninner_fix;
+    s.nc = a.ncols ? a.ncols[k] : a.ncols_fix;
+    s.KP = max(16, (s.ni + 15) & ~15);
+    s.nch = max(1, (s.nc + 15) >> 4);
+    s.row0 = a.spatial ? (long)a.g.rowoff[k] : (long)k * a.g.n;
+    return s;
   };
-  auto shape = [&](int f) {
-    OzTile t;
-    t.k = f / tps;
-    const int r0 = (f - t.k * tps) * TT_ROWS;
-    t.nrow = min(TT_ROWS, rows_of(t.k) - r0);
-    t.row0 = (a.spatial ? (long)a.g.rowoff[t.k] : (long)t.k * a.g.n) + r0;
-    t.ni = a.ninner ? a.ninner[t.k] : a.ninner_fix;
-    t.nc = a.ncols ? a.ncols[t.k] : a.ncols_fix;
-    t.N = t.nc <= 16 ? 16 : (t.nc + 15) / 16 * 16;
-    return t;
-  };
-  int f = next_valid(f0);
-  if (f >= f1) return;
+  // ---- this CTA's tiles: a contiguous range of (subdomain, tile) pairs of about equal cost,
+  // the tiles of subdomain k costing about 2 + KP / 16 + column chunks each (a conversion, an
+  // epilogue and the hand-over; subdomains of a batch differ in rank)
+  auto cost = [&](const OtShape& s) { return 2 + (s.KP >> 4) + s.nch; };
+  {
+    const int per = (nsub + 511) / 512, ka = min(nsub, tid * per), kb = tid < 512 ? min(nsub, ka + per) : ka;
+    int w = 0;
+    for (int k = ka; k < kb; ++k) {
+      const OtShape s = shape(k);
+      w += ((s.rows + TT_ROWS - 1) / TT_ROWS) * cost(s);
+    }
+    int inc = w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += t;
+    }
+    if (lane == 31) part_w[warp] = inc;
+    if (tid < 4) range[tid] = tid & 1 ? 0 : nsub;
+    __syncthreads();
+    int total = 0, before = 0;
+    for (int i = 0; i < 16; ++i) {
+      if (i < warp) before += part_w[i];
+      total += part_w[i];
+    }
+    const int lo = before + inc - w;                    // weight before subdomain ka
+    for (int side = 0; side < 2; ++side) {
+      // the first tile that starts at or after this side's share of the total
+      const int x = (int)((long)(blockIdx.x + side) * total / gridDim.x);
+      if (w > 0 && x >= lo && x < lo + w) {
+        int at = lo;
+        for (int k = ka; k < kb; ++k) {
+          const OtShape s = shape(k);
+          const int nt = (s.rows + TT_ROWS - 1) / TT_ROWS, wk = nt * cost(s);
+          if (x < at + wk) {
+            range[2 * side] = k;
+            range[2 * side + 1] = (x - at + cost(s) - 1) / cost(s);
+            break;
+          }
+          at += wk;
+        }
+      }
+    }
+  }
   if (tid == 0) {
-    tc::mbar_init(&bar_mma[0], 1);
-    tc::mbar_init(&bar_mma[1], 1);
+    for (int i = 0; i < 2; ++i) { tc::mbar_init(&full[i], OT_CONV); tc::mbar_init(&empty[i], 1); }
+    for (int i = 0; i < OT_NB; ++i) { tc::mbar_init(&tfull[i], 1); tc::mbar_init(&tempty[i], OT_EPI); }
+    for (int i = 0; i < OT_RING; ++i) tc::mbar_init(&meta[i], OT_CONV);
     tc::mbar_init_fence();
   }
-  if (warp == 0) tc::tmem_alloc(&tmem_s, 512);          // OZ_DIG accumulators of 64 columns
+  if (warp == 0) tc::tmem_alloc(&tmem_s, 512);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tmem_s;
+  const int k1 = range[2], j1 = range[3];
+  // walk over this CTA's tiles: (k, j), normalised to an existing tile or the end
+  auto settle = [&](int& k, int& j) {
+    while (k < nsub && j * TT_ROWS >= rows_of(k)) { ++k; j = 0; }
+    return k < k1 || (k == k1 && j < j1);
+  };
   bool alive = true;
-  // A stage is one pass of one tile: its digit planes go to buffer (stage & 1) and its MMAs
-  // commit to that buffer's barrier, completing that barrier's phase (stage >> 1).
-  int ns = 0, kcur = -1, tb = 0, prev_tb = 0;           // stages issued, tile parity (rexp)
-  bool pending = false;                                 // a tile's MMAs issued, epilogue not done
-  OzTile prev{};
-  auto wait_stage = [&](int j) {
-    alive = tc::mbar_wait(&bar_mma[j & 1], (j >> 1) & 1, kWait) && alive;
-  };
 
-  // epilogue of tile t (its MMAs complete; row bounds rexp[rb]), planes buffer b as scratch;
-  // worker warp w: TMEM lanes 32 (w % 4) .., 4-column groups w / 4, w / 4 + 4, ...
-  auto epilogue = [&](const OzTile& t, int rb, int b) {
-    const int q4 = warp & 3, m = q4 * 32 + lane;
-    const int er = rexp[rb][m];
-    double* ebuf = reinterpret_cast<double*>(asl0 + (size_t)b * ABUF) + warp * (32 * 5);
-    double* ybase = a.Y + t.row0 * a.ldy;
-    for (int c0 = (warp >> 2) * 4; c0 < t.N; c0 += 16) {
-      uint32_t D[OZ_DIG][4];
+  if (warp < OT_CONV) {
+    // ------------------------------------------------------------------ converters
+    const int rho = lane & 7, q = lane >> 3;
+    int k = range[0], j = range[1], kcur = -1, it = 0;
+    unsigned used[2] = {0, 0};
+    bool more = settle(k, j);
+    OtShape s = shape(min(k, nsub - 1));
+    const int r = 8 * warp + rho;                          // this lane's row of every tile
+    double2 x[8];
+    // (rows past the subdomain's read its last one; their results are not written)
+    auto load = [&](const OtShape& t, int jt) {
+      ot_load(x, a.A + (t.row0 + min(jt * TT_ROWS + r, t.rows - 1)) * a.lda, q, a.lda, t.KP);
+    };
+    if (more && tid == 0)
+      prefetch_rows(a.A, a.lda, s.row0 + (long)j * TT_ROWS, OT_AHEAD * TT_ROWS, a.nrows);
+    if (more) load(s, j);
+    uint8_t* asl0 = msl;
+    uint32_t APL = 0;
+    while (more) {
+      const int nst = s.KP <= 48 ? 2 : 1;
+      if (k != kcur) {
+        // ---- M's digit planes, once per subdomain.  The MMAs that read the old ones (and the
+        // stages, used as scratch here) are complete first; all converters agree on going on.
+        for (int b = 0; b < 2; ++b)
+          if (used[b] && alive) alive = tc::mbar_wait(&empty[b], (used[b] - 1) & 1, kWait);
+        alive = ot_conv_all(alive);
+        if (!alive) break;
+        kcur = k;
+        APL = TT_ROWS * 2 * s.KP;
+        asl0 = msl + (size_t)s.nch * 16 * OZ_DIG * 2 * s.KP;
+        const double* Mk = a.bsmall >= 0 ? a.smbase + ((long)k * NSMALL + a.bsmall) * RC * RC
+                                         : a.Bm + (long)k * RC * RC;
+        double* Ms = reinterpret_cast<double*>(asl0);     // [kk][DD_MAXC]
 #pragma unroll
-      for (int g = 0; g < OZ_DIG; ++g)
-        oz_tmem_ld4(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(g * t.N + c0), D[g]);
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-      for (int g = 0; g < OZ_DIG; ++g)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) asm volatile("" : "+r"(D[g][j]));
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int c = c0 + j;
-        double v = 0.0;
-        if (c < t.nc && m < t.nrow && alive) {
-          long long J = 0;
-#pragma unroll
-          for (int g = 0; g < OZ_DIG - 1; ++g)
-            J += (long long)__float2int_rn(__uint_as_float(D[g][j])) << (40 - 8 * g);
-          J += (long long)(__float2int_rn(__uint_as_float(D[OZ_DIG - 1][j])) >> 8);
-          v = oz_to_f64(J, er + fexp[c] - 56);
+        for (int i = 0; i < DD_MAXC * DD_MAXC / (OT_CONV * 32); ++i) {
+          const int e = tid + OT_CONV * 32 * i, kk = e >> 6, n = e & (DD_MAXC - 1);
+          if (kk < s.KP)
+            Ms[e] = (kk < s.ni && n < s.nc)
+                        ? __ldg(Mk + (a.mtrans ? (long)n * RC + kk : (long)kk * RC + n)) : 0.0;
         }
-        ebuf[lane * 5 + j] = v;
-      }
-      __syncwarp();
-      const int cc = c0 + (lane & 3);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int rl = 8 * i + (lane >> 2), rr = q4 * 32 + rl;
-        if (rr < t.nrow && cc < a.ldy) {
-          double* yp = ybase + (long)rr * a.ldy + cc;
-          if (!a.accumulate) *yp = ebuf[rl * 5 + (lane & 3)];
-          else if (cc < t.nc) *yp += (a.rowscale ? a.rowscale[t.row0 + rr] : 1.0) * ebuf[rl * 5 + (lane & 3)];
+        ot_conv_sync();
+        for (int kk = warp; kk < s.KP; kk += OT_CONV) {    // mu_k: warp per row
+          const int E0 = f64_bexp(Ms[kk * DD_MAXC + lane]), E1 = f64_bexp(Ms[kk * DD_MAXC + lane + 32]);
+          const int mx = __reduce_max_sync(0xffffffffu, max(E0 ? E0 - 1022 : OZ_NONE, E1 ? E1 - 1022 : OZ_NONE));
+          if (lane == 0) mexp[kk] = mx;
         }
-      }
-      __syncwarp();
-    }
-    if (warp < 4 && a.ldy > t.N && !a.accumulate)       // columns N .. ldy - 1
-      for (int e = lane; e < 32 * (a.ldy - t.N); e += 32) {
-        const int rr = q4 * 32 + e / (a.ldy - t.N), c = t.N + e % (a.ldy - t.N);
-        if (rr < t.nrow) ybase[(long)rr * a.ldy + c] = 0.0;
-      }
-  };
-  auto finish_prev = [&]() {          // wait for prev's MMAs (its last stage), its epilogue
-    wait_stage(ns - 1);
-    tc::fence_after_sync();
-    if (worker) epilogue(prev, prev_tb, (ns - 1) & 1);
-    tc::fence_before_sync();
-    alive = __syncthreads_and(alive) != 0;
-    pending = false;
-  };
-  // MMAs of tile t, K range k0 .. k0 + KA - 1 of its planes in buffer b.  M's planes are
-  // stacked along N (plane u = rows u N .. u N + N - 1) and accumulator g sits at TMEM
-  // columns g N .., so one MMA of A's plane s with planes u0 .. u0 + nu - 1 adds the pairs
-  // (s, u) into accumulators s + u0 .. s + u0 + nu - 1: at most 256 / N planes an MMA
-  auto issue = [&](const OzTile& t, int b, int k0, int acc0) {
-    tc::fence_after_sync();
-    const int ns = max(k0 == 0 ? 1 : 0, (min(t.ni, k0 + KA) - k0 + 15) >> 4);
-    const int nper = 256 / t.N;
-    const uint32_t MPLt = (uint32_t)t.N * 2 * KP;
-    const uint64_t ad0 = tc::sdesc(tc::smem_u32(asl0 + (size_t)b * ABUF), 128, 16 * KA);
-    const uint64_t bd0 = tc::sdesc(tc::smem_u32(msl) + 256 * (k0 / 16), 128, 16 * KP);
-    for (int j = 0; j < ns; ++j)
-      for (int s1 = 0; s1 < OZ_DIG; ++s1)
-        for (int u0 = 0; u0 < OZ_DIG - s1; u0 += nper) {
-          const int nu = min(nper, OZ_DIG - s1 - u0);
-          tc::mma_bf16(tmem + (uint32_t)((s1 + u0) * t.N), ad0 + ((s1 * APL + 256 * j) >> 4),
-                       bd0 + ((u0 * MPLt + 256 * j) >> 4), tc::idesc(tc::FMT_BF16, 128, nu * t.N),
-                       (acc0 || j > 0 || s1 > 0) ? 1u : 0u);
+        ot_conv_sync();
+        {                                                  // f_n: OT_CONV / 2 threads per column
+          const int n = tid & (DD_MAXC - 1), p = tid >> 6;
+          int mx = OZ_NONE;
+          for (int kk = p; kk < s.ni; kk += OT_CONV / 2) {
+            const int E = f64_bexp(Ms[kk * DD_MAXC + n]);
+            if (E) mx = max(mx, E - 1022 - mexp[kk]);
+          }
+          red[p][n] = mx;
         }
-    tc::mma_commit(&bar_mma[b]);
-  };
-
-  const int rho = lane & 7, q = lane >> 3, r = 8 * warp + rho;
-  double2 x[8];                                          // the warp's rows of the tile
-  OzTile t = shape(f);
-  if (worker) oz_load_rows(x, a.A, a.lda, t, r, q, KP);
-  while (alive) {
-    count_work(a.g, KS_OZ_TALL, 2.0 * t.nrow * t.ni * t.nc);
-    if (t.k != kcur) {
-      if (pending) finish_prev();                       // its MMAs read the old M planes
-      if (!alive) break;
-      // ---- M's digit planes, once per subdomain: M staged as FP64 [kk][DD_MAXC] in the
-      // (free) first planes buffer by coalesced loads, then bounds and digits from there
-      kcur = t.k;
-      const double* Mk = a.bsmall >= 0 ? a.smbase + ((long)t.k * NSMALL + a.bsmall) * RC * RC
-                                       : a.Bm + (long)t.k * RC * RC;
-      double* Ms = reinterpret_cast<double*>(asl0);
+        ot_conv_sync();
+        if (tid < DD_MAXC) {
+          int mx = red[0][tid];
 #pragma unroll
-      for (int i = 0; i < DD_MAXC * DD_MAXC / OZ_WORKERS; ++i) {
-        const int e = tid + OZ_WORKERS * i, kk = e >> 6, n = e & (DD_MAXC - 1);
-        if (worker && kk < KP)
-          Ms[e] = (kk < t.ni && n < t.nc)
-                      ? __ldg(Mk + (a.mtrans ? (long)n * RC + kk : (long)kk * RC + n)) : 0.0;
-      }
-      __syncthreads();
-      for (int kk = worker ? warp : KP; kk < KP; kk += OZ_WARPS) {   // mu_k: warp per row
-        int mx = OZ_NONE;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int E = f64_bexp(Ms[kk * DD_MAXC + lane + 32 * h]);
-          if (E) mx = max(mx, E - 1022);
+          for (int p = 1; p < OT_CONV / 2; ++p) mx = max(mx, red[p][tid]);
+          fnow[tid] = mx;
         }
-        mx = __reduce_max_sync(0xffffffffu, mx);
-        if (lane == 0) mexp[kk] = mx;
-      }
-      __syncthreads();
-      if (worker) {                                     // f_n: 8 threads per column
-        const int n = tid & (DD_MAXC - 1), q = tid >> 6;
-        int mx = OZ_NONE;
-        for (int kk = q; kk < t.ni; kk += 8) {
-          const int E = f64_bexp(Ms[kk * DD_MAXC + n]);
-          if (E) mx = max(mx, E - 1022 - mexp[kk]);
+        ot_conv_sync();
+        // digits of M'[kk][n] relative to 2^f_n, two adjacent kk per lane, 8 n x 4 pairs per warp
+        const int kb = s.KP >> 3;
+        for (int blk = warp; blk < s.nch * 2 * kb; blk += OT_CONV) {
+          const int n = (blk / kb) * 8 + rho, kk = ((blk % kb) * 4 + q) * 2;
+          uint32_t w[OZ_DIG];
+          oz_digits2(Ms[kk * DD_MAXC + n], fnow[n] + mexp[kk], Ms[(kk + 1) * DD_MAXC + n],
+                     fnow[n] + mexp[kk + 1], w);
+          const int r0 = (n >> 4) * (16 * OZ_DIG) + (n & 15);
+#pragma unroll
+          for (int u = 0; u < OZ_DIG; ++u)
+            *reinterpret_cast<uint32_t*>(msl + tc::op_off(r0 + 16 * u, kk * 2, 2 * s.KP)) = w[u];
         }
-        red[q][n] = mx;
+        tc::fence_async_smem();
+        ot_conv_sync();                                    // Ms is read before the digits below
       }
-      __syncthreads();
-      if (tid < DD_MAXC) {
-        int mx = red[0][tid];
-#pragma unroll
-        for (int q = 1; q < 8; ++q) mx = max(mx, red[q][tid]);
-        fexp[tid] = mx;
-      }
-      __syncthreads();
-      // digits of M'[kk][n] relative to 2^f_n, two adjacent kk per thread; plane u holds
-      // rows u N + n
-      const uint32_t MPLt = (uint32_t)t.N * 2 * KP;
-      for (int e = worker ? tid : t.N * (KP / 2); e < t.N * (KP / 2); e += OZ_WORKERS) {
-        const int n = e / (KP / 2), kk = 2 * (e - n * (KP / 2));
-        const double m0 = Ms[kk * DD_MAXC + n], m1 = Ms[(kk + 1) * DD_MAXC + n];
-        float d0[OZ_DIG], d1[OZ_DIG];
-        oz_digits(m0, fexp[n] + mexp[kk], d0);
-        oz_digits(m1, fexp[n] + mexp[kk + 1], d1);
-        const uint32_t off = tc::op_off(n, kk * 2, 2 * KP);
-#pragma unroll
-        for (int u = 0; u < OZ_DIG; ++u)
-          *reinterpret_cast<uint32_t*>(msl + u * MPLt + off) = oz_pack(d0[u], d1[u]);
-      }
-      __syncthreads();
-    }
-    // ---- the tile's rows (loaded during the previous tile): row bounds, digit planes
-    int mx = OZ_NONE;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const int kk = 8 * c + 2 * q;
-      if (worker && c < KP / 8 && kk < t.ni) {
-        const int E0 = f64_bexp(x[c].x), E1 = f64_bexp(x[c].y);
-        if (E0 && mexp[kk] != OZ_NONE) mx = max(mx, E0 - 1022 + mexp[kk]);
-        if (E1 && kk + 1 < t.ni && mexp[kk + 1] != OZ_NONE) mx = max(mx, E1 - 1022 + mexp[kk + 1]);
-      }
-    }
-    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
-    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
-    if (worker && q == 0) rexp[tb][r] = mx;
-    const int fn = next_valid(f + 1);
-    const OzTile tn = fn < f1 ? shape(fn) : t;
-    for (int p = 0; p < npass; ++p) {
-      const int k0 = p * KA, buf = ns & 1;
-      if (ns >= 2) wait_stage(ns - 2);                  // the buffer's previous stage is read
-      uint8_t* asl = asl0 + (size_t)buf * ABUF;
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const int kk = 8 * c + 2 * q;
-        if (worker && c < KP / 8 && kk >= k0 && kk < k0 + KA) {
-          // entries past ni, or whose row of M is zero, are zero (their digits too)
-          const double x0 = (kk < t.ni && mexp[kk] != OZ_NONE) ? x[c].x : 0.0;
-          const double x1 = (kk + 1 < t.ni && mexp[kk + 1] != OZ_NONE) ? x[c].y : 0.0;
-          float d0[OZ_DIG], d1[OZ_DIG];
-          oz_digits(x0, mx - mexp[kk], d0);
-          oz_digits(x1, mx - mexp[min(kk + 1, DD_MAXC - 1)], d1);
-          const uint32_t off = tc::op_off(r, (kk - k0) * 2, 2 * KA);
-#pragma unroll
-          for (int s = 0; s < OZ_DIG; ++s)
-            *reinterpret_cast<uint32_t*>(asl + s * APL + off) = oz_pack(d0[s], d1[s]);
-        }
-      }
-      if (worker && p == npass - 1 && fn < f1) oz_load_rows(x, a.A, a.lda, tn, r, q, KP);
+      if (a.g.work) count_work(a.g, KS_OZ_TALL, 2.0 * min(TT_ROWS, s.rows - j * TT_ROWS) * s.ni * s.nc);
+      const int b = nst == 2 ? it & 1 : 0, slot = it & (OT_RING - 1);
+      // (the rows of consecutive tiles follow each other in memory, across subdomains too)
+      if (tid == 0) prefetch_rows(a.A, a.lda, s.row0 + (long)(j + OT_AHEAD) * TT_ROWS, TT_ROWS, a.nrows);
+      if (used[b] && alive) alive = tc::mbar_wait(&empty[b], (used[b] - 1) & 1, kWait);
+      // the next tile
+      int kn = k, jn = j + 1;
+      more = settle(kn, jn);
+      const OtShape sn = (more && kn != k) ? shape(kn) : s;
+      uint8_t* asl = asl0 + (size_t)b * OZ_DIG * APL;
+      if (tid < DD_MAXC) fexp[slot][tid] = fnow[tid];
+      if (s.KP <= 16) ot_convert<2>(x, mexp, s.ni, q, r, asl, APL, rexp[slot]);
+      else if (s.KP <= 32) ot_convert<4>(x, mexp, s.ni, q, r, asl, APL, rexp[slot]);
+      else if (s.KP <= 48) ot_convert<6>(x, mexp, s.ni, q, r, asl, APL, rexp[slot]);
+      else ot_convert<8>(x, mexp, s.ni, q, r, asl, APL, rexp[slot]);
+      if (more) load(sn, jn);                              // under the fence and the next wait
       tc::fence_async_smem();
-      alive = __syncthreads_and(alive) != 0;
-      if (alive && p == 0 && pending) finish_prev();    // overlapped with the previous MMAs
-      if (!alive) break;
-      if (tid == OZ_WORKERS) issue(t, buf, k0, p > 0);   // the issuing warp
-      ++ns;
       __syncwarp();
+      if (lane == 0) {
+        tc::mbar_arrive(&meta[slot]);
+        tc::mbar_arrive(&full[b]);
+      }
+      ++used[b];
+      ++it;
+      k = kn;
+      j = jn;
+      s = sn;
     }
-    if (!alive) break;
-    pending = true;
-    prev = t;
-    prev_tb = tb;
-    tb ^= 1;
-    if (fn >= f1) break;
-    f = fn;
-    t = tn;
-  }
-  if (pending && alive) finish_prev();
-  if (!alive) {
-    if (tid == 0) atomicOr(a.status, (unsigned)ST_TIMEOUT);
-    if (ns > 0) tc::mbar_wait(&bar_mma[(ns - 1) & 1], ((ns - 1) >> 1) & 1, kWait);   // in flight
-  }
-  __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, 512);
-}
-
-// ---------------------------------------------------------------------------------------
-// FP64-accurate symmetric Gram partials on the BF16 tensor cores (Ozaki scheme)
-// ---------------------------------------------------------------------------------------
-// G_c = A_c^T A_c over a chunk of rows, with the chunks and the output of k_gram: one
-// RC x RC partial per (subdomain, chunk), zero outside the ma x ma block; with chunk
-// exponents, the Gram of 2^-e A_c (e = the chunk's scale when it is far from 1; INT_MIN for a
-// chunk below 2^-1000).  A pre-pass over the chunk's rows bounds every column i by 2^c_i;
-// the values become 7 balanced base-256 digits relative to 2^(c_i + 1) (as for the tall
-// products, one bit higher, so that every digit, the leading one included, is in
-// [-128, 128]), and the chunk's rows are taken in stages of 64 (double-buffered digit
-// planes of A'^T, the K dimension of the stage's MMAs).
-// The M = 128 A operand of an MMA starting at plane s1 covers h = 128 / P consecutive
-// planes (P = the padded column count): lanes u P .. u P + P - 1 ("band" u) hold plane
-// s1 + u.  One MMA per s1 in {0, h, 2h, ..} with the B operand's planes t = 0 .. 6 - s1
-// stacked along N (accumulator column block s1 + t) therefore serves every band at once:
-// in band u, column block c accumulates the digit pairs (s, t) of order s + t = c + u.
-// At most 4 pairs of products <= 2^14 meet in one band's block, so 128 rows (two stages)
-// stay below 2^24 and exact in FP32: the accumulators are read out every two stages.  The
-// read-out combines each band's blocks in 64-bit integers (< 2^62), exchanges the bands
-// through the free plane buffer (rows padded to P + 1 entries), sums them in a fixed order and adds the result, made FP64
-// with the chunk's column scales, to per-thread FP64 accumulators (thread t owns the
-// upper-triangle entries t + 512 m of the P x P block); a chunk's partial is written after
-// its last read-out.  Persistent CTAs (one per SM: 16 worker warps, one MMA-issue warp)
-// walk the (subdomain, chunk) items.
-#define OG_KS 64                          // rows per stage (K of one stage's MMAs)
-#define OG_RO 2                           // stages per read-out (128 rows)
-#define OG_PAD (128 * 2 * OG_KS)          // the M = 128 A operand reads past the last plane
-
-struct OzGram {
-  Geo g;
-  int spatial;
-  const double* A; int lda;
-  const int* acnt;
-  double* part; int nchunk;
-  int* cexp;
-  unsigned* status;
-};
-
-// dynamic shared memory of k_oz_gram for a column capacity RC <= DD_MAXC: two plane buffers
-// (and the alignment slack); at most 147.6 KB, beside 5.2 KB of static shared memory
-static size_t og_smem(int RC) {
-  const int PMAX = (RC + 15) / 16 * 16;
-  return 128 + 2 * ((size_t)OZ_DIG * PMAX * 2 * OG_KS + OG_PAD);
-}
-
-// what a read-out needs to know
-struct OgGroup {
-  int k, c, ma, P, ex, last, cp;
-};
-
-__global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gram(OzGram a) {
-  extern __shared__ uint8_t raw_og[];
-  uint8_t* buf0 = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw_og) + 127) &
-                                             ~uintptr_t(127));
-  const int RC = a.g.RC, PMAX = (RC + 15) / 16 * 16;
-  const uint32_t BUF = OZ_DIG * PMAX * 2 * OG_KS + OG_PAD;
-  __shared__ uint64_t bar_mma[2];
-  __shared__ uint32_t tmem_s;
-  __shared__ int cs[2][DD_MAXC];                 // column bound exponents (item parity)
-  __shared__ long long cred[8][DD_MAXC];
-  __shared__ long long cmb[DD_MAXC];             // column maxima (bits) of the item
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const bool worker = warp < OZ_WARPS;
-  const int nitems = a.g.nsub * a.nchunk;
-  if ((int)blockIdx.x >= nitems) return;
-  if (tid == 0) {
-    tc::mbar_init(&bar_mma[0], 1);
-    tc::mbar_init(&bar_mma[1], 1);
-    tc::mbar_init_fence();
-  }
-  if (warp == 0) tc::tmem_alloc(&tmem_s, 512);   // OZ_DIG column blocks of up to 64 columns
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = tmem_s;
-  bool alive = true;
-  int ns = 0;                                    // stages issued
-  int gs = 0;                                    // stages in the open read-out group
-  int cp = 0;                                    // item parity (cs)
-  bool pending = false;                          // a closed group not yet read out
-  OgGroup prev{};
-  double acc[8];
+  } else if (warp < OT_CONV + OT_EPI) {
+    // ------------------------------------------------------------------ epilogue
+    const int q4 = warp & 3, half = (warp - OT_CONV) >> 2, m = q4 * 32 + lane;
+    int k = range[0], j = range[1], kcur = -1, it = 0, qc = 0;
+    OtShape s{};
+    const bool wide = (a.ldy & 3) == 0;
+    while (alive && settle(k, j)) {
+      if (k != kcur) { s = shape(k); kcur = k; }
+      const int slot = it & (OT_RING - 1), r = j * TT_ROWS + m;
+      const bool in = r < s.rows;
+      double* yr = a.Y + (s.row0 + r) * a.ldy;
+      alive = __all_sync(0xffffffffu, tc::mbar_wait(&meta[slot], (it / OT_RING) & 1, kWait));
+      const int er = rexp[slot][m];
+      const double rs = (a.accumulate && a.rowscale && in) ? a.rowscale[s.row0 + r] : 1.0;
+      for (int c = 0; c < s.nch && alive; ++c, ++qc) {
+        const int buf = qc & (OT_NB - 1);
+        int c0 = 16 * c + 8 * half;
+        alive = __all_sync(0xffffffffu, tc::mbar_wait(&tfull[buf], (qc / OT_NB) & 1, kWait));
+        if (!alive) break;
+        tc::fence_after_sync();
+        const int lim = a.zfill ? a.ldy : s.nc;            // columns written
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h, c0 += 4) {
+          __syncwarp();                                    // (lanes past the last row came early)
+          uint32_t D[OZ_DIG][4];
 #pragma unroll
-  for (int m = 0; m < 8; ++m) acc[m] = 0.0;
-  auto wait_stage = [&](int j) {
-    alive = tc::mbar_wait(&bar_mma[j & 1], (j >> 1) & 1, kWait) && alive;
-  };
-  // read out the closed group prev (its MMAs complete) into acc; write the chunk's partial
-  // after its last group.  Scratch: the planes buffer of the group's last stage.
-  auto readout = [&]() {
-    wait_stage(ns - 1);
-    tc::fence_after_sync();
-    const int P = prev.P, h = 128 / P, nb = h < OZ_DIG ? h : OZ_DIG;
-    long long* X = reinterpret_cast<long long*>(buf0 + (size_t)((ns - 1) & 1) * BUF);
-    if (worker) {
-      // worker warp w: TMEM lanes 32 (w % 4) .. (band u = lane / P, row i), 4-column groups
-      // 4 (w / 4) + 16 t
-      const int q4 = warp & 3, L = q4 * 32 + lane, u = L / P, i = L - u * P;
-      const bool lv = u < nb && i < prev.ma;
+          for (int g = 0; g < OZ_DIG; ++g)
+            oz_tmem_ld4(tmem + ((uint32_t)(q4 * 32) << 16) +
+                            (uint32_t)(128 * buf + 16 * g + 8 * half + 4 * h), D[g]);
+          double2 o[2];
+          if (a.accumulate && in) {                        // Y's entries
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const int c0 = 4 * (warp >> 2) + 16 * t;
-        if (c0 >= P) continue;                   // warp-uniform
-        uint32_t D[OZ_DIG][4];
+            for (int i = 0; i < 2; ++i)
+              o[i] = *reinterpret_cast<const double2*>(yr + min(c0 + 2 * i, a.ldy - 2));
+          }
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-        for (int c = 0; c < OZ_DIG; ++c)
-          oz_tmem_ld4(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(c * P + c0), D[c]);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          for (int g = 0; g < OZ_DIG; ++g)
 #pragma unroll
-        for (int c = 0; c < OZ_DIG; ++c)
+            for (int i = 0; i < 4; ++i) asm volatile("" : "+r"(D[g][i]));
+          if (h == 1) {                                    // the buffer is free again
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&tempty[buf]);
+          }
+          double v[4];
 #pragma unroll
-          for (int jj = 0; jj < 4; ++jj) asm volatile("" : "+r"(D[c][jj]));
+          for (int i = 0; i < 4; ++i) {
+            v[i] = oz_round(oz_combine(&D[0][i], 4), er + fexp[slot][c0 + i] - 56);
+            if (c0 + i >= s.nc) v[i] = 0.0;
+          }
+          if (!in) continue;
+          double* yp = yr + c0;
+          if (a.accumulate) {
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-          const int j = c0 + jj;
-          if (lv && j < prev.ma && j >= i) {
-            long long J = 0;
-#pragma unroll
-            for (int c = 0; c < OZ_DIG; ++c) {
-              const int g = c + u;                 // the digit order this block holds
-              const int d = __float2int_rn(__uint_as_float(D[c][jj]));
-              if (g < OZ_DIG - 1) J += (long long)d << (40 - 8 * g);
-              else if (g == OZ_DIG - 1) J += (long long)(d >> 8);
+            for (int i = 0; i < 2; ++i) {
+              v[2 * i] = fma(rs, v[2 * i], o[i].x);
+              v[2 * i + 1] = fma(rs, v[2 * i + 1], o[i].y);
             }
-            X[(u * P + i) * (P + 1) + j] = J;
+          }
+          if (c0 + 4 <= lim) {
+            if (wide) {
+              asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(yp), "d"(v[0]), "d"(v[1]),
+                           "d"(v[2]), "d"(v[3])
+                           : "memory");
+            } else {
+              *reinterpret_cast<double2*>(yp) = make_double2(v[0], v[1]);
+              *reinterpret_cast<double2*>(yp + 2) = make_double2(v[2], v[3]);
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (c0 + i < lim) yp[i] = v[i];
           }
         }
       }
+      if (alive && a.zfill && in)                          // columns 16 nch .. ldy - 1
+        for (int c = 16 * s.nch + 2 * half; c < a.ldy; c += 4)
+          *reinterpret_cast<double2*>(yr + c) = make_double2(0.0, 0.0);
+      ++it;
+      ++j;
     }
-    __syncthreads();
-    if (worker && alive) {
-      const int* csr = cs[prev.cp];
-#pragma unroll
-      for (int m = 0; m < 8; ++m) {
-        const int e = tid + OZ_WORKERS * m, i = e / P, j = e - i * P;
-        if (e < P * P && i < prev.ma && j < prev.ma && j >= i) {
-          long long J = 0;
-          for (int u = 0; u < nb; ++u) J += X[(u * P + i) * (P + 1) + j];
-          acc[m] += oz_to_f64(J, csr[i] + csr[j] + 2 - 56 - 2 * prev.ex);
-        }
-      }
-    }
-    if (prev.last && worker) {
-      double* out = a.part + ((long)prev.k * a.nchunk + prev.c) * RC * RC;
-#pragma unroll
-      for (int m = 0; m < 8; ++m) {
-        const int e = tid + OZ_WORKERS * m, i = e / P, j = e - i * P;
-        if (e < P * P && i < prev.ma && j < prev.ma && j >= i) {
-          out[i * RC + j] = acc[m];
-          out[j * RC + i] = acc[m];
-        }
-        acc[m] = 0.0;
-      }
-      for (int e = tid; e < RC * RC; e += OZ_WORKERS) {
-        const int r = e / RC, cc = e - r * RC;
-        if (r >= prev.ma || cc >= prev.ma) out[e] = 0.0;
-      }
-    }
-    tc::fence_before_sync();
-    alive = __syncthreads_and(alive) != 0;
-    pending = false;
-  };
-  // MMAs of one stage from plane buffer b (planes of P rows): for s1 = 0, h, 2h, .. the
-  // A operand is planes s1 .. s1 + h - 1 (one per band; past the last plane it reads junk
-  // into blocks never read out), the B operand planes u0 .. u0 + nu - 1 (u0 + nu <= 7 - s1)
-  // stacked along N into column blocks s1 + u0 ..
-  auto issue = [&](int b, int P, bool first) {
-    tc::fence_after_sync();
-    const int nper = 256 / P, h = 128 / P;
-    const uint32_t PL = (uint32_t)P * 2 * OG_KS;
-    const uint64_t d0 = tc::sdesc(tc::smem_u32(buf0 + (size_t)b * BUF), 128, 16 * OG_KS);
-    for (int j = 0; j < OG_KS / 16; ++j)
-      for (int s1 = 0; s1 < OZ_DIG; s1 += h)
-        for (int u0 = 0; u0 < OZ_DIG - s1; u0 += nper) {
-          const int nu = min(nper, OZ_DIG - s1 - u0);
-          tc::mma_bf16(tmem + (uint32_t)((s1 + u0) * P), d0 + ((s1 * PL + 256 * j) >> 4),
-                       d0 + ((u0 * PL + 256 * j) >> 4), tc::idesc(tc::FMT_BF16, 128, nu * P),
-                       (!first || j > 0 || s1 > 0) ? 1u : 0u);
-        }
-    tc::mma_commit(&bar_mma[b]);
-  };
-
-  for (int w = blockIdx.x; w < nitems && alive; w += gridDim.x) {
-    const int k = w / a.nchunk, c = w - k * a.nchunk;
-    const int rows = a.spatial ? a.g.N[k] : a.g.n;
-    const long rb = a.spatial ? (long)a.g.rowoff[k] : (long)k * a.g.n;
-    const int ch = (rows + a.nchunk - 1) / a.nchunk;
-    const int i0 = min(rows, c * ch), i1 = min(rows, i0 + ch);
-    const int ma = a.acnt[k], P = ma <= 16 ? 16 : (ma + 15) / 16 * 16;
-    // ---- pre-pass: column bounds (largest |entry| of each column on the integer order of
-    // its bits; non-finite entries other than infinities are left out) and the chunk scale,
-    // into the parity cn of cs (a pending read-out of the previous item uses parity cp)
-    const int ci = tid & 63, rg = tid >> 6, cn = cp ^ 1;
-    {
-      long long mb = 0;
-      if (worker && ci < ma)
-        for (int row = i0 + rg; row < i1; row += 8) {
-          const long long bits =
-              __double_as_longlong(a.A[(rb + row) * a.lda + ci]) & 0x7fffffffffffffffll;
-          if (bits <= 0x7ff0000000000000ll) mb = max(mb, bits);
-        }
-      if (worker) cred[rg][ci] = mb;
-    }
-    __syncthreads();
-    if (tid < DD_MAXC) {
-      long long m2 = cred[0][tid];
-#pragma unroll
-      for (int r = 1; r < 8; ++r) m2 = max(m2, cred[r][tid]);
-      const int E = (int)((unsigned long long)m2 >> 52);
-      cs[cn][tid] = E ? E - 1022 : OZ_NONE;
-      cmb[tid] = tid < ma ? m2 : 0;
-    }
-    __syncthreads();                              // cred is read before the next item's writes
-    int ex = 0;
-    bool zero = ma == 0 || i1 <= i0;
-    if (a.cexp) {
-      long long cmx = 0;                          // the chunk's largest |entry|
-      for (int q = 0; q < DD_MAXC; ++q) cmx = max(cmx, cmb[q]);
-      const double mx = __longlong_as_double(cmx);
-      const int e0 = (mx > 0.0 && isfinite(mx)) ? ilogb(mx) : 0;
-      zero = zero || !(mx > 0.0) || e0 < -1000;
-      ex = (!zero && (e0 < -400 || e0 > 400)) ? e0 : 0;
-      if (tid == 0) a.cexp[(long)k * a.nchunk + c] = zero ? INT_MIN : ex;
-    }
-    if (zero) {                                   // an all-zero partial, no stages
-      double* out = a.part + ((long)k * a.nchunk + c) * RC * RC;
-      for (int e = tid; e < RC * RC; e += OZ_THREADS) out[e] = 0.0;
-      continue;
-    }
-    cp = cn;
-    count_work(a.g, KS_OZ_GRAM, 2.0 * (i1 - i0) * (ma * (ma + 1) / 2));
-    const int nst = (i1 - i0 + OG_KS - 1) / OG_KS;
-    const int e1 = cs[cp][ci] + 1;                // this thread's column: digits relative to 2^e1
-    for (int sgi = 0; sgi < nst; ++sgi) {
-      const int r0 = i0 + sgi * OG_KS, b = ns & 1;
-      // ---- loads: thread (column ci, row pairs tid / 64 + 8 t)
-      double2 x[4];
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const int rp = rg + 8 * t, r = r0 + 2 * rp;
-        x[t] = make_double2(0.0, 0.0);
-        if (worker && ci < ma) {
-          if (r < i1) x[t].x = __ldg(a.A + (rb + r) * a.lda + ci);
-          if (r + 1 < i1) x[t].y = __ldg(a.A + (rb + r + 1) * a.lda + ci);
-        }
-      }
-      if (ns >= 2) wait_stage(ns - 2);           // buffer b's previous stage is done
-      // ---- digit planes: element (i, r) of A'^T at op_off(i, 2 (r - r0), 2 OG_KS)
-      if (worker && ci < ma) {
-        uint8_t* pl = buf0 + (size_t)b * BUF;
-        const uint32_t PL = (uint32_t)P * 2 * OG_KS;
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          const int rp = rg + 8 * t;
-          float d0[OZ_DIG], d1[OZ_DIG];
-          oz_digits(x[t].x, e1, d0);
-          oz_digits(x[t].y, e1, d1);
-          const uint32_t off = tc::op_off(ci, rp * 4, 2 * OG_KS);
-#pragma unroll
-          for (int s = 0; s < OZ_DIG; ++s)
-            *reinterpret_cast<uint32_t*>(pl + s * PL + off) = oz_pack(d0[s], d1[s]);
-        }
-      }
-      tc::fence_async_smem();
-      alive = __syncthreads_and(alive) != 0;
-      if (alive && pending) readout();            // the closed group's MMAs, under this conversion
+  } else if (lane == 0) {
+    // ------------------------------------------------------------------ MMA issue
+    int k = range[0], j = range[1], kcur = -1, it = 0, qc = 0;
+    unsigned used[2] = {0, 0};
+    OtShape s{};
+    while (alive && settle(k, j)) {
+      if (k != kcur) { s = shape(k); kcur = k; }
+      const int b = s.KP <= 48 ? it & 1 : 0;
+      alive = tc::mbar_wait(&full[b], used[b] & 1, kWait);
       if (!alive) break;
-      if (tid == OZ_WORKERS) issue(b, P, gs == 0);
-      ++ns;
-      ++gs;
-      if (gs == OG_RO || sgi == nst - 1) {       // close the group
-        pending = true;
-        prev.k = k; prev.c = c; prev.ma = ma; prev.P = P; prev.ex = ex; prev.cp = cp;
-        prev.last = sgi == nst - 1;
-        gs = 0;
+      tc::fence_after_sync();
+      const uint32_t APL = TT_ROWS * 2 * s.KP, MB = 16 * OZ_DIG * 2 * s.KP;
+      const uint64_t ad0 = tc::sdesc(tc::smem_u32(msl + (size_t)s.nch * MB + (size_t)b * OZ_DIG * APL),
+                                     128, 16 * s.KP);
+      const uint64_t bd0 = tc::sdesc(tc::smem_u32(msl), 128, 16 * s.KP);
+      const int nslab = s.KP >> 4;
+      for (int c = 0; c < s.nch && alive; ++c, ++qc) {
+        const int buf = qc & (OT_NB - 1);
+        if (qc >= OT_NB) {
+          alive = tc::mbar_wait(&tempty[buf], (qc / OT_NB - 1) & 1, kWait);
+          if (!alive) break;
+          tc::fence_after_sync();
+        }
+        for (int sl = 0; sl < nslab; ++sl)
+#pragma unroll
+          for (int d = 0; d < OZ_DIG; ++d)
+            tc::mma_bf16(tmem + (uint32_t)(128 * buf + 16 * d), ad0 + ((d * APL + 256 * sl) >> 4),
+                         bd0 + ((c * MB + 256 * sl) >> 4),
+                         tc::idesc(tc::FMT_BF16, 128, 16 * (OZ_DIG - d)), (sl > 0 || d > 0) ? 1u : 0u);
+        tc::mma_commit(&tfull[buf]);
       }
-      __syncwarp();
+      if (!alive) break;
+      tc::mma_commit(&empty[b]);
+      ++used[b];
+      ++it;
+      ++j;
     }
+    // nothing of this CTA's MMAs is in flight when its memory goes back: the last commit of
+    // each stage has arrived
+    for (int b = 0; b < 2; ++b)
+      if (used[b]) alive = tc::mbar_wait(&empty[b], (used[b] - 1) & 1, kWait) && alive;
   }
-  if (pending && alive) readout();
-  if (!alive) {
-    if (tid == 0) atomicOr(a.status, (unsigned)ST_TIMEOUT);
-    if (ns > 0) tc::mbar_wait(&bar_mma[(ns - 1) & 1], ((ns - 1) >> 1) & 1, kWait);
-  }
+  if (!alive && lane == 0) atomicOr(a.status, (unsigned)ST_TIMEOUT);
+  __syncwarp();
+  tc::fence_before_sync();
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(tmem, 512);
+}
+
+// ---------------------------------------------------------------------------------------
+// FP64-accurate tall-skinny products A^T diag(w) B on the BF16 tensor cores (Ozaki scheme)
+// ---------------------------------------------------------------------------------------
+// One launch forms up to OG_PROD products per subdomain (the orthonormalisations' Grams, the
+// Galerkin coefficients): each product's rows are cut into chunks of crows rows, and every
+// (subdomain, product, chunk) item gives one partial, na x nb entries of an RC x RC block,
+// summed by its consumer in chunk order.  With chunk exponents (symmetric Grams) the partial is
+// the Gram of 2^-e A (e = the chunk's scale when it is far from 1; INT_MIN for a chunk below
+// 2^-1000).
+//
+// A column's largest exponent over the chunk bounds it by 2^c; the values (weights multiplied
+// in, in FP64) become 7 balanced base-256 digits relative to 2^(c + 1) (as for the tall
+// products, one bit higher, so that every digit, the leading one included, is in
+// [-128, 128]).  The rows are the K dimension of the MMAs: stages of 32 rows, digit planes
+// P x 32 (P = the column count rounded up to 16) of both operands.  The M = 128 operand of an
+// MMA starting at plane s1 covers h = 128 / P consecutive planes of A: lanes u P .. u P + P - 1
+// ("band" u) hold plane s1 + u.  One MMA per s1 in {0, h, 2h, ..} with B's planes t = 0 .. 6 - s1
+// stacked along N (accumulator column block s1 + t) serves every band at once: in band u, block
+// c accumulates the digit pairs (s, t) of order s + t = c + u, at most 4 of them: over 256 rows
+// their sums stay within 2^24, exact in FP32, and the accumulators are read out.  The read-out
+// combines a band's blocks in 64-bit integers (< 2^63), shifts band u down by 8 u bits, adds the
+// bands and converts to FP64.  Error: a few units of 2^-54 of the product of the two columns'
+// largest entries per row (an FP64 dot product rounds every partial sum to 2^-53 of it).
+//
+// One CTA per SM, its warps specialised, each CTA walking a contiguous range of items of about
+// equal cost:
+//   16 converter warps 8 x 8 blocks of an operand -> registers (a stage ahead) -> digit planes
+//                      (a warp's 32 stores of a plane are 128 consecutive bytes);
+//   8 auxiliary warps  the column bounds of the item after the one being converted, then the
+//                      read-out of the item before it;
+//   1 MMA warp.
+// The FP64 pipe does 2 operations per clock and SM, which made these products the largest part
+// of a step with the rank at 20 (r_t = 40): spatial coefficients of 262144 x 40, per launch:
+// 1700 us on the FP64 pipe, 190 now; the angular ones (131072 directions) 1300 -> 230; an
+// orthonormalisation's Gram 271 on the FP64 pipe, 150 with this scheme but CTA-wide phases, 38
+// now.
+#define OG_KS 32                          // rows per stage (K of one stage's MMAs)
+#define OG_GROUP 256                      // rows per read-out
+#define OG_RING 4                         // items whose column exponents are kept
+#define OG_XLD 17
+#define OG_CONV 8                         // converter warps
+#define OG_THREADS ((OG_CONV + 8 + 1) * 32)
+
+// dynamic shared memory: stages, the space an M = 128 operand may read past the last plane,
+// the read-out's exchange buffer
+static __host__ __device__ __forceinline__ uint32_t og_stage(int RC) {
+  return (uint32_t)OZ_DIG * 2 * ((RC + 15) / 16 * 16) * (2 * OG_KS);
+}
+static __host__ __device__ __forceinline__ int og_stages(int RC) { return og_stage(RC) * 4 <= 120 * 1024 ? 4 : 3; }
+static size_t og_smem(int RC) {
+  return 128 + (size_t)og_stages(RC) * og_stage(RC) + 128 * 2 * OG_KS + (size_t)128 * OG_XLD * 8;
+}
+
+__device__ __forceinline__ void og_aux_sync() { asm volatile("bar.sync 3, 256;" ::: "memory"); }
+
+// rows of product p of subdomain k, columns of its operands
+__device__ __forceinline__ void og_shape(const OzGram& a, int k, const OzProd& p, int* rows, int* na,
+                                         int* nb) {
+  *rows = p.rows == OG_CELLS ? a.g.N[k] : p.rows == OG_DIRS ? a.g.n : lines_of(a.g, k, a.axis).nlines;
+  int ka = k;
+  if (p.aside >= 0) {
+    ka = a.g.nb[k * 4 + 2 * a.axis + p.aside];
+    if (ka < 0) {                        // no neighbour: its physical inflow's column, or nothing
+      const bool in = a.infl_on && a.infl_on[k * 4 + 2 * a.axis + p.aside];
+      *na = in ? 1 : 0;
+      *nb = p.bcnt ? p.bcnt[k] : p.bfix;
+      if (!in) *rows = 0;
+      return;
+    }
+  }
+  *na = p.acnt ? p.acnt[ka] : p.afix;
+  *nb = p.B ? (p.bcnt ? p.bcnt[k] : p.bfix) : *na;
+}
+__device__ __forceinline__ int og_chunks(const OzGram& a, int rows) {
+  return rows > 0 ? (rows + a.crows - 1) / a.crows : 0;
+}
+
+// an item's operands: element (row, column) of A at A[row * astep + column]
+struct OgItem {
+  const double *A, *B, *w;              // w: row weights (null: none)
+  long astep, bstep;
+  int k, blk, c, r0, r1, na, nb, PA, PB, wsel, nx, shift;   // nx: row length for the line starts
+  int rsafe;                            // a row of B that may be read in place of one left out
+  bool sym, eok;
+};
+__device__ __forceinline__ OgItem og_item(const OzGram& a, int k, int pi, int c) {
+  const OzProd& p = a.p[pi];
+  OgItem t;
+  int rows;
+  og_shape(a, k, p, &rows, &t.na, &t.nb);
+  t.k = k; t.c = c; t.blk = p.blk;
+  t.r0 = c * a.crows;
+  t.r1 = min(rows, t.r0 + a.crows);
+  t.PA = t.na <= 16 ? 16 : (t.na + 15) & ~15;
+  t.PB = t.nb <= 16 ? 16 : (t.nb + 15) & ~15;
+  t.sym = p.B == nullptr;
+  t.shift = p.shift;
+  t.wsel = p.wsel;
+  // (a shifted operand's rows start one cell early; row rsafe is inside)
+  t.rsafe = p.shift ? (a.axis == 0 ? 1 : a.g.nxk[k]) : t.r0;
+  t.w = nullptr;
+  t.nx = p.shift ? (a.axis == 0 ? a.g.nxk[k] : 0) : 0;
+  t.eok = a.cexp != nullptr;
+  t.astep = p.lda;
+  t.bstep = p.ldb;
+  if (p.rows == OG_DIRS) {
+    const int ka = p.aside >= 0 ? a.g.nb[k * 4 + 2 * a.axis + p.aside] : k;
+    if (ka >= 0) {
+      t.A = p.A + (long)ka * a.g.n * p.lda;
+    } else {                            // physical inflow: one column, already masked
+      t.A = a.infl_hw + ((long)k * 4 + 2 * a.axis + p.aside) * a.g.n;
+      t.astep = 1;
+    }
+    t.B = t.sym ? t.A : p.B + (long)k * a.g.n * p.ldb;
+    if (p.wsel != W_NONE) t.w = a.axis == 0 ? a.ox : a.oy;
+  } else {
+    const long row0 = a.g.rowoff[k];
+    if (p.rows == OG_CELLS) {
+      t.A = p.A + row0 * p.lda;
+      t.B = t.sym ? t.A : p.B + row0 * p.ldb;
+      if (p.shift) t.B = t.A - (long)(a.axis == 0 ? 1 : a.g.nxk[k]) * p.lda;
+      if (p.shift) t.bstep = p.lda;
+      if (p.wsel == W_ROW) t.w = p.wrow + row0;
+    } else {
+      const Lines L = lines_of(a.g, k, a.axis);
+      const int side = p.rows == OG_FACE_HI;
+      t.A = p.A + (row0 + cell_of(L, 0, side ? L.len - 1 : 0)) * p.lda;
+      t.astep = (long)L.stride_line * p.lda;
+      t.B = p.B + ((long)k * 2 + side) * a.maxlines * p.ldb;
+    }
+  }
+  return t;
+}
+// whether a shift leaves row r of B inside its line
+__device__ __forceinline__ bool og_inside(const OzGram& a, const OgItem& t, int r) {
+  return !t.shift || (a.axis == 0 ? r % t.nx != 0 : r >= a.g.nxk[t.k]);
+}
+// whether a row of weight w is on the right side of a mask
+__device__ __forceinline__ bool og_side(const OgItem& t, double w) {
+  const long long ob = __double_as_longlong(w);
+  const bool ng = ob < 0 && ob != (long long)0x8000000000000000ull;
+  return !(t.wsel == W_NEG || t.wsel == W_NONNEG) || (t.wsel == W_NEG) == ng;
+}
+// the weight of a row (Omega+ and Omega- vanish on the other side)
+__device__ __forceinline__ double og_weight(const OgItem& t, double w) {
+  if (t.wsel == W_OMEGA_POS) return w > 0.0 ? w : 0.0;
+  if (t.wsel == W_OMEGA_NEG) return w < 0.0 ? w : 0.0;
+  return w;
+}
+__device__ __forceinline__ bool og_weighted(const OgItem& t) {
+  return t.wsel == W_OMEGA || t.wsel == W_OMEGA_POS || t.wsel == W_OMEGA_NEG || t.wsel == W_ROW;
+}
+
+// Two rows (p0, p1) of an operand: column ci of the 8-column groups cg + 2 i, i < NB (columns past n
+// read the last one)
+template <int NB>
+__device__ __forceinline__ void og_load(double (&d)[4][2], const double* p0, const double* p1, int cg,
+                                        int ci, int n) {
+#pragma unroll
+  for (int i = 0; i < NB; ++i) {
+    const int col = max(0, min(8 * (cg + 2 * i) + ci, n - 1));
+    d[i][0] = __ldg(p0 + col);
+    d[i][1] = __ldg(p1 + col);
+  }
+}
+__device__ __forceinline__ void og_load(double (&d)[4][2], const double* p0, const double* p1, int cg,
+                                        int ci, int n, int P) {
+  if (P <= 16) og_load<1>(d, p0, p1, cg, ci, n);                // warp-uniform; P a multiple of 16
+  else if (P <= 32) og_load<2>(d, p0, p1, cg, ci, n);
+  else if (P <= 48) og_load<3>(d, p0, p1, cg, ci, n);
+  else og_load<4>(d, p0, p1, cg, ci, n);
+}
+// their digits (rows rp, rp + 1 of the stage; weights w multiplied in when mul; rows that are not
+// ok count as zero; cs: column exponents) into the planes at base, PL apart
+template <int NB>
+__device__ __forceinline__ void og_convert(const double (&x)[4][2], const double (&w)[2], bool mul,
+                                           const bool (&ok)[2], int cg, int ci, int rp, const int* cs,
+                                           int n, uint8_t* base, uint32_t PL) {
+  double v[NB][2];
+#pragma unroll
+  for (int i = 0; i < NB; ++i) { v[i][0] = x[i][0]; v[i][1] = x[i][1]; }
+  if (mul)
+#pragma unroll
+    for (int i = 0; i < NB; ++i) { v[i][0] *= w[0]; v[i][1] *= w[1]; }
+#pragma unroll
+  for (int i = 0; i < NB; ++i) {
+    const int col = 8 * (cg + 2 * i) + ci, e1 = cs[col] + 1;
+    uint32_t d[OZ_DIG];
+    oz_digits2(ok[0] && col < n ? v[i][0] : 0.0, e1, ok[1] && col < n ? v[i][1] : 0.0, e1, d);
+    uint8_t* pl = base + tc::op_off(col, rp * 2, 2 * OG_KS);
+#pragma unroll
+    for (int s = 0; s < OZ_DIG; ++s) *reinterpret_cast<uint32_t*>(pl + s * PL) = d[s];
+  }
+}
+__device__ __forceinline__ void og_convert(const double (&x)[4][2], const double (&w)[2], bool mul,
+                                           const bool (&ok)[2], int cg, int ci, int rp, const int* cs,
+                                           int n, uint8_t* base, uint32_t PL, int P) {
+  if (P <= 16) og_convert<1>(x, w, mul, ok, cg, ci, rp, cs, n, base, PL);
+  else if (P <= 32) og_convert<2>(x, w, mul, ok, cg, ci, rp, cs, n, base, PL);
+  else if (P <= 48) og_convert<3>(x, w, mul, ok, cg, ci, rp, cs, n, base, PL);
+  else og_convert<4>(x, w, mul, ok, cg, ci, rp, cs, n, base, PL);
+}
+
+__global__ void __launch_bounds__(OG_THREADS, 1) k_oz_gram(const __grid_constant__ OzGram a) {
+  extern __shared__ uint8_t raw_og[];
+  uint8_t* buf0 = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw_og) + 127) &
+                                             ~uintptr_t(127));
+  const int RC = a.g.RC, NST = og_stages(RC);
+  const uint32_t SB = og_stage(RC);
+  long long* X = reinterpret_cast<long long*>(buf0 + (size_t)NST * SB + 128 * 2 * OG_KS);
+  __shared__ uint64_t full[4], empty[4], tfull[2], tempty[2], bnd[OG_RING];
+  __shared__ uint32_t tmem_s;
+  __shared__ int cs[OG_RING][2][DD_MAXC], exs[OG_RING], cred[8][2][DD_MAXC];
+  __shared__ int part_w[32], range[4];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int npair = a.g.nsub * a.nprod;
+  // ---- this CTA's items: pairs (subdomain, product) in order, chunks within a pair; an item
+  // costs its stages' conversions (and their MMAs) and a read-out
+  auto pair_cost = [&](int u, int* nck) {
+    int rows, na, nb;
+    const OzProd& p = a.p[u % a.nprod];
+    og_shape(a, u / a.nprod, p, &rows, &na, &nb);
+    *nck = og_chunks(a, rows);
+    const int st = (min(rows, a.crows) + OG_KS - 1) / OG_KS;
+    return st * (2 + ((na + 15) >> 4) + (p.B ? (nb + 15) >> 4 : 1)) + 20;
+  };
+  {
+    const int per = (npair + 511) / 512, ua = min(npair, tid * per), ub = tid < 512 ? min(npair, ua + per) : ua;
+    int w = 0;
+    for (int u = ua; u < ub; ++u) {
+      int nck;
+      const int c = pair_cost(u, &nck);
+      w += nck * c;
+    }
+    int inc = w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += t;
+    }
+    if (lane == 31) part_w[warp] = inc;
+    if (tid < 4) range[tid] = tid & 1 ? 0 : npair;
+    __syncthreads();
+    int total = 0, before = 0;
+    for (int i = 0; i < 16; ++i) {
+      if (i < warp) before += part_w[i];
+      total += part_w[i];
+    }
+    const int lo = before + inc - w;
+    for (int side = 0; side < 2; ++side) {
+      const int x = (int)((long)(blockIdx.x + side) * total / gridDim.x);
+      if (w > 0 && x >= lo && x < lo + w) {
+        int at = lo;
+        for (int u = ua; u < ub; ++u) {
+          int nck;
+          const int c = pair_cost(u, &nck);
+          if (x < at + nck * c) {
+            range[2 * side] = u;
+            range[2 * side + 1] = (x - at + c - 1) / c;
+            break;
+          }
+          at += nck * c;
+        }
+      }
+    }
+  }
+  if (tid == 0) {
+    for (int i = 0; i < 4; ++i) { tc::mbar_init(&full[i], OG_CONV); tc::mbar_init(&empty[i], 1); }
+    for (int i = 0; i < 2; ++i) { tc::mbar_init(&tfull[i], 1); tc::mbar_init(&tempty[i], 8); }
+    for (int i = 0; i < OG_RING; ++i) tc::mbar_init(&bnd[i], 8);
+    tc::mbar_init_fence();
+  }
+  if (warp == 0) tc::tmem_alloc(&tmem_s, 512);
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tmem = tmem_s;
+  const int u1 = range[2], c1 = range[3];
+  // the next existing item at or after (u, c); false past this CTA's last
+  auto settle = [&](int& u, int& c) {
+    while (u < npair && (u < u1 || (u == u1 && c < c1))) {
+      int rows, na, nb;
+      og_shape(a, u / a.nprod, a.p[u % a.nprod], &rows, &na, &nb);
+      if (c < og_chunks(a, rows)) return true;
+      ++u;
+      c = 0;
+    }
+    return false;
+  };
+  bool alive = true;
+
+  if (warp < OG_CONV) {
+    // ------------------------------------------------------------------ converters
+    // A stage's 8 x 8 blocks: warp w takes row group w % 4 and the column groups w / 4 + 2 i of A,
+    // then of B; an operand's loads are under way while the one before it converts
+    int u = range[0], c = range[1], it = 0, st = 0;
+    const int ci = lane & 7, rp = 8 * (warp & 3) + 2 * (lane >> 3), cg = warp >> 2;
+    while (settle(u, c)) {
+      const OgItem t = og_item(a, u / a.nprod, u % a.nprod, c);
+      const int slot = it & (OG_RING - 1);
+      const int nst = (t.r1 - t.r0 + OG_KS - 1) / OG_KS, nh = t.sym ? nst : 2 * nst;
+      const bool wtd = og_weighted(t);
+      double x[4][2], y[4][2], xw[2], yw[2];
+      bool xo[2], yo[2];
+      // half-stage hs: operand A or B of a stage (a symmetric product has A alone)
+      auto load = [&](double(&d)[4][2], double(&w)[2], bool(&ok)[2], int hs) {
+        const bool isB = !t.sym && (hs & 1);
+        const int r = t.r0 + (t.sym ? hs : hs >> 1) * OG_KS + rp, n = isB ? t.nb : t.na;
+        const double* p[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int rr = min(r + h, t.r1 - 1);
+          ok[h] = r + h < t.r1;
+          // (the row's weight or mask is looked at only when the row is converted: an address
+          // that waited for it would hold up the conversion before)
+          w[h] = 1.0;
+          bool in = true;
+          if (isB || t.sym) {
+            in = og_inside(a, t, rr);
+            ok[h] = ok[h] && in;
+            if (t.w) w[h] = t.w[rr];
+          }
+          p[h] = (isB ? t.B : t.A) + (long)(in ? rr : t.rsafe) * (isB ? t.bstep : t.astep);
+        }
+        og_load(d, p[0], p[1], cg, ci, n, isB ? t.PB : t.PA);
+      };
+      load(x, xw, xo, 0);
+      if (a.g.work)
+        count_work(a.g, KS_OZ_GRAM, (t.sym ? 1.0 : 2.0) * (t.r1 - t.r0) * t.na * (t.sym ? t.na + 1 : t.nb));
+      alive = tc::mbar_wait(&bnd[slot], (it / OG_RING) & 1, kWait) && alive;
+      const uint32_t PLA = (uint32_t)t.PA * 2 * OG_KS, PLB = (uint32_t)t.PB * 2 * OG_KS;
+#pragma unroll 1
+      for (int hs = 0; hs < nh; ++hs) {
+        if (hs + 1 < nh) load(y, yw, yo, hs + 1);
+        const bool isB = !t.sym && (hs & 1), first = !isB, lasth = t.sym || isB;
+        const int b4 = st % NST, use = st / NST;
+        if (first && use > 0 && alive) alive = tc::mbar_wait(&empty[b4], (use - 1) & 1, kWait);
+        uint8_t* base = buf0 + (size_t)b4 * SB + (isB ? OZ_DIG * PLA : 0u);
+        const bool mul = wtd && (isB || t.sym);
+        if (t.w && (isB || t.sym)) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            xo[h] = xo[h] && og_side(t, xw[h]);
+            xw[h] = og_weight(t, xw[h]);
+          }
+        }
+        og_convert(x, xw, mul, xo, cg, ci, rp, cs[slot][isB], isB ? t.nb : t.na, base, isB ? PLB : PLA,
+                   isB ? t.PB : t.PA);
+        if (lasth) {
+          tc::fence_async_smem();
+          __syncwarp();
+          if (lane == 0) tc::mbar_arrive(&full[b4]);
+          ++st;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { x[i][0] = y[i][0]; x[i][1] = y[i][1]; }
+        xw[0] = yw[0]; xw[1] = yw[1];
+        xo[0] = yo[0]; xo[1] = yo[1];
+      }
+      ++it;
+      ++c;
+    }
+  } else if (warp < OG_CONV + 8) {
+    // ------------------------------------------------------------------ bounds and read-out
+    const int w8 = warp - OG_CONV, q4 = warp & 3, half = w8 >> 2, at = tid - 32 * OG_CONV;
+    // column exponents of item number it: A (and B when it is another operand)
+    auto bounds = [&](const OgItem& t, int it) {
+      const int slot = it & (OG_RING - 1);
+      const bool wtd = og_weighted(t);
+#pragma unroll
+      for (int op = 0; op < 2; ++op) {
+        if (op == 1 && t.sym) break;
+        const double* base = op ? t.B : t.A;
+        const long step = op ? t.bstep : t.astep;
+        const int n = op ? t.nb : t.na;
+        const bool side = op == 1 || t.sym;
+        int m0 = 0, m1 = 0;                              // biased exponents
+        const int c0 = max(0, min(lane, n - 1)), c1 = max(0, min(lane + 32, n - 1));
+        const bool plain = !side || !(wtd || t.shift || t.wsel == W_NEG || t.wsel == W_NONNEG);
+        for (int rb = t.r0 + w8; rb < t.r1; rb += 128) {     // 16 rows at a time, all loads first
+          int h0[16], h1[16], ew[16];
+          if (plain) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const int* hw = reinterpret_cast<const int*>(base + (long)min(rb + 8 * i, t.r1 - 1) * step) + 1;
+              h0[i] = __ldg(hw + 2 * c0);
+              h1[i] = __ldg(hw + 2 * c1);
+              ew[i] = 0;
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const int r = min(rb + 8 * i, t.r1 - 1);
+              const bool in = og_inside(a, t, r);
+              const double w = t.w ? t.w[r] : 1.0;
+              const int* hw = reinterpret_cast<const int*>(base + (long)(in ? r : t.rsafe) * step) + 1;
+              h0[i] = __ldg(hw + 2 * c0);
+              h1[i] = __ldg(hw + 2 * c1);
+              const int E = wtd ? f64_bexp(og_weight(t, w)) : 1022;
+              ew[i] = in && og_side(t, w) && E ? E - 1022 : -4096;
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const int E0 = (h0[i] >> 20) & 0x7ff, E1 = (h1[i] >> 20) & 0x7ff;
+            m0 = max(m0, E0 ? E0 + ew[i] : 0);
+            m1 = max(m1, E1 ? E1 + ew[i] : 0);
+          }
+        }
+        if (lane >= n) m0 = 0;
+        if (lane + 32 >= n) m1 = 0;
+        cred[w8][op][lane] = m0;
+        cred[w8][op][lane + 32] = m1;
+      }
+      og_aux_sync();
+      if (at < 2 * DD_MAXC) {
+        const int op = at >> 6, col = at & 63;
+        if (op == 0 || !t.sym) {
+          int m = cred[0][op][col];
+#pragma unroll
+          for (int i = 1; i < 8; ++i) m = max(m, cred[i][op][col]);
+          const int e = m > 0 ? m - 1022 : OZ_NONE;
+          cs[slot][op][col] = e;
+          if (t.sym) cs[slot][1][col] = e;
+        }
+      }
+      if (t.eok && w8 == 0) {                            // the chunk's scale
+        int m = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) m = max(m, max(cred[i][0][lane], cred[i][0][lane + 32]));
+        m = __reduce_max_sync(0xffffffffu, m);
+        const int e0 = m > 0 && m < 2047 ? m - 1023 : 0;
+        const bool zero = m <= 0 || e0 < -1000;
+        const int ex = (!zero && (e0 < -400 || e0 > 400)) ? e0 : 0;
+        if (lane == 0) {
+          exs[slot] = ex;
+          a.cexp[(long)t.k * a.nchunk + t.c] = zero ? INT_MIN : ex;
+        }
+      }
+      __syncwarp();
+      og_aux_sync();                                     // cred is read; cs, exs are written
+      if (lane == 0) tc::mbar_arrive(&bnd[slot]);
+    };
+    int grp = 0;                                         // read-out groups done
+    auto readout = [&](const OgItem& t, int it) {
+      const int slot = it & (OG_RING - 1), h = 128 / t.PA, nbd = min(h, OZ_DIG);
+      const int tb = 14 * t.PB <= 512 ? 2 : 1;
+      const int L = q4 * 32 + lane, u = L / t.PA;
+      double* out = a.part + (((long)t.k * a.nchunk + t.c) * a.nblk + t.blk) * RC * RC;
+      for (int r = t.r0; r < t.r1; r += OG_GROUP, ++grp) {
+        // the group's TMEM half (all of it where 7 blocks do not fit twice)
+        const int b2 = grp & 1;
+        alive = __all_sync(0xffffffffu, tc::mbar_wait(&tfull[b2], (grp >> 1) & 1, kWait)) && alive;
+        alive = __all_sync(0xffffffffu, alive);
+        tc::fence_after_sync();
+        for (int cg = 0; cg < t.PB; cg += 16) {
+          if (alive) {
+#pragma unroll 1
+            for (int c4 = 8 * half; c4 < 8 * half + 8; c4 += 4) {
+              uint32_t D[OZ_DIG][4];
+#pragma unroll
+              for (int g = 0; g < OZ_DIG; ++g)
+                oz_tmem_ld4(tmem + ((uint32_t)(q4 * 32) << 16) +
+                                (uint32_t)((tb == 2 ? 256 * b2 : 0) + g * t.PB + cg + c4), D[g]);
+              asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+              for (int g = 0; g < OZ_DIG; ++g)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  asm volatile("" : "+r"(D[g][i]));
+                  if (g + u > OZ_DIG - 1) D[g][i] = 0u;  // orders past the last (junk planes among them)
+                }
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                X[L * OG_XLD + c4 + i] = u < nbd ? oz_combine(&D[0][i], 4) >> (8 * u) : 0ll;
+            }
+          }
+          if (cg + 16 >= t.PB) {                         // the accumulators are free again
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&tempty[b2]);
+          }
+          og_aux_sync();
+          if (alive) {
+            const int j = at & 15, col = cg + j;
+            const int ex = t.eok ? 2 * exs[slot] : 0;
+            if (col < t.nb)
+              for (int i = at >> 4; i < t.na; i += 16) {
+                long long J = 0;
+                for (int v = 0; v < nbd; ++v) J += X[(v * t.PA + i) * OG_XLD + j];
+                const double v = oz_round(J, cs[slot][0][i] + cs[slot][1][col] + 2 - 56 - ex);
+                double* o = out + i * RC + col;
+                *o = r == t.r0 ? v : *o + v;
+              }
+          }
+          og_aux_sync();                                 // X is free
+        }
+      }
+    };
+    int u = range[0], c = range[1], it = 0;
+    bool more = settle(u, c);
+    OgItem prev{};
+    bool have = false;
+    while (more || have) {
+      OgItem cur{};
+      const bool now = more;
+      if (now) {
+        cur = og_item(a, u / a.nprod, u % a.nprod, c);
+        ++c;
+        more = settle(u, c);
+        if (more && at == 0 && a.p[u % a.nprod].rows <= OG_DIRS) {   // the next item's rows into L2
+          const OgItem nx = og_item(a, u / a.nprod, u % a.nprod, c);
+          if (!(nx.astep & 1)) prefetch_rows(nx.A, nx.astep, nx.r0, nx.r1 - nx.r0, nx.r1);
+          if (!nx.sym && !nx.shift && !(nx.bstep & 1))
+            prefetch_rows(nx.B, nx.bstep, nx.r0, nx.r1 - nx.r0, nx.r1);
+        }
+        bounds(cur, it);
+      }
+      if (have) readout(prev, it - 1);
+      prev = cur;
+      have = now;
+      ++it;
+    }
+  } else if (lane == 0) {
+    // ------------------------------------------------------------------ MMA issue
+    int u = range[0], c = range[1], st = 0, grp = 0, last = -1;
+    bool dbl = true;                                     // the previous group left the other half free
+    while (alive && settle(u, c)) {
+      const OgItem t = og_item(a, u / a.nprod, u % a.nprod, c);
+      const int h = 128 / t.PA, nper = 256 / t.PB, tb = 14 * t.PB <= 512 ? 2 : 1;
+      const uint32_t PLA = (uint32_t)t.PA * 2 * OG_KS, PLB = (uint32_t)t.PB * 2 * OG_KS;
+      for (int r = t.r0; r < t.r1 && alive; r += OG_GROUP, ++grp) {
+        const int b2 = grp & 1;
+        // this group's accumulators: the half's previous group is read out, and where either
+        // this group or the one before it spans both halves, that one too
+        if (grp >= 2) alive = tc::mbar_wait(&tempty[b2], ((grp >> 1) - 1) & 1, kWait);
+        if (alive && grp >= 1 && (tb == 1 || !dbl))
+          alive = tc::mbar_wait(&tempty[b2 ^ 1], ((grp - 1) >> 1) & 1, kWait);
+        if (!alive) break;
+        tc::fence_after_sync();
+        dbl = tb == 2;
+        const uint32_t d0 = tmem + (tb == 2 ? 256u * b2 : 0u);
+        const int re = min(t.r1, r + OG_GROUP);
+        for (int s0 = r; s0 < re; s0 += OG_KS, ++st) {
+          const int b4 = st % NST;
+          alive = tc::mbar_wait(&full[b4], (st / NST) & 1, kWait);
+          if (!alive) break;
+          tc::fence_after_sync();
+          const uint32_t sa = tc::smem_u32(buf0 + (size_t)b4 * SB);
+          const uint64_t ad = tc::sdesc(sa, 128, 16 * OG_KS);
+          const uint64_t bd = t.sym ? ad : tc::sdesc(sa + OZ_DIG * PLA, 128, 16 * OG_KS);
+          for (int j = 0; j < OG_KS / 16; ++j)
+            for (int s1 = 0; s1 < OZ_DIG; s1 += h)
+              for (int v0 = 0; v0 < OZ_DIG - s1; v0 += nper) {
+                const int nu = min(nper, OZ_DIG - s1 - v0);
+                tc::mma_bf16(d0 + (uint32_t)((s1 + v0) * t.PB), ad + ((s1 * PLA + 256 * j) >> 4),
+                             bd + ((v0 * PLB + 256 * j) >> 4),
+                             tc::idesc(tc::FMT_BF16, 128, nu * t.PB),
+                             (s0 > r || j > 0 || s1 > 0) ? 1u : 0u);
+              }
+          tc::mma_commit(&empty[b4]);
+          last = st;
+        }
+        if (!alive) break;
+        tc::mma_commit(&tfull[b2]);
+      }
+      ++c;
+    }
+    // every MMA issued is complete before the memory goes back
+    if (last >= 0) alive = tc::mbar_wait(&empty[last % NST], (last / NST) & 1, kWait) && alive;
+  }
+  if (!alive && lane == 0) atomicOr(a.status, (unsigned)ST_TIMEOUT);
+  __syncwarp();
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tmem, 512);
+}
+
+// Sum of the chunk partials of every product, in chunk order, into the small matrices (slot
+// dst[blk]), zero outside the product's na x nb entries.
+__global__ void __launch_bounds__(DD_THREADS) k_oz_reduce(const __grid_constant__ OzGram a, OzDst dst,
+                                                          double* sm) {
+  const int k = blockIdx.y / a.nprod, RC = a.g.RC;
+  const OzProd& p = a.p[blockIdx.y - k * a.nprod];
+  int rows, na, nb;
+  og_shape(a, k, p, &rows, &na, &nb);
+  const int nck = og_chunks(a, rows);
+  const double* part = a.part + ((long)k * a.nchunk * a.nblk + p.blk) * RC * RC;
+  double* out = sm + ((long)k * NSMALL + dst.idx[p.blk]) * RC * RC;
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= RC * RC) return;
+  const int i = e / RC, j = e - i * RC;
+  double s = 0.0;
+  if (i < na && j < nb) {
+#pragma unroll 8
+    for (int c = 0; c < nck; ++c) s += part[(long)c * a.nblk * RC * RC + e];
+  }
+  out[e] = s;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1215,7 +1694,7 @@ cudaError_t tc_init() {
                            (int)tc_gram_smem());
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_oz_tall, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)OZ_SMEM_LIMIT);
+                           (int)ot_smem(DD_MAXC));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_oz_gram, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)og_smem(DD_MAXC));
@@ -1235,7 +1714,7 @@ bool tc_tall(const Problem& P, unsigned* status, cudaStream_t st, int spatial, c
   a.g = P.g; a.spatial = spatial; a.lda = lda; a.ninner = ninner; a.ninner_fix = ninner_fix;
   a.Bm = Bm; a.bsmall = bsmall; a.smbase = smbase; a.ncols = ncols; a.ncols_fix = ncols_fix;
   a.Y = Y; a.ldy = ldy; a.alpha = alpha; a.accumulate = accumulate; a.status = status;
-  a.A = A; a.mtrans = 0; a.rowscale = nullptr;
+  a.A = A; a.mtrans = 0; a.rowscale = nullptr; a.nrows = 0; a.zfill = 1;
   a.tps = ((spatial ? P.maxN : P.g.n) + TT_ROWS - 1) / TT_ROWS;
   const long ntot = (long)P.g.nsub * a.tps;
   const int grid = (int)std::min<long>(ntot, P.nsm);
@@ -1252,21 +1731,21 @@ bool oz_tall(const Problem& P, unsigned* status, cudaStream_t st, int spatial, c
              int lda, const int* ninner, int ninner_fix, const double* Bm, int bsmall,
              const double* smbase, const int* ncols, int ncols_fix, double* Y, int ldy,
              int mtrans, int accumulate, const double* rowscale) {
-  if (lda > DD_MAXC || (lda & 1)) return false;
-  const OzPlan pl = oz_plan(lda, OZ_SMEM_LIMIT);
-  if (pl.total > OZ_SMEM_LIMIT) return false;
+  if (lda > DD_MAXC || (lda & 1) || (ldy & 1)) return false;
   TcTall a;
   a.g = P.g; a.spatial = spatial; a.lda = lda; a.ninner = ninner; a.ninner_fix = ninner_fix;
   a.Bm = Bm; a.bsmall = bsmall; a.smbase = smbase; a.ncols = ncols; a.ncols_fix = ncols_fix;
   a.Y = Y; a.ldy = ldy; a.alpha = 1.0; a.accumulate = accumulate; a.status = status;
   a.A = A;
+  a.nrows = spatial ? P.Ntot : (long)P.g.nsub * P.g.n;
+  a.zfill = !accumulate && P.prec >= PREC_TF32;
   a.mtrans = mtrans;
   a.rowscale = rowscale;
   a.tps = ((spatial ? P.maxN : P.g.n) + TT_ROWS - 1) / TT_ROWS;
   const long ntot = (long)P.g.nsub * a.tps;
   const int grid = (int)std::min<long>(ntot, P.nsm);
   pbeg(st, KS_OZ_TALL);
-  k_oz_tall<<<grid, OZ_THREADS, pl.total, st>>>(a, pl.KP, pl.KA, pl.npass, pl.nbuf);
+  k_oz_tall<<<grid, OT_THREADS, ot_smem(lda), st>>>(a);
   pend(st);
   return true;
 }
@@ -1300,17 +1779,21 @@ bool tc_gram(const Problem& P, cudaStream_t st, const TcGram& a0) {
   return true;
 }
 
-bool oz_gram(const Problem& P, unsigned* status, cudaStream_t st, int spatial, const double* A,
-             int lda, const int* acnt, double* part, int nchunk, int* cexp) {
-  if (P.g.RC > DD_MAXC) return false;
-  const size_t smem = og_smem(P.g.RC);
-  OzGram a;
-  a.g = P.g; a.spatial = spatial; a.A = A; a.lda = lda; a.acnt = acnt; a.part = part;
-  a.nchunk = nchunk; a.cexp = cexp; a.status = status;
-  const int grid = (int)std::min<long>((long)P.g.nsub * nchunk, P.nsm);
+bool oz_gram(const Problem& P, cudaStream_t st, OzGram& a, const OzDst* dst, double* sm) {
+  if (P.g.RC > DD_MAXC || a.nprod < 1) return false;
+  a.g = P.g;
+  a.ox = P.ox; a.oy = P.oy;
+  a.maxlines = P.maxlines;
+  a.infl_on = P.infl_on; a.infl_hw = P.infl_hw;
   pbeg(st, KS_OZ_GRAM);
-  k_oz_gram<<<grid, OZ_THREADS, smem, st>>>(a);
+  k_oz_gram<<<P.nsm, OG_THREADS, og_smem(P.g.RC), st>>>(a);
   pend(st);
+  if (dst) {
+    pbeg(st, KS_REDUCE);
+    k_oz_reduce<<<dim3((P.g.RC * P.g.RC + DD_THREADS - 1) / DD_THREADS, P.g.nsub * a.nprod), DD_THREADS, 0, st>>>(
+        a, *dst, sm);
+    pend(st);
+  }
   return true;
 }
 
