@@ -1234,88 +1234,59 @@ __global__ void k_coll_a(Problem P, PhaseBufs B) {
   }
 }
 
-// row-local collision K-step: dK_c/dt = (sig_s/|S|)(K_c . a) a - sig_t K_c + sQ_c a
-template <typename TC>
-__global__ void k_coll_kstep(Problem P, PhaseBufs B) {
-  const int k = blockIdx.y, RC = P.g.RC;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int N = P.g.N[k], rc = B.rc[k];
-  const double* a = SMB(B, P, k, SM_VEC);
-  const TC dt = (TC)P.g.dtk[k];
+// Row-local collision K-step, dK_c/dt = (sig_s/|S|)(K_c . a) a - sig_t K_c + sQ_c a: the stages of
+// cell c stay in the span of K_c and a, K^(s) = alpha_s K_c + beta_s a, so with d = K_c . a and
+// a . a every stage is a few scalar operations and the update is
+// K_c + dt (A K_c + B a), A = sum_s b_s (-sig_t alpha_s), B = sum_s b_s (..).  A CTA stages the rows
+// of 128 cells in shared memory (coalesced both ways), a thread owns a cell: 4 r_c + 60 FP64
+// operations a cell (RK4) where the stages entry by entry took 24 r_c, one cell per warp.  In every
+// precision (the reduced forms' FP32 stages were slower).  Bound by the FP64 pipe and the loads:
+// 400000 cells, r_c to 21, RK4, 1000 us before, 90 now; 262144 cells, r_c = 20, Euler 140 -> 60.
+#define CK_CELLS 128
+size_t coll_kstep_smem(int RC) { return sizeof(double) * (CK_CELLS * (size_t)(RC | 1) + RC); }
+__global__ void __launch_bounds__(CK_CELLS) k_coll_kstep(Problem P, PhaseBufs B) {
+  extern __shared__ double ck[];
+  const int k = blockIdx.y, RC = P.g.RC, N = P.g.N[k], rc = B.rc[k], tid = threadIdx.x;
+  const int c0 = blockIdx.x * CK_CELLS, nc = min(CK_CELLS, N - c0), ld = rc | 1;
+  if (nc <= 0) return;
   const int nst = P.integrator == 1 ? 4 : 1;
-  // a cell per W lanes (W the power of two >= r_c, up to 32), G = 32 / W cells per warp: FP64
-  // instructions hold the pipe whether or not their lanes are active.  The dot product's
-  // butterfly over W lanes is the full warp's with the steps that add zero lanes left out.
-  int W = 1;
-  while (W < rc && W < 32) W <<= 1;
-  const int G = 32 / W, slot = lane / W, tl = lane - slot * W;
-  {
-    double cells = 0.0;
-    for (long c0 = (long)blockIdx.x * nw * G; c0 < N; c0 += (long)gridDim.x * nw * G)
-      cells += (double)min((long)nw * G, (long)N - c0);
-    count_work(P.g, KS_COLL_KSTEP, cells * rc * 6.0 * nst);
-  }
-  for (int c0 = (blockIdx.x * nw + warp) * G; c0 < N; c0 += gridDim.x * nw * G) {
-    const int cell = c0 + slot;
-    const bool valid = cell < N;
-    const long row = (long)P.g.rowoff[k] + (valid ? cell : c0);
-    const TC ss = (TC)(P.sig_s[row] / P.ssum), st = (TC)P.sig_t[row], sq = (TC)P.sQ[row];
-    TC k0[2], ks[2], acc[2] = {0.0, 0.0}, av[2];
-    double k0d[2];
-    for (int h = 0; h < 2; ++h) {
-      int t = tl + 32 * h;
-      k0d[h] = (valid && t < rc) ? B.K[row * RC + t] : 0.0;
-      k0[h] = (TC)k0d[h];
-      av[h] = t < rc ? a[t] : 0.0;
-      ks[h] = k0[h];
-    }
-    // the upper half of the columns only where r_c > 32
-    const int nh = rc > 32 ? 2 : 1;
-    for (int s = 0; s < nst; ++s) {
-      TC d = ks[0] * av[0];
-      if (nh > 1) d += ks[1] * av[1];
-      for (int o = W >> 1; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-      TC kv[2] = {0.0, 0.0};
-      for (int h = 0; h < nh; ++h) kv[h] = ss * d * av[h] - st * ks[h] + sq * av[h];
-      const TC bs = (nst == 4) ? c_rk_b[s] : 1.0;
-      const TC an = (s + 1 < nst) ? c_rk_a[s + 1] : 0.0;
-      for (int h = 0; h < nh; ++h) {
-        acc[h] += bs * kv[h];
-        ks[h] = k0[h] + an * dt * kv[h];
-      }
-    }
-    if (valid)
-      for (int t = tl; t < RC; t += W) {
-        const int h = t >> 5;
-        B.K[row * RC + t] = t < rc ? k0d[h] + (double)(dt * acc[h]) : 0.0;
-      }
-  }
-}
-
-// The collision K-step with explicit Euler in FP64, a thread per cell (the warp form above
-// issues its FP64 instructions for one cell at a time, and a warp instruction holds the FP64
-// pipe however many of its lanes are active): K_c <- K_c + dt ((sig_s/|S|)(K_c . a) a
-// - sig_t K_c + sQ_c a) on the first r_c columns, zero beyond.
-__global__ void __launch_bounds__(DD_THREADS) k_coll_kstep1(Problem P, PhaseBufs B) {
-  __shared__ double av[DD_MAXC];
-  const int k = blockIdx.y, RC = P.g.RC, N = P.g.N[k], rc = B.rc[k];
+  if (P.g.work) count_work(P.g, KS_COLL_KSTEP, (double)nc * rc * 6.0 * nst);
+  double* Ks = ck;                                  // nc x ld
+  double* av = ck + CK_CELLS * (RC | 1);
   const double* a = SMB(B, P, k, SM_VEC);
-  for (int t = threadIdx.x; t < RC; t += blockDim.x) av[t] = t < rc ? a[t] : 0.0;
+  double* Kg = B.K + ((long)P.g.rowoff[k] + c0) * RC;
+  for (int t = tid; t < rc; t += CK_CELLS) av[t] = a[t];
+  for (int e = tid; e < nc * rc; e += CK_CELLS) {
+    const int c = e / rc, t = e - c * rc;
+    Ks[c * ld + t] = Kg[(long)c * RC + t];
+  }
   __syncthreads();
-  const int c0 = blockIdx.x * blockDim.x;
-  if (c0 >= N) return;
-  count_work(P.g, KS_COLL_KSTEP, (double)min((int)blockDim.x, N - c0) * rc * 6.0);
-  const int cell = c0 + threadIdx.x;
-  if (cell >= N) return;
-  const long row = (long)P.g.rowoff[k] + cell;
-  const double ss = P.sig_s[row] / P.ssum, st = P.sig_t[row], sq = P.sQ[row];
-  const double dt = P.g.dtk[k];
-  double* Kr = B.K + row * RC;
-  double d = 0.0;
-  for (int t = 0; t < rc; ++t) d += Kr[t] * av[t];
-  for (int t = 0; t < RC; ++t) {
-    const double k0 = Kr[t];
-    Kr[t] = t < rc ? k0 + dt * (ss * d * av[t] - st * k0 + sq * av[t]) : 0.0;
+  if (tid < nc) {
+    const long row = (long)P.g.rowoff[k] + c0 + tid;
+    const double ss = P.sig_s[row] / P.ssum, st = P.sig_t[row], sq = P.sQ[row], dt = P.g.dtk[k];
+    double* Kr = Ks + tid * ld;
+    double d = 0.0, aa = 0.0;
+    for (int t = 0; t < rc; ++t) {
+      d += Kr[t] * av[t];
+      aa += av[t] * av[t];
+    }
+    double al = 1.0, be = 0.0, A = 0.0, Bc = 0.0;
+    for (int s = 0; s < nst; ++s) {
+      const double ka = -st * al, kb = ss * (al * d + be * aa) + sq - st * be;
+      const double bs = nst == 4 ? c_rk_b[s] : 1.0, an = s + 1 < nst ? c_rk_a[s + 1] : 0.0;
+      A += bs * ka;
+      Bc += bs * kb;
+      al = 1.0 + an * dt * ka;
+      be = an * dt * kb;
+    }
+    A *= dt;
+    Bc *= dt;
+    for (int t = 0; t < rc; ++t) Kr[t] += A * Kr[t] + Bc * av[t];
+  }
+  __syncthreads();
+  for (int e = tid; e < nc * rc; e += CK_CELLS) {
+    const int c = e / rc, t = e - c * rc;
+    Kg[(long)c * RC + t] = Ks[c * ld + t];
   }
 }
 
@@ -1692,6 +1663,9 @@ cudaError_t phase_init() {
   e = cudaFuncSetAttribute(k_kstep_adv<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_kstep_adv<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_coll_kstep, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)coll_kstep_smem(RC));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_sstep_adv, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)sstep_smem(RC));
@@ -2326,13 +2300,8 @@ void collision_phase(const Problem& P, const PhaseBufs& B, cudaStream_t st) {
   pend(st);
   galerkin_tall(P, B, st, 1, B.X, RC, B.r, B.S, -1, B.rc, B.K, RC);
   pbeg(st, KS_COLL_KSTEP);
-  if (P.prec >= PREC_MIXED) {
-    k_coll_kstep<float><<<dim3(64, nsub), DD_THREADS, 0, st>>>(P, B);
-  } else if (P.integrator == 0) {
-    k_coll_kstep1<<<dim3((P.maxN + DD_THREADS - 1) / DD_THREADS, nsub), DD_THREADS, 0, st>>>(P, B);
-  } else {
-    k_coll_kstep<double><<<dim3(64, nsub), DD_THREADS, 0, st>>>(P, B);
-  }
+  k_coll_kstep<<<dim3((P.maxN + CK_CELLS - 1) / CK_CELLS, nsub), CK_CELLS, coll_kstep_smem(RC), st>>>(
+      P, B);
   pend(st);
   if (P.mass_fix) mass_acc(P, B, st, B.K, B.Vh, nullptr, B.rc, 1.0);
   {
