@@ -877,6 +877,107 @@ __global__ void __launch_bounds__(DD_THREADS) k_sstep_adv(Problem P, PhaseBufs B
   }
 }
 
+// The S-step with RK4 in the eigenbasis of C (S~ = S P), where its columns are independent:
+//   dS~_j/dt = (c/h) lambda_j (S~_j - T S~_j - G_lo~_j)     (lambda_j > 0)
+//              (c/h) lambda_j (T^T S~_j - S~_j + G_hi~_j)   (lambda_j < 0),   G~ = G P
+// so a CTA takes some columns through all four stages (one matrix-vector product per column and
+// stage where the form above takes five), and k_sstep_back adds the rotated increment.  The
+// eigen-split itself is the K-step's, P and lambda from k_small_adv1 (slots S3T and VB); the
+// increment goes to slot UB.  64 FP64-bound CTAs of four launches before: 16 subdomains,
+// r_t = 20: 59 us per S-step, 18 now; 70 of r_t <= 42: 598 us, 130 now.
+size_t sstep_cols_smem(int RC, int cols) {
+  return sizeof(double) * ((size_t)RC * (RC | 1) + 5 * (size_t)cols * RC);
+}
+__global__ void __launch_bounds__(DD_THREADS) k_sstep_cols(Problem P, PhaseBufs B, int axis, int CL, int cols) {
+  extern __shared__ double sh[];
+  const int k = blockIdx.x / CL, RC = P.g.RC, rt = B.rt[k], ld = RC | 1;
+  const int j0 = (blockIdx.x - k * CL) * cols, nj = min(cols, rt - j0);
+  if (nj <= 0) return;
+  double* T = sh;                                    // rt x rt, row-major, odd pitch
+  double* Y = T + (size_t)RC * ld;                   // stage values, column c at c rt
+  double* Yn = Y + (size_t)cols * RC;                // the next stage's
+  double* Y0 = Yn + (size_t)cols * RC;
+  double* G = Y0 + (size_t)cols * RC;
+  double* D = G + (size_t)cols * RC;                 // sum_s b_s rate_s
+  const double* Tg = SMB(B, P, k, SM_T);
+  const double* Pg = SMB(B, P, k, SM_S3T);
+  const double* lam = SMB(B, P, k, SM_VB);
+  const double* S1 = SMB(B, P, k, SM_S1);
+  for (int e = threadIdx.x; e < rt * rt; e += blockDim.x) {
+    const int i = e / rt, l = e - i * rt;
+    T[i * ld + l] = Tg[i * RC + l];
+  }
+  for (int e = threadIdx.x; e < nj * rt; e += blockDim.x) {
+    const int c = e / rt, i = e - c * rt, j = j0 + c;
+    const double* Gs = SMB(B, P, k, lam[j] > 0.0 ? SM_G_LO : SM_G_HI) + i * RC;
+    double y = 0.0, g = 0.0;
+#pragma unroll 8
+    for (int l = 0; l < rt; ++l) {
+      const double p = Pg[l * RC + j];
+      y += S1[i * RC + l] * p;
+      g += Gs[l] * p;
+    }
+    Y[c * rt + i] = y; Y0[c * rt + i] = y; G[c * rt + i] = g; D[c * rt + i] = 0.0;
+  }
+  __syncthreads();
+  const double coef = P.c_adv / (axis == 0 ? P.g.hxk[k] : P.g.hyk[k]), dt = P.g.dtk[k];
+  for (int s = 0; s < 4; ++s) {
+    for (int e = threadIdx.x; e < nj * rt; e += blockDim.x) {
+      const int c = e / rt, i = e - c * rt;
+      const double l1 = lam[j0 + c];
+      const double* y = Y + c * rt;
+      const bool up = l1 > 0.0;
+      const double* Tr = up ? T + i * ld : T + i;
+      const int step = up ? 1 : ld;
+      double x = 0.0, x1 = 0.0;
+      int l = 0;
+#pragma unroll 4
+      for (; l + 2 <= rt; l += 2) {
+        x += Tr[l * step] * y[l];
+        x1 += Tr[(l + 1) * step] * y[l + 1];
+      }
+      if (l < rt) x += Tr[l * step] * y[l];
+      x += x1;
+      const double f = coef * l1 * (up ? y[i] - x - G[c * rt + i] : x - y[i] + G[c * rt + i]);
+      D[c * rt + i] += c_rk_b[s] * f;
+      if (s < 3) Yn[c * rt + i] = Y0[c * rt + i] + c_rk_a[s + 1] * dt * f;
+    }
+    __syncthreads();
+    double* t = Y;
+    Y = Yn;
+    Yn = t;
+  }
+  double* out = SMB(B, P, k, SM_UB);
+  for (int e = threadIdx.x; e < nj * rt; e += blockDim.x) {
+    const int i = e / nj, c = e - i * nj;
+    out[i * RC + j0 + c] = dt * D[c * rt + i];
+  }
+}
+// S2 = S1 + D P^T, zero outside r_t x r_t, and the L-step matrices A_+ = I - T, A_- = T^T - I
+__global__ void __launch_bounds__(DD_THREADS) k_sstep_back(Problem P, PhaseBufs B, int CL) {
+  const int k = blockIdx.x / CL, cr = blockIdx.x - k * CL, RC = P.g.RC, rt = B.rt[k];
+  const int rpb = (RC + CL - 1) / CL, i0 = cr * rpb, i1 = min(RC, i0 + rpb);
+  const double* T = SMB(B, P, k, SM_T);
+  const double* S1 = SMB(B, P, k, SM_S1);
+  const double* D = SMB(B, P, k, SM_UB);
+  const double* Pg = SMB(B, P, k, SM_S3T);
+  double* S2 = SMB(B, P, k, SM_S2);
+  double* Ap = SMB(B, P, k, SM_AP);
+  double* Am = SMB(B, P, k, SM_AM);
+  for (int e = threadIdx.x; e < (i1 - i0) * RC; e += blockDim.x) {
+    const int li = e / RC, j = e - li * RC, i = i0 + li;
+    double x = 0.0, p = 0.0, m = 0.0;
+    if (i < rt && j < rt) {
+#pragma unroll 8
+      for (int l = 0; l < rt; ++l) x += D[i * RC + l] * Pg[j * RC + l];
+      x += S1[i * RC + j];
+      p = (i == j ? 1.0 : 0.0) - T[i * RC + j];
+      m = T[j * RC + i] - (i == j ? 1.0 : 0.0);
+    }
+    S2[i * RC + j] = x; Ap[i * RC + j] = p; Am[i * RC + j] = m;
+  }
+}
+
 // ---------------------------------------------------------------------------
 // L-step of the advection with explicit Euler as products over all directions.  The
 // Euler step of direction q's ODE is L_q = S2 v_q + dt kappa_q (A_s S2 v_q + g_q), with s
@@ -1667,6 +1768,9 @@ cudaError_t phase_init() {
   e = cudaFuncSetAttribute(k_coll_kstep, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)coll_kstep_smem(RC));
   if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_sstep_cols, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)sstep_cols_smem(RC, RC));
+  if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_sstep_adv, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)sstep_smem(RC));
   if (e != cudaSuccess) return e;
@@ -2234,9 +2338,19 @@ void advection_phase(const Problem& P, const PhaseBufs& B, int axis, cudaStream_
   {
     // blocks per subdomain: enough to cover the SMs, at most 8
     const int CL = std::max(1, std::min(8, P.nsm / std::max(1, nsub)));
-    const int nst = P.integrator == 1 ? 4 : 1;
-    for (int s = 0; s < nst; ++s)
-      k_sstep_adv<<<nsub * CL, DD_THREADS, sstep_smem(RC), st>>>(P, B, axis, s, CL);
+    if (P.integrator == 1 && P.kstep_split == 0) {
+      // (explicit Euler: one launch of the form below, 83 us against 78 and 12 against 15 for
+      // 64 subdomains of r_t = 40 and 4 of 15)
+      // columns per CTA from the largest possible r_t (at most 16 CTAs a subdomain)
+      const int cl = std::max(1, std::min(16, 2 * P.nsm / std::max(1, nsub)));
+      const int cols = (std::min(P.r_aug_max, RC) + cl - 1) / cl;
+      k_sstep_cols<<<nsub * cl, DD_THREADS, sstep_cols_smem(RC, cols), st>>>(P, B, axis, cl, cols);
+      k_sstep_back<<<nsub * CL, DD_THREADS, 0, st>>>(P, B, CL);
+    } else {
+      const int nst = P.integrator == 1 ? 4 : 1;
+      for (int s = 0; s < nst; ++s)
+        k_sstep_adv<<<nsub * CL, DD_THREADS, sstep_smem(RC), st>>>(P, B, axis, s, CL);
+    }
   }
   pend(st);
   // 9. L-step
