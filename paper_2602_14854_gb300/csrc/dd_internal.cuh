@@ -80,23 +80,6 @@ __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-template <typename T>
-__device__ __forceinline__ T warp_sum_t(T v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-template <typename T>
-__device__ __forceinline__ T warp_max_t(T v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-__device__ __forceinline__ double warp_max(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
 // Block-wide sum returned to every thread; red must hold >= 33 doubles.
 __device__ __forceinline__ double block_sum(double v, double* red) {
   int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
@@ -140,36 +123,6 @@ __device__ __forceinline__ void block_sum3f(float* a, float* b, float* c, float*
   }
   __syncthreads();
   *a = red[96]; *b = red[97]; *c = red[98];
-}
-__device__ __forceinline__ double block_max(double v, double* red) {
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  v = warp_max(v);
-  __syncthreads();
-  if (lane == 0) red[wid] = v;
-  __syncthreads();
-  if (wid == 0) {
-    double t = (lane < nw) ? red[lane] : 0.0;
-    t = warp_max(t);
-    if (lane == 0) red[32] = t;
-  }
-  __syncthreads();
-  return red[32];
-}
-
-// Stable descending order of v[0..n) by ranks (block-wide, one thread per entry):
-// perm[t] is the index of the t-th largest value, ties by index.  NaN ranks as
-// -infinity, so perm is a permutation for any input.
-__device__ __forceinline__ double rank_key(double x) { return x == x ? x : -INFINITY; }
-__device__ __forceinline__ void rank_sort_desc(const double* v, int n, int* perm) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double x = rank_key(v[i]);
-    int r = 0;
-    for (int j = 0; j < n; ++j) {
-      const double y = rank_key(v[j]);
-      r += (y > x) || (y == x && j < i);
-    }
-    perm[r] = i;
-  }
 }
 
 // The same order for non-negative, non-NaN values, compared by their bit patterns
@@ -278,12 +231,8 @@ __device__ __forceinline__ float2 df_from_double(double x) {
   return make_float2(h, __double2float_rn(x - (double)h));
 }
 __device__ __forceinline__ double df_to_double(float2 a) { return (double)a.x + (double)a.y; }
-__device__ __forceinline__ float2 z2f() { return make_float2(0.f, 0.f); }
 __device__ __forceinline__ float2 df_shfl_xor(unsigned mask, float2 v, int o) {
   return make_float2(__shfl_xor_sync(mask, v.x, o), __shfl_xor_sync(mask, v.y, o));
-}
-__device__ __forceinline__ float2 df_shfl(unsigned mask, float2 v, int src) {
-  return make_float2(__shfl_sync(mask, v.x, src), __shfl_sync(mask, v.y, src));
 }
 
 }  // namespace dd

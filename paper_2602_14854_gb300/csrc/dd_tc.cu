@@ -501,40 +501,11 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_tc_gram(const __grid_constant
 // arithmetic runs in the kernel.
 //
 #define OZ_DIG 7
-#define OZ_WORKERS 512                       // 16 warps: loads, digits, epilogue
-#define OZ_THREADS (OZ_WORKERS + 32)         // + one warp that issues the MMAs
-#define OZ_WARPS (OZ_WORKERS / 32)
 #define OZ_NONE (-(1 << 20))                 // exponent of an all-zero row / column
 
 // biased FP64 exponent of x (0 for zero and subnormals)
 __device__ __forceinline__ int f64_bexp(double x) {
   return (int)((unsigned)(__double_as_longlong(x) >> 52) & 0x7ffu);
-}
-// The 7 digits of T = trunc(x 2^(56 - e)) (|x| < 2^e, so |T| < 2^56), T = sum_s d_s 2^(48 - 8 s),
-// as exact FP32 values, by integer operations: with the mantissa left-aligned (implicit bit
-// at bit 63) T is one right shift; adding 128 at each of the six low byte positions makes
-// every low byte of V = T + 0x808080808080 equal to d_s + 128 with the borrows and carries
-// of a balanced representation (d_s in [-128, 127] for s >= 1, and d_0 = V >> 48 in
-// [-256, 256]); byte b becomes the FP32 (0x4B4000bb = 1.5 2^23 + b) minus 1.5 2^23 + 128.
-// Signed T needs nothing more: the identity is modular.
-__device__ __forceinline__ void oz_digits(double x, int e, float* d) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  const unsigned hi = (unsigned)(u >> 32);
-  const int E = (int)((hi >> 20) & 0x7ffu);
-  const int sh = 1030 + e - E;                       // >= 8
-  const unsigned long long m = (u << 11) | 0x8000000000000000ull;
-  long long T = (E != 0 && sh < 64) ? (long long)(m >> sh) : 0ll;
-  if (hi >> 31) T = -T;
-  const unsigned long long V = (unsigned long long)T + 0x808080808080ull;
-  const unsigned vl = (unsigned)V, vh = (unsigned)(V >> 32);
-  const float c = 12583040.0f;                       // 1.5 2^23 + 128
-  d[6] = __int_as_float((int)__byte_perm(vl, 0x4B400000u, 0x7650)) - c;
-  d[5] = __int_as_float((int)__byte_perm(vl, 0x4B400000u, 0x7651)) - c;
-  d[4] = __int_as_float((int)__byte_perm(vl, 0x4B400000u, 0x7652)) - c;
-  d[3] = __int_as_float((int)__byte_perm(vl, 0x4B400000u, 0x7653)) - c;
-  d[2] = __int_as_float((int)__byte_perm(vh, 0x4B400000u, 0x7650)) - c;
-  d[1] = __int_as_float((int)__byte_perm(vh, 0x4B400000u, 0x7651)) - c;
-  d[0] = __int_as_float(0x4B400000 + ((int)vh >> 16)) - 12582912.0f;
 }
 // the BF16 digits of two values packed in one word (each digit has <= 8 significant bits:
 // its BF16 is the top half of its FP32)
@@ -551,7 +522,7 @@ __device__ __forceinline__ uint32_t oz_pack(float lo, float hi) {
 // Conversion (integer and FP32 issue), the tensor cores and the epilogue (integer issue) of
 // different tiles overlap; before, all 16 worker warps converted a tile's digits, then all of
 // them ran the previous tile's epilogue, with CTA-wide barriers between, and issued on 40% of
-// the cycles.  262144 x 40 x 40 (64 subdomains, lda 60), per launch: 166 us before, 47 now.
+// the cycles.  262144 x 40 x 40 (64 subdomains, lda 60), per launch: 166 us before, 106 now.
 //
 // Digit planes of A: rows of 2 KP bytes (KP = the inner dimension rounded up to 16), plane s
 // of a stage at s APL; two stages while KP <= 48, one for KP = 64.  M: for column chunk c of
@@ -590,10 +561,15 @@ __device__ __forceinline__ bool ot_conv_all(bool p) {
   return r != 0;
 }
 
-// The digits of oz_digits for two values, packed: word s holds the BF16 digits s of x0 (low
-// half) and x1.  A low byte b = d + 128 becomes d in BF16 by two logic operations and one
-// packed subtraction: 128 + (b & 127) is 0x4300 | (b & 127), and what has to come off it is
-// 128 where bit 7 of b is set, else 256: 0x4300 | (~b & 128).
+// The 7 digits of T = trunc(x 2^(56 - e)) (|x| < 2^e, so |T| < 2^56), T = sum_s d_s 2^(48 - 8 s),
+// of two values, packed: word s holds the BF16 digits s of x0 (low half) and x1.  By integer
+// operations: with the mantissa left-aligned (implicit bit at bit 63) T is one right shift;
+// adding 128 at each of the six low byte positions makes every low byte of
+// V = T + 0x808080808080 equal to d_s + 128 with the borrows and carries of a balanced
+// representation (d_s in [-128, 127] for s >= 1, and d_0 = V >> 48 in [-256, 256]).  Signed T
+// needs nothing more: the identity is modular.  A low byte b = d + 128 becomes d in BF16 by two
+// logic operations and one packed subtraction: 128 + (b & 127) is 0x4300 | (b & 127), and what
+// has to come off it is 128 where bit 7 of b is set, else 256: 0x4300 | (~b & 128).
 __device__ __forceinline__ void oz_digits2(double x0, int e0, double x1, int e1, uint32_t* w) {
   uint32_t vl[2], vh[2];
 #pragma unroll
@@ -1075,16 +1051,18 @@ __global__ void __launch_bounds__(OT_THREADS, 1) k_oz_tall(TcTall a) {
 //
 // One CTA per SM, its warps specialised, each CTA walking a contiguous range of items of about
 // equal cost:
-//   16 converter warps 8 x 8 blocks of an operand -> registers (a stage ahead) -> digit planes
+//   8 converter warps  8 x 8 blocks of an operand -> registers (a stage ahead) -> digit planes
 //                      (a warp's 32 stores of a plane are 128 consecutive bytes);
 //   8 auxiliary warps  the column bounds of the item after the one being converted, then the
 //                      read-out of the item before it;
 //   1 MMA warp.
 // The FP64 pipe does 2 operations per clock and SM, which made these products the largest part
 // of a step with the rank at 20 (r_t = 40): spatial coefficients of 262144 x 40, per launch:
-// 1700 us on the FP64 pipe, 190 now; the angular ones (131072 directions) 1300 -> 230; an
-// orthonormalisation's Gram 271 on the FP64 pipe, 150 with this scheme but CTA-wide phases, 38
-// now.
+// 1700 us on the FP64 pipe, 470 now; the angular ones (131072 directions) 1300 -> 620; an
+// orthonormalisation's Gram 271 on the FP64 pipe, 150 with this scheme but CTA-wide phases, 85
+// (angular) to 140 (spatial) now.  Bound by instruction issue: 45% of the cycles, a third of the
+// stalls for instructions (the roles' code together), the rest loads; 25 warps with the bounds
+// and the read-out apart (72 registers, spills) were 25% slower, 16 converter warps 7%.
 #define OG_KS 32                          // rows per stage (K of one stage's MMAs)
 #define OG_GROUP 256                      // rows per read-out
 #define OG_RING 4                         // items whose column exponents are kept
