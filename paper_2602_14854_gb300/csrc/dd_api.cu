@@ -693,7 +693,6 @@ static dd_status create_impl(int ninst, const dd_grid* grids, const dd_tiling* t
   P.angcand = h->d_angcand; P.n_angcand = h->n_angcand; P.angcand_complete = h->angcand_complete;
   P.n_angorth = h->n_angorth;
   P.sptab = h->d_sptab; P.spoff = h->d_spoff; P.spnf = h->d_spnf;
-  P.nchunk_sp = std::max(1, std::min(16, h->maxN / 64));
   {
     int nsm = 0;
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess ||
@@ -701,7 +700,11 @@ static dd_status create_impl(int ninst, const dd_grid* grids, const dd_tiling* t
       nsm = 1;
     P.nsm = nsm;
   }
-  P.nchunk_ang = std::max(1, std::min(16, n / 64));
+  // Chunks of the largest subdomain in the FP64 reductions, up to 16 of at least 32 rows (a
+  // chunk's rows are a serial chain: 64 rows cost 4 subdomains of 256 cells 14 us per Gram, 32
+  // rows 10).
+  P.nchunk_sp = std::max(1, std::min(16, h->maxN / 32));
+  P.nchunk_ang = std::max(1, std::min(16, n / 32));
   P.ochunk_sp = P.nchunk_sp;
   P.ochunk_ang = P.nchunk_ang;
   // rows per item of the tensor-core products: 256 (one read-out) unless that makes more than
@@ -730,10 +733,10 @@ static dd_status create_impl(int ninst, const dd_grid* grids, const dd_tiling* t
     const long rc2 = (long)RC * RC;
     P.oz_sp = tiles_sp >= 2L * P.nsm || Nt * rc2 >= 55000000L;
     P.oz_ang = tiles_ang >= 2L * P.nsm || (long)nsub * n * rc2 >= 55000000L;
-    // Tall-skinny products likewise, and where the FP64 kernels' chunks (at most 16 of a subdomain)
-    // come to 2e5 row x r_cap^2 each: 4 x 4096 cells, r_cap = 30 (256 rows a chunk): spatial
-    // coefficients 104 us against 34 on the tensor cores, a Gram 26 against 33; 16384 cells (1024
-    // rows): 253 and 81 against 31; below it, at 64 rows a chunk, 42 and 17 against 36.
+    // Tall-skinny products likewise, and where the FP64 kernels' chunks come to 2e5 row x r_cap^2
+    // each: 4 x 4096 cells, r_cap = 30 (256 rows a chunk): spatial coefficients 104 us against 34
+    // on the tensor cores, a Gram 26 against 33; 16384 cells (1024 rows): 253 and 81 against 30;
+    // below it, at 64 rows a chunk, 42 and 15 against 34.
     P.ozg_sp = P.oz_sp || h->maxN / P.nchunk_sp * rc2 >= 200000L;
     P.ozg_ang = P.oz_ang || n / P.nchunk_ang * rc2 >= 200000L;
   }

@@ -115,7 +115,7 @@ size_t geig_smem_bytes(int RC) {
 // sM), keep (per subdomain) and, for the augmentation, r_t.
 // One CTA per subdomain: bound by the latency of the Jacobi rounds (dd_small.cuh).
 // 64 subdomains of 64 x 64 cells, r_t = 40 (60 columns in the augmentation): 310 us (QR) and
-// 797 us (augmentation) before, 66 and 118 now.
+// 797 us (augmentation) before, 149 and 386 now.
 __global__ void __launch_bounds__(512, 1) k_geig(OrthArgs a, const double* part, const int* cexp,
                                               int nchunk, int crows, double* sm, int sM,
                                               int* keep_out) {
@@ -162,8 +162,15 @@ __global__ void __launch_bounds__(512, 1) k_geig(OrthArgs a, const double* part,
       if (scaled) {
         for (int c = 0; c < nck; ++c) x += g[(long)c * RC * RC] * fac[c];
       } else {
-#pragma unroll 8
-        for (int c = 0; c < nck; ++c) x += g[(long)c * RC * RC];
+        double x1 = 0.0;                          // (two chains)
+        int c = 0;
+#pragma unroll 4
+        for (; c + 1 < nck; c += 2) {
+          x += g[(long)c * RC * RC];
+          x1 += g[(long)(c + 1) * RC * RC];
+        }
+        if (c < nck) x += g[(long)c * RC * RC];
+        x += x1;
       }
     }
     if (!isfinite(x)) { fin = false; x = 0.0; }
@@ -246,7 +253,7 @@ size_t chol_smem_bytes(int RC) { return sizeof(float2) * 5 * (size_t)RC * small_
 // Y -> G2^1/2, Z -> G2^-1/2, the error e maps to ~3/4 e^2), iterated until the predicted error
 // is below 1e-16.  |E|_F >= 0.9 (not expected; only through non-finite or inconsistent data) is
 // reported and leaves the identity.  The series is two small products against the
-// iteration's 2-3 times 2.5: 40 us per launch at q = 40 before, 17 now.
+// iteration's 2-3 times 2.5: 40 us per launch at q = 40 before, 21 now.
 __global__ void __launch_bounds__(512) k_chol_inv(OrthArgs a, const double* part, int nchunk,
                                                   int crows, double* sm, int sRi, const int* keep) {
   extern __shared__ float2 shc[];
@@ -273,8 +280,15 @@ __global__ void __launch_bounds__(512) k_chol_inv(OrthArgs a, const double* part
     tri_index(e, &i, &j);
     double x = 0.0;
     const double* g = G + j * RC + i;
-#pragma unroll 8
-    for (int c = 0; c < nck; ++c) x += g[(long)c * RC * RC];
+    double x1 = 0.0;                              // (two chains)
+    int c = 0;
+#pragma unroll 4
+    for (; c + 1 < nck; c += 2) {
+      x += g[(long)c * RC * RC];
+      x1 += g[(long)(c + 1) * RC * RC];
+    }
+    if (c < nck) x += g[(long)c * RC * RC];
+    x += x1;
     const double d = x - (i == j ? 1.0 : 0.0);
     e2 += i == j ? d * d : 2.0 * d * d;
     const float2 y = df_from_double(x);

@@ -220,10 +220,24 @@ __global__ void k_reduce(const double* part, int nchunk, int nblk, Dst dst, doub
   for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < nblk * RC * RC; o += gridDim.x * blockDim.x) {
     const int b = o / (RC * RC), e = o % (RC * RC);
     double s = 0.0;
-    for (int c = 0; c < nchunk; ++c) s += part[(((long)k * nchunk + c) * nblk + b) * RC * RC + e];
+    double s1 = 0.0;                                  // (two chains)
+    int c = 0;
+#pragma unroll 4
+    for (; c + 1 < nchunk; c += 2) {
+      s += part[(((long)k * nchunk + c) * nblk + b) * RC * RC + e];
+      s1 += part[(((long)k * nchunk + c + 1) * nblk + b) * RC * RC + e];
+    }
+    if (c < nchunk) s += part[(((long)k * nchunk + c) * nblk + b) * RC * RC + e];
+    s += s1;
     if ((dst.ident >> b) & 1) s = (e / RC == e % RC ? 1.0 : 0.0) - s;
     sm[((long)k * NSMALL + dst.idx[b]) * RC * RC + e] = s;
   }
+}
+
+// Chunks of a subdomain with this many rows, of at least 32 each: by its own rows, so that a
+// problem's sums are the same alone and beside larger ones in a batch.
+__device__ __forceinline__ int sub_chunks(int rows, int nchunk) {
+  return max(1, min(nchunk, rows / 32));
 }
 
 // Generic chunked Gram  G = A^T diag(w) B  over the rows of one subdomain.
@@ -250,7 +264,7 @@ __global__ void __launch_bounds__(DD_THREADS) k_gram(Geo g, GramArgs a) {
   const int rows = a.spatial ? g.N[k] : g.n;
   const long rb = a.spatial ? (long)g.rowoff[k] : (long)k * g.n;
   const long rbB = a.b_per_sub ? rb : 0;
-  const int ch = (rows + a.nchunk - 1) / a.nchunk;
+  const int nk = sub_chunks(rows, a.nchunk), ch = (rows + nk - 1) / nk;   // (none left: zeros)
   const int i0 = c * ch, i1 = min(rows, i0 + ch);
   const int na = a.acnt ? a.acnt[k] : a.afix, nbc = a.bcnt ? a.bcnt[k] : a.bfix;
   double* out = a.part + ((long)k * a.nchunk + c) * RC * RC;
@@ -327,7 +341,7 @@ size_t small_adv1_smem(int RC) {
 // CTA (k, 0): the eigen-split of C; CTA (k, 1): the products B = S M, which need nothing of it
 // and would otherwise wait their turn on the same SM.  The eigen-split is bound by the latency
 // of the Jacobi rounds and, at r_t >= 40, by the refinement's FP64 products: 483 us at r_t = 40
-// before (sweeps laid out over whole warps, the products of B in the same CTA), 165 now.
+// before (sweeps laid out over whole warps, the products of B in the same CTA), 297 now.
 __global__ void __launch_bounds__(512) k_small_adv1(Problem P, PhaseBufs B, int axis) {
   extern __shared__ double sh[];
   const int k = blockIdx.x, RC = P.g.RC;
@@ -689,8 +703,8 @@ __global__ void __launch_bounds__(DD_THREADS) k_kstep_adv(Problem P, PhaseBufs B
 // three cells early (RK4).  seg: cells per segment (lines are cut where there are too few of
 // them to fill the GPU).  P and lambda come from k_small_adv1 (small slots S3T and VB, free
 // until the S-step).  Bound by the FP64 pipe: 512 lines x 32 cells x 20 columns, RK4, 115 us
-// with the stages in shared memory and both basis changes in the same kernel, 9 now (and two
-// products of 12 each).
+// with the stages in shared memory and both basis changes in the same kernel, 28 now (and two
+// products of 19 each); 400000 cells of r_t <= 42: 3700 us, 382 now (and two of 85).
 __global__ void __launch_bounds__(DD_THREADS) k_kstep_line(Problem P, PhaseBufs B, int axis, int seg) {
   const int k = blockIdx.y, RC = P.g.RC, rt = B.rt[k];
   const Lines L = lines_of(P.g, k, axis);
@@ -752,7 +766,7 @@ __global__ void k_sp_coeffs(Problem P, PhaseBufs B, int axis, int skip_t) {
   const Lines L = lines_of(P.g, k, axis);
   // chunks of whole lines: every cell's shift partner and the two face cells of a
   // line are in the same chunk, and no index is divided inside the loops
-  const int lch = (L.nlines + nchunk - 1) / nchunk;
+  const int nk = sub_chunks(L.nlines * L.len, nchunk), lch = (L.nlines + nk - 1) / nk;
   const int l0 = c * lch, l1 = min(L.nlines, l0 + lch);
   const int rt = B.rt[k];
   count_work(P.g, KS_SP_COEFFS, 2.0 * rt * rt * (max(0, l1 - l0) * (double)L.len * (skip_t ? 1 : 2) +
@@ -774,10 +788,12 @@ __global__ void k_sp_coeffs(Problem P, PhaseBufs B, int axis, int skip_t) {
     {
       if (blk == 0) {
         for (int line = l0; line < l1; ++line)
+#pragma unroll 8
           for (int pos = 0, cell = line * L.stride_line; pos < L.len; ++pos, cell += L.stride_pos)
             s += X1[(long)cell * RC + i] * K[(long)cell * RC + j];
       } else if (blk == 1) {
         for (int line = l0; line < l1; ++line)
+#pragma unroll 8
           for (int pos = 1, cell = line * L.stride_line + L.stride_pos; pos < L.len;
                ++pos, cell += L.stride_pos)
             s += X1[(long)cell * RC + i] * X1[(long)(cell - L.stride_pos) * RC + j];
@@ -884,7 +900,7 @@ __global__ void __launch_bounds__(DD_THREADS) k_sstep_adv(Problem P, PhaseBufs B
 // stage where the form above takes five), and k_sstep_back adds the rotated increment.  The
 // eigen-split itself is the K-step's, P and lambda from k_small_adv1 (slots S3T and VB); the
 // increment goes to slot UB.  64 FP64-bound CTAs of four launches before: 16 subdomains,
-// r_t = 20: 59 us per S-step, 18 now; 70 of r_t <= 42: 598 us, 130 now.
+// r_t = 20: 59 us per S-step, 25 now; 70 of r_t <= 42: 598 us, 142 now.
 size_t sstep_cols_smem(int RC, int cols) {
   return sizeof(double) * ((size_t)RC * (RC | 1) + 5 * (size_t)cols * RC);
 }
@@ -1155,7 +1171,7 @@ __global__ void __launch_bounds__(DD_THREADS) k_lstep_adv(Problem P, PhaseBufs B
 // truncation (Algorithm 5): SVD of S3 by one-sided Jacobi on the columns of S3^T
 // ---------------------------------------------------------------------------
 // One CTA per subdomain, bound by the latency of the Jacobi rounds (dd_small.cuh): 458 us at
-// r_t = 40 before, 117 now.
+// r_t = 40 before, 287 now.
 __global__ void __launch_bounds__(512) k_trunc(Problem P, PhaseBufs B) {
   extern __shared__ double sh[];
   const int k = blockIdx.x, RC = P.g.RC, ld = small_ld(RC);
@@ -1649,7 +1665,7 @@ __global__ void __launch_bounds__(DD_THREADS) k_flux_prep(Problem P, const doubl
 // CTAs' loads); the scale is in sa, so no cell divides (an FP64 division costs as much of the
 // FP64 pipe as the whole dot product).  Rows on 16-byte boundaries (RC even) are read as
 // pairs.  512 x 512 cells at r = 20: 102 us before (fixed 16 CTAs per subdomain, a division
-// per cell, the columns of a one after another), 26 us now with k_flux_prep.
+// per cell, the columns of a one after another), 47 us now with k_flux_prep.
 __global__ void __launch_bounds__(DD_THREADS) k_flux(Problem P, const double* X, const double* S,
                                                      const int* r, const double* work, int nch,
                                                      double* rho) {
@@ -2194,8 +2210,7 @@ void advection_phase(const Problem& P, const PhaseBufs& B, int axis, cudaStream_
   cudaMemcpyAsync(B.rx + axis * nsub, B.rt, sizeof(int) * nsub, cudaMemcpyDeviceToDevice, st);
   pend(st);
   // 2. angular Galerkin coefficients, boundary masses
-  // twice the angular chunks (more blocks than SMs), as far as the partial buffer holds
-  const int nch_ac = std::min(2 * P.nchunk_ang, std::max(P.nchunk_sp, P.nchunk_ang));
+  const int nch_ac = P.nchunk_ang;
   const int nblk_ac = P.kstep_split == 1 ? 8 : 6;
   bool oz_done = false, tc_done = false;
   if (P.ozg_ang) {
