@@ -17,13 +17,13 @@
 // subdomain):
 //   G1 = A^T A                      chunked Gram (k_gram; partials summed by k_geig)
 //   G1 = V diag(lambda) V^T         k_geig: pivoted Cholesky G1 = X X^T, one-sided
-//                                   Jacobi on X (FP32 sweeps, double-float finish),
-//                                   one FP64 refinement; sigma_j = lambda_j^1/2 give
-//                                   the rank decision; M = V_keep diag(sigma)^-1
+//                                   Jacobi on X (FP32 sweeps, double-float finish);
+//                                   sigma_j = lambda_j^1/2 give the rank decision;
+//                                   M = V_keep diag(sigma)^-1
 //   U1 = A M                        k_tall: the leading left singular vectors, up to
 //                                   errors of order eps |A|^2 / sigma_j^2
-//   G2 = U1^T U1                    k_gram + k_chol_inv (G2^-1/2 by Newton-Schulz in
-//                                   double-float)
+//   G2 = U1^T U1                    k_gram + k_chol_inv (G2^-1/2 by a series in
+//                                   G2 - I, or Newton-Schulz in double-float)
 //   Q  = U1 G2^-1/2                 k_tall: orthonormal to ~1e-14
 //   completion                      k_kc_w / k_kca_w, k_kc_sel, k_kc_apply (QR and
 //                                   augmentation: Gram-Schmidt in coefficient space),
