@@ -107,7 +107,9 @@ enum { DD_EULER = 0, DD_RK4 = 1 };
  * The orthonormalisations, the small SVDs and eigendecompositions, the advection K-step
  * (Appendix A's eigenbasis form) and the storage stay FP64.  With physical inflow the
  * angular coefficients stay FP64.  The advection K-step is FP64 in every form except the
- * matrix stencil of the flux-split form outside DD_FP64. */
+ * matrix stencil of the flux-split form outside DD_FP64.  Where a row family's FP64 products
+ * run on the tensor cores (products below), these contractions take that FP64-accurate form
+ * in DD_TF32 and DD_BF16 too. */
 enum { DD_FP64 = 0, DD_MIXED = 1, DD_TF32 = 2, DD_BF16 = 3 };
 
 typedef struct dd_options {
