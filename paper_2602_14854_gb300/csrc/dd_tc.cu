@@ -1606,11 +1606,13 @@ __global__ void __launch_bounds__(OG_THREADS, 1) k_oz_gram(const __grid_constant
 }
 
 // Sum of the chunk partials of every product, in chunk order, into the small matrices (slot
-// dst[blk]), zero outside the product's na x nb entries.
+// dst[blk]), zero outside the product's na x nb entries.  Grid: (entries, subdomains, products):
+// y ends at 65535, so the products have a dimension of their own and this kernel takes as many
+// subdomains as every other one.
 __global__ void __launch_bounds__(DD_THREADS) k_oz_reduce(const __grid_constant__ OzGram a, OzDst dst,
                                                           double* sm) {
-  const int k = blockIdx.y / a.nprod, RC = a.g.RC;
-  const OzProd& p = a.p[blockIdx.y - k * a.nprod];
+  const int k = blockIdx.y, RC = a.g.RC;
+  const OzProd& p = a.p[blockIdx.z];
   int rows, na, nb;
   og_shape(a, k, p, &rows, &na, &nb);
   const int nck = og_chunks(a, rows);
@@ -1768,7 +1770,7 @@ bool oz_gram(const Problem& P, cudaStream_t st, OzGram& a, const OzDst* dst, dou
   pend(st);
   if (dst) {
     pbeg(st, KS_REDUCE);
-    k_oz_reduce<<<dim3((P.g.RC * P.g.RC + DD_THREADS - 1) / DD_THREADS, P.g.nsub * a.nprod), DD_THREADS, 0, st>>>(
+    k_oz_reduce<<<dim3((P.g.RC * P.g.RC + DD_THREADS - 1) / DD_THREADS, P.g.nsub, a.nprod), DD_THREADS, 0, st>>>(
         a, *dst, sm);
     pend(st);
   }
