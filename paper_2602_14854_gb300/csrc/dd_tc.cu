@@ -502,6 +502,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_tc_gram(const __grid_constant
 //
 #define OZ_DIG 7
 #define OZ_NONE (-(1 << 20))                 // exponent of an all-zero row / column
+#define OZ_BAD (1 << 21)                     // of one with a NaN or an infinity (above -OZ_NONE)
 
 // biased FP64 exponent of x (0 for zero and subnormals)
 __device__ __forceinline__ int f64_bexp(double x) {
@@ -664,6 +665,8 @@ __device__ __forceinline__ void ot_load(double2 (&d)[8], const double* row, int 
   else ot_load<8>(d, row, q, lda);
 }
 // Their digit planes (row r of the stage asl, planes APL apart) and the row bound (lanes q = 0).
+// A row with a NaN or an infinity has the bound OZ_BAD and no digits (as fixed-point numbers they
+// would come out as large finite values); the epilogue makes its products NaN.
 // One body per KP: with the column count a run-time bound every pair of values sat in a branch
 // of its own and waited for the one before (7 clocks per instruction and warp; the converters
 // took 12000 clocks per tile).
@@ -671,17 +674,17 @@ template <int C>
 __device__ __forceinline__ void ot_convert(const double2 (&x)[8], const int* mexp, int ni, int q, int r,
                                            uint8_t* asl, uint32_t APL, int* rexp) {
   int2 me[C];
-  int mx = OZ_NONE;
+  int mx = OZ_NONE, top = 0;
 #pragma unroll
   for (int c = 0; c < C; ++c) {
     const int kk = 8 * c + 2 * q;
-    me[c] = *reinterpret_cast<const int2*>(mexp + kk);
-    if (kk >= ni) me[c].x = OZ_NONE;             // past ni, or zero rows of M: the digits are zero
-    if (kk + 1 >= ni) me[c].y = OZ_NONE;
-    const int E0 = f64_bexp(x[c].x), E1 = f64_bexp(x[c].y);
+    me[c] = *reinterpret_cast<const int2*>(mexp + kk);   // OZ_NONE past ni and for zero rows of M
+    const int E0 = kk < ni ? f64_bexp(x[c].x) : 0, E1 = kk + 1 < ni ? f64_bexp(x[c].y) : 0;
+    top = max(top, max(E0, E1));
     mx = max(mx, E0 && me[c].x != OZ_NONE ? E0 - 1022 + me[c].x : OZ_NONE);
     mx = max(mx, E1 && me[c].y != OZ_NONE ? E1 - 1022 + me[c].y : OZ_NONE);
   }
+  if (top == 0x7ff) mx = OZ_BAD;
   mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
   mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
   if (q == 0) rexp[r] = mx;
@@ -830,7 +833,8 @@ __global__ void __launch_bounds__(OT_THREADS, 1) k_oz_tall(TcTall a) {
         ot_conv_sync();
         for (int kk = warp; kk < s.KP; kk += OT_CONV) {    // mu_k: warp per row
           const int E0 = f64_bexp(Ms[kk * DD_MAXC + lane]), E1 = f64_bexp(Ms[kk * DD_MAXC + lane + 32]);
-          const int mx = __reduce_max_sync(0xffffffffu, max(E0 ? E0 - 1022 : OZ_NONE, E1 ? E1 - 1022 : OZ_NONE));
+          const int mx = __reduce_max_sync(0xffffffffu, max(E0 && E0 != 0x7ff ? E0 - 1022 : OZ_NONE,
+                                                            E1 && E1 != 0x7ff ? E1 - 1022 : OZ_NONE));
           if (lane == 0) mexp[kk] = mx;
         }
         ot_conv_sync();
@@ -839,7 +843,7 @@ __global__ void __launch_bounds__(OT_THREADS, 1) k_oz_tall(TcTall a) {
           int mx = OZ_NONE;
           for (int kk = p; kk < s.ni; kk += OT_CONV / 2) {
             const int E = f64_bexp(Ms[kk * DD_MAXC + n]);
-            if (E) mx = max(mx, E - 1022 - mexp[kk]);
+            if (E) mx = max(mx, E != 0x7ff ? E - 1022 - mexp[kk] : OZ_BAD);
           }
           red[p][n] = mx;
         }
@@ -942,7 +946,9 @@ __global__ void __launch_bounds__(OT_THREADS, 1) k_oz_tall(TcTall a) {
           double v[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            v[i] = oz_round(oz_combine(&D[0][i], 4), er + fexp[slot][c0 + i] - 56);
+            const int sc = er + fexp[slot][c0 + i] - 56;
+            v[i] = oz_round(oz_combine(&D[0][i], 4), sc);
+            if (sc > OZ_BAD / 4) v[i] = __longlong_as_double(0x7ff8000000000000ll);
             if (c0 + i >= s.nc) v[i] = 0.0;
           }
           if (!in) continue;
