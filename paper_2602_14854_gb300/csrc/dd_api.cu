@@ -850,8 +850,16 @@ dd_status dd_dlra_step(dd_dlra_t h, int nsteps) {
       h->stream = cap;
       cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
+        // a launch that the runtime refuses is missing from the graph, which is then never run
+        const bool clean = cudaPeekAtLastError() == cudaSuccess;
         enqueue_step(h);
+        const cudaError_t refused = clean ? cudaGetLastError() : cudaSuccess;
         e = cudaStreamEndCapture(cap, &graph);
+        if (refused != cudaSuccess) {
+          if (e == cudaSuccess) cudaGraphDestroy(graph);
+          e = refused;
+          (void)cudaGetLastError();
+        }
       }
       h->stream = user;
       cudaStreamDestroy(cap);
