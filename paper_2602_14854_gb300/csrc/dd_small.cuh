@@ -688,6 +688,7 @@ __device__ __forceinline__ int pchol(double* A, double* X, int m, int ld, double
 // The smallest r whose tail (sum_{t >= r} sigma_t^2)^1/2 is within tol, for n <= 64 values by
 // val(t), descending (one warp; every lane returns it).  A suffix sum over the lanes: 13
 // dependent FP64 operations, where a sum per r afresh took n^2 / 2 and a square root each.
+// (The root is compared, not the square with tol^2: a tolerance below zero cuts nothing.)
 template <class F>
 __device__ __forceinline__ int tail_rank(int n, double tol, F val) {
   const int lane = threadIdx.x & 31;
@@ -700,9 +701,8 @@ __device__ __forceinline__ int tail_rank(int n, double tol, F val) {
     if (lane + o < 32) { a += u; b += v; }
   }
   a += __shfl_sync(0xffffffffu, b, 0);
-  const double t2 = tol * tol;
-  const unsigned in0 = __ballot_sync(0xffffffffu, a <= t2 || lane >= n);
-  const unsigned in1 = __ballot_sync(0xffffffffu, b <= t2 || lane + 32 >= n);
+  const unsigned in0 = __ballot_sync(0xffffffffu, sqrt(a) <= tol || lane >= n);
+  const unsigned in1 = __ballot_sync(0xffffffffu, sqrt(b) <= tol || lane + 32 >= n);
   if (in0) return min(n, __ffs(in0) - 1);
   if (in1) return min(n, 31 + __ffs(in1));
   return n;
