@@ -2004,8 +2004,15 @@ cudaError_t autotune(Problem& P, const PhaseBufs& B, cudaStream_t st, int tune_p
   for (int i = 0; i < 8; ++i) ms[i] = -1.0;
   if (!tune_products && !tune_chunks) return cudaSuccess;
   const int RC = P.g.RC, nsub = P.g.nsub;
-  const std::vector<long> key = {nsub, P.maxN, P.g.n, RC, P.prec, P.Ntot, tune_products,
-                                 tune_chunks, P.ochunk_sp, P.ochunk_ang};
+  int dev = 0;
+  {
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+  }
+  // (engines that are not tuned are the caller's: what is timed then is theirs alone)
+  const std::vector<long> key = {dev, nsub, P.maxN, P.g.n, RC, P.prec, P.Ntot, tune_products,
+                                 tune_chunks, P.ochunk_sp, P.ochunk_ang, P.ocrows_sp, P.ocrows_ang,
+                                 tune_products ? -1 : P.ozg_sp, tune_products ? -1 : P.ozg_ang};
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune_cache.find(key);
