@@ -137,7 +137,9 @@ __global__ void __launch_bounds__(512, 1) k_geig(OrthArgs a, const double* part,
   float* J32 = B32 + (size_t)ldf * (ldf - 4);
   int* perm = reinterpret_cast<int*>(nrm + RC);
   // the chunk partials are Grams of 2^-e_c A: G1 of 2^-emax A is their sum with
-  // weights 4^(e_c - emax)
+  // weights 4^(e_c - emax).  (INT_MIN: a chunk without rows or below 2^-1000, its partial is
+  // zero.  It does not make the others scaled: a subdomain beside larger ones of a batch has
+  // such chunks past its own, and is summed as it is alone.)
   __shared__ double fac[GRAM_CHUNKS];
   __shared__ int s_keep;
   int emax = INT_MIN;
@@ -145,7 +147,7 @@ __global__ void __launch_bounds__(512, 1) k_geig(OrthArgs a, const double* part,
   for (int c = 0; c < nck; ++c) {
     const int ec = cexp[(long)k * nchunk + c];
     emax = max(emax, ec);
-    scaled |= ec != 0;
+    scaled |= ec != 0 && ec != INT_MIN;
   }
   for (int c = tid; c < nck; c += blockDim.x) {
     const int ec = cexp[(long)k * nchunk + c];

@@ -234,8 +234,11 @@ __global__ void k_reduce(const double* part, int nchunk, int nblk, Dst dst, doub
   }
 }
 
-// Chunks of a subdomain with this many rows, of at least 32 each: by its own rows, so that a
-// problem's sums are the same alone and beside larger ones in a batch.
+// Chunks of a subdomain with this many rows, of at least 32 each: by its own rows, so that in the
+// FP64 kernels a problem's sums are the same alone and beside larger ones in a batch while the
+// largest has at most 4096 rows (past that the second Gram of an orthonormalisation is not
+// formed with its product).  The engine and the tensor-core products' rows per item follow the
+// batch's totals: their results agree to FP64 rounding.
 __device__ __forceinline__ int sub_chunks(int rows, int nchunk) {
   return max(1, min(nchunk, rows / 32));
 }
