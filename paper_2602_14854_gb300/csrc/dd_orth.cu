@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(512, 1) k_geig(OrthArgs a, const double* part,
     for (int r = lane; r < ldf - 4; r += 32) {
       float2 x = make_float2(0.f, 0.f);
       if (r < m) {
-        x = df_split(X[c * ld + r] * f);
+        x = df_from_double(X[c * ld + r] * f);
         T[c * ld + r] = x;
       }
       B32[c * ldf + r] = x.x;
