@@ -92,31 +92,33 @@ __device__ __forceinline__ int orth_chunks(const OrthArgs& a, int k, int nchunk,
 
 // the vectors lam, sig, nrm and perm, padded to 16 bytes (the FP32 region follows)
 __host__ __device__ __forceinline__ size_t geig_vec_bytes(int RC) {
-  const size_t b = 4 * small_region(RC) + (sizeof(double) * 2 + sizeof(float2) + sizeof(int)) * RC;
-  return ((b + 15) & ~(size_t)15) - 4 * small_region(RC);
+  const size_t b = 3 * small_region(RC) + (sizeof(double) * 2 + sizeof(float2) + sizeof(int)) * RC;
+  return ((b + 15) & ~(size_t)15) - 3 * small_region(RC);
 }
 size_t geig_smem_bytes(int RC) {
-  return 4 * small_region(RC) + geig_vec_bytes(RC) + small_f32_region(RC);
+  return 3 * small_region(RC) + geig_vec_bytes(RC) + small_f32_region(RC);
 }
 
 // Singular values and leading right singular vectors of A from its Gram G1 (m x m, the sum of
 // the chunk partials): G1 = X X^T by pivoted Cholesky (columns graded), one-sided Jacobi on X:
 // the columns of X J = W are orthogonal, sigma_j = |w_j| and w_j / |w_j| are the eigenvectors of
-// G1 (jacobi_core, dd_small.cuh; double-float).  Jacobi on the graded factor takes a fraction of
-// the sweeps that Jacobi on G1 would.  One refinement step against G1 (refine_sym_eig) takes the
-// eigenpairs to the FP64 level.  On smooth data the step without it is as close to 64 bits
-// (densities 4.1e-15 off, 4.0e-15 with it); a narrow source amplifies the difference: after 10
-// steps of one on 256 x 256 cells the density is less than 3e-10 off the oracle's with it and 8e-9
-// to 9e-9 without, the same with every change of rounding elsewhere that was tried.  The
-// factor goes down to the rounding level of G1 (1e-16 of the largest diagonal entry, or 1/100 of
-// the squared rank threshold when that is smaller): what it leaves out, against eigenvalues of
-// tau^2 sigma_1^2 = 1e-10 sigma_1^2, turns the directions near the threshold (unrefined, 1e-13 cost
-// the density three digits; 1e-17 to 1e-20 change nothing).  Writes M = V_keep diag(sigma_keep)^-1
-// (row-major, slot sM), keep (per subdomain) and, for the augmentation, r_t.
-// One CTA per subdomain: bound by the latency of the Jacobi rounds (dd_small.cuh) and by the
-// refinement's FP64 products.  64 subdomains of 64 x 64 cells, r_t = 40 (60 columns in the
-// augmentation): 310 us (QR) and 797 us (augmentation) with the sweeps laid out over whole warps,
-// 183 and 510 now (149 and 365 of it without the refinement).
+// G1 (jacobi_core, dd_small.cuh).  Jacobi on the graded factor takes a fraction of the sweeps that
+// Jacobi on G1 would.  The eigenpairs are double-float: an error F in the orthogonality of J turns
+// into a relative error F sigma_i sigma_j in the coupling of w_i and w_j, where G1 itself carries
+// eps sigma_1^2.  An FP64 refinement step against G1 took 4% of a time step and changed no
+// accuracy.  Distance of a step's density from 64 bits, geometric means without it / with it / with
+// the refined eigensolver of other operands that came before: batch of ten problems (16 inputs)
+// 7.7e-13 / 9.4e-13 / 2.2e-12, checkerboard (12) 3.3e-11 / 4.5e-11 / 9.1e-11, 61 x 47 cells (24)
+// 5.8e-15 / 6.0e-15 / 6.9e-15, lognormal 512^2 (6) 1.3e-14 / 1.5e-14 / 1.6e-14, 32^2 cells (24)
+// 7.4e-15 / 6.7e-15 / 7.9e-15, the Hohlraum (24) 6.2e-15 / 6.3e-15 / 6.3e-15.  The factor
+// goes down to the rounding level of G1 (1e-16 of the largest diagonal entry, or 1/100 of the
+// squared rank threshold when that is smaller): what it leaves out, against eigenvalues of
+// tau^2 sigma_1^2 = 1e-10 sigma_1^2, turns the directions near the threshold (at 1e-13 by 1e-2,
+// which cost the density three digits).  Writes M = V_keep diag(sigma_keep)^-1 (row-major, slot
+// sM), keep (per subdomain) and, for the augmentation, r_t.
+// One CTA per subdomain: bound by the latency of the Jacobi rounds (dd_small.cuh).
+// 64 subdomains of 64 x 64 cells, r_t = 40 (60 columns in the augmentation): 310 us (QR) and
+// 797 us (augmentation) with the sweeps laid out over whole warps, 149 and 365 now.
 __global__ void __launch_bounds__(512, 1) k_geig(OrthArgs a, const double* part, const int* cexp,
                                               int nchunk, int crows, double* sm, int sM,
                                               int* keep_out) {
@@ -131,11 +133,10 @@ __global__ void __launch_bounds__(512, 1) k_geig(OrthArgs a, const double* part,
   double* X = A + (size_t)ld * RC;                  // pivot columns, then W
   const int ldf = small_ldf(RC);
   double* R3 = X + (size_t)ld * RC;                 // scratch of the Jacobi
-  double* G1 = R3 + (size_t)ld * RC;                // G1, kept for the refinement
-  double* lam = G1 + (size_t)ld * RC;               // sigma^2, by column
+  double* lam = X + 2 * (size_t)ld * RC;            // sigma^2, by column
   double* sig = lam + RC;                           // pivots, then singular values of A, descending
   float2* nrm = reinterpret_cast<float2*>(sig + RC);
-  float* B32 = reinterpret_cast<float*>(reinterpret_cast<char*>(shg) + 4 * small_region(RC) + geig_vec_bytes(RC));
+  float* B32 = reinterpret_cast<float*>(reinterpret_cast<char*>(shg) + 3 * small_region(RC) + geig_vec_bytes(RC));
   float* J32 = B32 + (size_t)ldf * (ldf - 4);
   int* perm = reinterpret_cast<int*>(nrm + RC);
   // the chunk partials are Grams of 2^-e_c A: G1 of 2^-emax A is their sum with
@@ -179,8 +180,6 @@ __global__ void __launch_bounds__(512, 1) k_geig(OrthArgs a, const double* part,
     }
     if (!isfinite(x)) { fin = false; x = 0.0; }
     A[j * ld + i] = x;
-    G1[j * ld + i] = x;
-    G1[i * ld + j] = x;
   }
   if (emax == INT_MIN) emax = 0;
   if (!fin) atomicOr(a.status, (unsigned)ST_NONFINITE);
@@ -207,20 +206,8 @@ __global__ void __launch_bounds__(512, 1) k_geig(OrthArgs a, const double* part,
   __syncthreads();
   jacobi_core<false>(T, B32, J32, X, R3, m, kr, ld, ldf, nrm);
   const float2* W = reinterpret_cast<const float2*>(X);
-  // one FP64 refinement step against G1, scaled like X: by 2^(-2 ex)
-  const double g2 = ldexp(1.0, -2 * ex);
-  for (int e = tid; e < m * m; e += blockDim.x) {
-    const int j = e / m, i = e - j * m;
-    G1[j * ld + i] *= g2;
-  }
-  for (int c = warp; c < kr; c += nw) {
-    const double f = nrm[c].x > 0.f ? rsqrt(df_to_double(nrm[c])) : 0.0;
-    for (int r = lane; r < m; r += 32) A[c * ld + r] = df_to_double(W[c * ld + r]) * f;
-  }
-  __syncthreads();
-  refine_sym_eig(G1, A, lam, m, kr, ld, X, R3, reinterpret_cast<double*>(B32));
   for (int j = tid; j < m; j += blockDim.x) {
-    const double l = j < kr && nrm[j].x != 0.f ? lam[j] : 0.0;   // (a zero column has no lambda)
+    const double l = j < kr ? df_to_double(nrm[j]) : 0.0;
     if (!isfinite(l)) atomicOr(a.status, (unsigned)ST_NONFINITE);
     lam[j] = l > 0.0 ? l : 0.0;
   }
@@ -240,22 +227,26 @@ __global__ void __launch_bounds__(512, 1) k_geig(OrthArgs a, const double* part,
   }
   __syncthreads();
   const int keep = s_keep;
-  // M = V_keep diag(sigma)^-1 for A itself: V 2^-(emax + ex) / sigma (sigma of the scaled A), the
-  // power of two in two halves
+  // M = V_keep diag(sigma)^-1 for A itself: the unit columns w / |w| times 1 / sigma and
+  // 2^-(emax + ex), the power of two in two halves (1 / (|w| sigma) alone may overflow)
   const int eh = (emax + ex) / 2;
   const double s2 = ldexp(1.0, -(emax + ex - eh));
-  for (int t = tid; t < keep; t += blockDim.x) sig[t] = ldexp(1.0 / sqrt(lam[perm[t]]), -eh);
+  for (int t = tid; t < keep; t += blockDim.x) {
+    const double l = lam[perm[t]];
+    sig[t] = ldexp(1.0 / sqrt(l), -eh);
+    lam[perm[t]] = rsqrt(l);
+  }
   __syncthreads();
   for (int t = warp; t < RC; t += nw) {
     const int c = t < keep ? perm[t] : 0;
-    const double f = t < keep ? sig[t] : 0.0;
+    const double n = lam[c], f = t < keep ? sig[t] : 0.0;
     for (int i = lane; i < RC; i += 32)
-      X[t * ld + i] = (i < m && t < keep) ? A[c * ld + i] * f * s2 : 0.0;
+      A[t * ld + i] = (i < m && t < keep) ? df_to_double(W[c * ld + i]) * n * f * s2 : 0.0;
   }
   __syncthreads();
   for (int e = tid; e < RC * RC; e += blockDim.x) {
     const int i = e / RC, t = e - i * RC;
-    M[e] = X[t * ld + i];
+    M[e] = A[t * ld + i];
   }
 }
 

@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(512) k_small_adv1(Problem P, PhaseBufs B, int 
     Pm[j * ld + i] = df_to_double(reinterpret_cast<const float2*>(R3)[j * ld + i]);
   }
   __syncthreads();
-  refine_sym_eig(R0, Pm, lam, rt, rt, ld, R2, R3, R4);
+  refine_sym_eig(R0, Pm, lam, rt, ld, R2, R3, R4);
   // C+ = P diag(max(l,0)) P^T, C- = C - C+, |C| = C+ - C- (upper triangles, mirrored)
   double* Cp = SMB(B, P, k, SM_CP);
   double* Cn = SMB(B, P, k, SM_CM);

@@ -700,32 +700,27 @@ __device__ __forceinline__ int tail_rank(int n, double tol, F val) {
 // Aishima, 2018): with R = I - V^T V, S = V^T G V, lambda_i = s_ii / (1 - r_ii),
 // V <- V (I + E), e_ij = (s_ij + lambda_j r_ij) / (lambda_j - lambda_i) for separated pairs,
 // r_ij / 2 within clusters and on the diagonal; the error of V maps to about its square.
-// G (nr x nr, symmetric) and V (nr x m, V_ij = V[j * ld + i], refined in place; with m < nr within
-// its span, whose complement G maps to rounding): leading dimension ld; lam: the m refined
-// eigenvalues (not sorted).  S and R are symmetric (upper triangles computed,
+// G (symmetric) and V (V_ij = V[j * ld + i], refined in place): leading dimension ld; lam: the
+// refined eigenvalues (not sorted).  S and R are symmetric (upper triangles computed,
 // mirrored); the norms that set the cluster threshold, the quotients of E (a first-order
 // correction) and the product V E are taken in FP32.  T, S, R: regions of scratch.  Block-wide.
-static __device__ __noinline__ void refine_sym_eig(const double* G, double* V, double* lam, int nr,
-                                                   int m, int ld, double* T, double* S, double* R) {
+static __device__ __noinline__ void refine_sym_eig(const double* G, double* V, double* lam, int m,
+                                                   int ld, double* T, double* S, double* R) {
   __shared__ double rred[50];            // >= 99 floats for block_sum3f
-  for (int e = threadIdx.x; e < nr * m; e += blockDim.x) {           // T = G V
-    const int j = e / nr, i = e - j * nr;
+  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {            // T = G V
+    const int j = e / m, i = e - j * m;
     double x = 0.0;
-    for (int l = 0; l < nr; ++l) x += G[l * ld + i] * V[j * ld + l];
+    for (int l = 0; l < m; ++l) x += G[l * ld + i] * V[j * ld + l];
     T[j * ld + i] = x;
   }
   __syncthreads();
   float offn = 0.f, rn = 0.f, gn = 0.f;
   const int ntri = m * (m + 1) / 2;
-  for (int e = threadIdx.x; e < nr * (nr + 1) / 2; e += blockDim.x) {   // S = V^T T, R = I - V^T V
+  for (int e = threadIdx.x; e < ntri; e += blockDim.x) {             // S = V^T T, R = I - V^T V
     int i, j;
     tri_index(e, &i, &j);
-    const float wgt = i == j ? 1.f : 2.f;
-    const float gf = (float)G[i * ld + j];
-    gn += wgt * gf * gf;
-    if (e >= ntri) continue;
     double x = 0.0, y = 0.0;
-    for (int l = 0; l < nr; ++l) {
+    for (int l = 0; l < m; ++l) {
       const double v = V[i * ld + l];
       x += v * T[j * ld + l];
       y += v * V[j * ld + l];
@@ -733,9 +728,11 @@ static __device__ __noinline__ void refine_sym_eig(const double* G, double* V, d
     const double rr = (i == j ? 1.0 : 0.0) - y;
     S[i * ld + j] = x; S[j * ld + i] = x;
     R[i * ld + j] = rr; R[j * ld + i] = rr;
-    const float xf = (float)x, rf = (float)rr;
+    const float xf = (float)x, rf = (float)rr, gf = (float)G[i * ld + j];
+    const float wgt = i == j ? 1.f : 2.f;
     if (i != j) offn += 2.f * xf * xf;
     rn += wgt * rf * rf;
+    gn += wgt * gf * gf;
   }
   block_sum3f(&offn, &rn, &gn, reinterpret_cast<float*>(rred));
   const float delta = 2.f * (sqrtf(offn) + sqrtf(gn) * sqrtf(rn));   // cluster separation
@@ -753,15 +750,15 @@ static __device__ __noinline__ void refine_sym_eig(const double* G, double* V, d
   }
   __syncthreads();
   float* Vf = reinterpret_cast<float*>(R);      // V in FP32 (R is dead)
-  for (int e = threadIdx.x; e < nr * m; e += blockDim.x) {
-    const int j = e / nr, i = e - j * nr;
+  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
+    const int j = e / m, i = e - j * m;
     Vf[j * ld + i] = (float)V[j * ld + i];
   }
   __syncthreads();
   // V + V E with the correction V E in FP32 (E is itself a first-order FP32 quantity of the
   // size of V's error, so FP32 rounding of V E lies far below FP64 rounding of V)
-  for (int e = threadIdx.x; e < nr * m; e += blockDim.x) {
-    const int j = e / nr, i = e - j * nr;
+  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
+    const int j = e / m, i = e - j * m;
     float x = 0.f;
     for (int l = 0; l < m; ++l) x = __fmaf_rn(Vf[l * ld + i], Ef[j * ld + l], x);
     V[j * ld + i] += (double)x;
