@@ -583,7 +583,8 @@ static __device__ __noinline__ int svd_jacobi(double* R0, float* R1, double* R2,
 // short: warp 0 holds the diagonal in registers and picks the next pivot and its reciprocal
 // while the warps of the other three schedulers update the remaining pairs (i > j), enumerated
 // densely.  2200-4500 clocks per step with a square root and two reductions in the chain
-// before, 600-900 now up to 20 columns, 1900 at 60 (the update's pairs).
+// before, 600-900 now up to 20 columns, 1900 at 60 (the update's pairs).  (The reciprocal is the
+// division: Newton steps on an FP32 one gave the same densities, and steps 1.2% longer.)
 __device__ __forceinline__ int pchol(double* A, double* X, int m, int ld, double thr_rel,
                                      double* dp) {
   __shared__ double cv[64], wv[64];
@@ -607,16 +608,7 @@ __device__ __forceinline__ int pchol(double* A, double* X, int m, int ld, double
     // (positive doubles order as their bits)
     if (b >= 0 && __double_as_longlong(d) <= __double_as_longlong(thr)) b = -1;
     if (b >= 0) {
-      // 1 / d: an FP32 reciprocal of the mantissa, two Newton steps in FP64 (the shortest chain
-      // of FP64 operations that gives every bit)
-      const int h = __double2hiint(d), ed = h >> 20;                     // biased exponent, >= 1
-      const double dm = __hiloint2double((h & 0xfffff) | 0x3ff00000, __double2loint(d));   // in [1, 2)
-      const float ym = __frcp_rn(__int_as_float(0x3f800000 | ((h & 0xfffff) << 3) | (__double2loint(d) >> 29 & 7)));
-      const int yb = __float_as_int(ym);                                 // in (1/2, 1]
-      double y = __hiloint2double(((yb >> 23) + 896) << 20 | (yb >> 3 & 0xfffff), yb << 29);
-      y = fma(y, fma(-dm, y, 1.0), y);
-      y = fma(y, fma(-dm, y, 1.0), y);
-      inv = scalbn(y, 1023 - ed);
+      inv = 1.0 / d;
       if (lane == 0) dp[k] = d;
     }
     if (lane == 0) piv = b;
