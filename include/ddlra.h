@@ -145,8 +145,9 @@ typedef struct dd_options {
                       /* bits.  DD_PRODUCTS_AUTO: per row family (spatial rows, angular rows)  */
                       /* the faster of the two: timed when the solver is created if autotune  */
                       /* is set, else the tensor cores where the family has at least two      */
-                      /* 128-row tiles per SM or rows x r_cap^2 >= 5.5e7 (the tall-skinny      */
-                      /* products also where a subdomain's rows are many for the FP64 form).   */
+                      /* 128-row tiles per SM and a subdomain that fills one, or rows x        */
+                      /* r_cap^2 >= 5.5e7 (the tall-skinny products also where a subdomain's   */
+                      /* rows are many for the FP64 form).                                     */
   int autotune;       /* 1: when the solver is created, time the launch choices on its own    */
                       /* workspace and keep the fastest: the products' and the               */
                       /* orthonormalisations' Grams' engines per row family (with            */

@@ -724,15 +724,19 @@ static dd_status create_impl(int ninst, const dd_grid* grids, const dd_tiling* t
   if (dd::orth_init() != cudaSuccess || dd::phase_init() != cudaSuccess)
     return bail(DD_ERR_CUDA, "kernel attribute setup failed");
   if (opt->products == DD_PRODUCTS_AUTO) {      // the heuristic; the autotuner may revise it
-    // Per row family.  Tall products: two 128-row tiles per SM, or rows x r_cap^2 past 5.5e7 (the FP64
-    // pipe does 2 FMA per clock and SM; the tensor form costs 15 us at least).  16 x 1024
+    // Per row family.  Tall products: two 128-row tiles per SM where the largest subdomain fills one
+    // (a smaller one leaves its tiles mostly empty: 1600 subdomains of 16 cells and 8 directions,
+    // r_cap = 6, a step of 7.3 ms against 2.3 with the FP64 kernels; 1600 of 100 and 96, r_cap = 18,
+    // 13.0 against 9.7), or rows x r_cap^2 past 5.5e7 (the FP64 pipe does 2 FMA per clock and SM; the
+    // tensor form costs 15 us at least; 400 subdomains of 100 cells, 96 directions: r_cap = 60, 15.7 ms a
+    // step against 18.5 in FP64; 30, 5.6 against 5.0).  16 x 1024
     // cells and 16 x 512 directions: r_cap = 30, 19.4 against 18.1 us per product and a step 2.24
     // against 2.59 ms (the Gram of an orthonormalisation comes with the FP64 product); r_cap = 60,
     // 48.6 against 24.8 us, 6.55 against 5.93 ms; 50, but with ranks well below it, 2.33 against 2.50.
     const long tiles_sp = (long)nsub * ((h->maxN + 127) / 128), tiles_ang = (long)nsub * ((n + 127) / 128);
     const long rc2 = (long)RC * RC;
-    P.oz_sp = tiles_sp >= 2L * P.nsm || Nt * rc2 >= 55000000L;
-    P.oz_ang = tiles_ang >= 2L * P.nsm || (long)nsub * n * rc2 >= 55000000L;
+    P.oz_sp = (h->maxN >= 128 && tiles_sp >= 2L * P.nsm) || Nt * rc2 >= 55000000L;
+    P.oz_ang = (n >= 128 && tiles_ang >= 2L * P.nsm) || (long)nsub * n * rc2 >= 55000000L;
     // Tall-skinny products likewise, and where the FP64 kernels' chunks come to 2e5 row x r_cap^2
     // each: 4 x 4096 cells, r_cap = 30 (256 rows a chunk): spatial coefficients 104 us against 34
     // on the tensor cores, a Gram 26 against 33; 16384 cells (1024 rows): 253 and 81 against 30;

@@ -26,14 +26,12 @@ def B():
 @pytest.mark.parametrize("use_graph", [False, True])
 def test_batch_of_small_problems(B, split, problems, use_graph):
     """11200 subdomains (6 x 11200 = 67200 pairs, 8 x 11200 = 89600) and 8320 (66560): past
-    65535 with the tensor products, which products = "auto" takes at this size."""
+    65535 with the tensor products."""
     one = [inputs.random_small_problem(s, nx=16, ny=16, tiles_x=4, tiles_y=4, n_mu=0, n_phi=8,
                                        rank=2, r_aug_max=4, integrator="rk4").with_(kstep_split=split)
            for s in range(4)]
     refs = [dd_dlra.DDDLRA(wl).run(2).scalar_flux() for wl in one]
-    s = B.Solver([one[i % 4] for i in range(problems)], products="auto", use_graph=use_graph)
-    choice, _ = s.tuning()
-    assert choice["oz_gram_spatial"] == 1 and choice["oz_gram_angular"] == 1
+    s = B.Solver([one[i % 4] for i in range(problems)], products="tensor", use_graph=use_graph)
     s.step(2)
     rho = s.scalar_flux()
     for i in range(problems):
