@@ -998,7 +998,8 @@ __global__ void __launch_bounds__(OT_THREADS, 1) k_oz_tall(TcTall a) {
                                      128, 16 * s.KP);
       const uint64_t bd0 = tc::sdesc(tc::smem_u32(msl), 128, 16 * s.KP);
       const int nslab = s.KP >> 4;
-      for (int c = 0; c < s.nch && alive; ++c, ++qc) {
+      int c = 0;
+      for (; c < s.nch; ++c, ++qc) {
         const int buf = qc & (OT_NB - 1);
         if (qc >= OT_NB) {
           alive = tc::mbar_wait(&tempty[buf], (qc / OT_NB - 1) & 1, kWait);
@@ -1013,9 +1014,11 @@ __global__ void __launch_bounds__(OT_THREADS, 1) k_oz_tall(TcTall a) {
                          tc::idesc(tc::FMT_BF16, 128, 16 * (OZ_DIG - d)), (sl > 0 || d > 0) ? 1u : 0u);
         tc::mma_commit(&tfull[buf]);
       }
+      if (c > 0) {                                     // (a tile cut short by a wait that ran out too)
+        tc::mma_commit(&empty[b]);
+        ++used[b];
+      }
       if (!alive) break;
-      tc::mma_commit(&empty[b]);
-      ++used[b];
       ++it;
       ++j;
     }
