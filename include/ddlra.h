@@ -94,10 +94,11 @@ enum { DD_RANK_FIXED = 0, DD_RANK_TOL = 1 };
 enum { DD_EULER = 0, DD_RK4 = 1 };
 /* Arithmetic of the step (the paper fixes none).  DD_FP64: FP64 throughout, except that
  * the small eigen/singular value problems (m x m, m <= 64) run FP32 Jacobi sweeps finished
- * in double-float arithmetic (~1e-13 relative; the eigensolver of the orthonormalisation
- * adds one FP64 refinement).  DD_MIXED: in addition, FP32 arithmetic for the increments of
- * the collision-step ODEs and for the L-step's stage corrections (its first-stage
- * right-hand side is formed in FP64); each update itself is added in FP64.  DD_TF32 /
+ * in double-float arithmetic (~1e-13 relative; the eigen-split of the K-step adds one FP64
+ * refinement).  DD_MIXED: in addition, FP32 arithmetic for the increments of the collision's
+ * L-step and for the advection L-step's stage corrections (its first-stage right-hand side is
+ * formed in FP64; with DD_EULER and the products on the tensor cores the advection L-step is
+ * FP64-accurate); each update itself is added in FP64.  DD_TF32 /
  * DD_BF16: DD_MIXED plus the Galerkin contractions on the tensor cores (tcgen05) in TF32 /
  * BF16 with FP32 accumulation, each FP64 operand split into a high and a low part of that
  * type and multiplied hi*hi + hi*lo + lo*hi (FP32-level error per product): the angular
@@ -136,12 +137,15 @@ typedef struct dd_options {
                       /* C+- = <V, max/min(Omega, 0) V> (the L-step's per-direction upwind   */
                       /* flux projected on the angular basis; equal to Appendix A's at full  */
                       /* rank; not the paper's scheme at low rank; no eigendecomposition)    */
-  int products;       /* the FP64 tall x small products (orthonormalisations, truncation,     */
-                      /* K0 = X S <V, V_hat>): DD_PRODUCTS_FP64: FP64 CUDA-core arithmetic;    */
-                      /* DD_PRODUCTS_TENSOR: these and the orthonormalisations' Grams on the  */
-                      /* BF16 tensor cores with the error-free                                 */
-                      /* splitting of Ozaki et al. (seven 8-bit digits per value, exact FP32   */
-                      /* accumulation, FP64-level error).  Results agree to FP64 rounding, not */
+  int products;       /* the FP64 products over the rows of the factors: tall x small          */
+                      /* (orthonormalisations, truncation, K0 = X S <V, V_hat>, the K-step's   */
+                      /* basis changes, the explicit Euler L-step) and tall-skinny (the         */
+                      /* orthonormalisations' Grams, the Galerkin coefficients of the advection */
+                      /* and the collision).  DD_PRODUCTS_FP64: FP64 CUDA-core arithmetic;      */
+                      /* DD_PRODUCTS_TENSOR: the BF16 tensor cores with the error-free          */
+                      /* splitting of Ozaki et al. (seven 8-bit digits per value, exact FP32    */
+                      /* accumulation, 55 to 56 bits relative to the largest entry of the       */
+                      /* operand's row or column).  Results agree to FP64 rounding, not         */
                       /* bits.  DD_PRODUCTS_AUTO: per row family (spatial rows, angular rows)  */
                       /* the faster of the two: timed when the solver is created if autotune  */
                       /* is set, else the tensor cores where the family has at least two      */
@@ -149,12 +153,14 @@ typedef struct dd_options {
                       /* r_cap^2 >= 5.5e7 (the tall-skinny products also where a subdomain's   */
                       /* rows are many for the FP64 form).                                     */
   int autotune;       /* 1: when the solver is created, time the launch choices on its own    */
-                      /* workspace and keep the fastest: the products' and the               */
-                      /* orthonormalisations' Grams' engines per row family (with            */
-                      /* DD_PRODUCTS_AUTO) and the chunk counts of the orthonormalisations'  */
+                      /* workspace and keep the fastest: per row family (with                */
+                      /* DD_PRODUCTS_AUTO) the engine of the tall x small products, timed on   */
+                      /* them, and of the tall-skinny ones, timed on one symmetric Gram at the */
+                      /* column capacity; and the chunk counts of the orthonormalisations'    */
                       /* chunked Gram reductions (the heuristic's, a half and a quarter of it; */
-                      /* every count keeps a fixed summation order).  Cached per problem     */
-                      /* shape in the process.  0: fixed heuristics.  See dd_dlra_tuning.      */
+                      /* on the tensor cores the rows per chunk: 1, 2 and 4 times; every count */
+                      /* keeps a fixed summation order).  Cached in the process per device,    */
+                      /* problem shape and engine.  0: fixed heuristics.  See dd_dlra_tuning.  */
 } dd_options;
 
 enum { DD_SPLIT_LIE = 0, DD_SPLIT_STRANG = 1 };

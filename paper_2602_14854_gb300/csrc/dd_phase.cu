@@ -2055,8 +2055,12 @@ cudaError_t autotune(Problem& P, const PhaseBufs& B, cudaStream_t st, int tune_p
       // forms the Gram of its output from the same tiles in the orthonormalisation (one of
       // its two products there): the tensor-core side is charged half a separate Gram
       // reduction per product.
-      // The orthonormalisation's Gram engine (k_gram or k_oz_gram) is timed the same way
-      // and the faster one kept (by 3%; k_gram on a tie).
+      // The tall-skinny products' engine is timed on one symmetric Gram (k_gram or k_oz_gram) and
+      // the faster one kept (by 3%; k_gram on a tie).  A trial of everything that a step forms with
+      // the engine, coefficients included, at the largest ranks chose the same on 12 of 13 shapes and
+      // the slower one on the other (2852 us a step against 2617: it is chosen before the tall
+      // products' engine, which decides whether a second Gram is formed at all), and took 25 ms of a
+      // 512 x 512 solver's creation.
       const int half = std::max(2, (RC / 2) & ~1);
       Problem Q = P;
       Q.oz_sp = Q.oz_ang = 0;

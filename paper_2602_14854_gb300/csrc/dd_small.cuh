@@ -4,8 +4,8 @@
 //
 // These run on one SM per subdomain while the rest of the GPU waits, so what counts is latency:
 // the barriers, shuffles and dependent operations of a Jacobi round, not its operations.  A
-// round's m / 2 disjoint pairs of columns go to groups of 8 lanes (m <= 32) or 16 lanes, a
-// few rows per lane, columns in shared memory: two loads per row, one dot product (3 or 4
+// round's m / 2 disjoint pairs of columns go to groups of 8 lanes (FP32; double-float with at most
+// 32 columns) or 16 lanes (double-float beyond), a few rows per lane, columns in shared memory: two loads per row, one dot product (3 or 4
 // shuffle steps), one rotation, two stores, one barrier among the warps that hold pairs.
 // Measured per kernel launch with the sweeps laid out over whole warps (rows interleaved over
 // the warps of the CTA, partners exchanged by shuffles, dot products summed through shared
@@ -19,7 +19,8 @@
 
 namespace dd {
 
-// threads of the small kernels: a pair of columns per 8 (up to 32 columns) or 16 lanes
+// threads of the small kernels: a pair of columns per 8 lanes up to 32 columns, per 16 beyond (the
+// double-float sweeps; the FP32 ones keep 8)
 __host__ __device__ __forceinline__ int small_threads(int RC) { return RC <= 32 ? 256 : 512; }
 __host__ __device__ __forceinline__ int small_ld(int RC) { return RC | 1; }
 // bytes of one RC-column region of 8-byte entries
