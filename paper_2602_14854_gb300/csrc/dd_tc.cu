@@ -1615,19 +1615,21 @@ __global__ void __launch_bounds__(OG_THREADS, 1) k_oz_gram(const __grid_constant
 }
 
 // Sum of the chunk partials of every product, in chunk order, into the small matrices (slot
-// dst[blk]), zero outside the product's na x nb entries.  Grid: (entries, subdomains, products):
-// y ends at 65535, so the products have a dimension of their own and this kernel takes as many
-// subdomains as every other one.
+// dst[blk]), zero outside the product's na x nb entries.  Grid: (products x entries, subdomains): y
+// ends at 65535, so that this kernel takes as many subdomains as every other one.  (The product in
+// z, where its descriptor's index is uniform, took 14 us a launch instead of 11: one subdomain of
+// 16384 cells, 64 chunks of 30 x 30.)
 __global__ void __launch_bounds__(DD_THREADS) k_oz_reduce(const __grid_constant__ OzGram a, OzDst dst,
                                                           double* sm) {
   const int k = blockIdx.y, RC = a.g.RC;
-  const OzProd& p = a.p[blockIdx.z];
+  const int nbx = (RC * RC + DD_THREADS - 1) / DD_THREADS, pi = blockIdx.x / nbx;
+  const OzProd& p = a.p[pi];
   int rows, na, nb;
   og_shape(a, k, p, &rows, &na, &nb);
   const int nck = og_chunks(a, rows);
   const double* part = a.part + ((long)k * a.nchunk * a.nblk + p.blk) * RC * RC;
   double* out = sm + ((long)k * NSMALL + dst.idx[p.blk]) * RC * RC;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  const int e = (blockIdx.x - pi * nbx) * DD_THREADS + threadIdx.x;
   if (e >= RC * RC) return;
   const int i = e / RC, j = e - i * RC;
   double s = 0.0;
@@ -1779,8 +1781,8 @@ bool oz_gram(const Problem& P, cudaStream_t st, OzGram& a, const OzDst* dst, dou
   pend(st);
   if (dst) {
     pbeg(st, KS_REDUCE);
-    k_oz_reduce<<<dim3((P.g.RC * P.g.RC + DD_THREADS - 1) / DD_THREADS, P.g.nsub, a.nprod), DD_THREADS, 0, st>>>(
-        a, *dst, sm);
+    const int nbx = (P.g.RC * P.g.RC + DD_THREADS - 1) / DD_THREADS;
+    k_oz_reduce<<<dim3(nbx * a.nprod, P.g.nsub), DD_THREADS, 0, st>>>(a, *dst, sm);
     pend(st);
   }
   return true;
